@@ -191,7 +191,7 @@ void esplit_destroy(esplit_ctx* c) {
   void* ps[] = {b.Qref, b.J,       b.nu,      b.pair,   b.Lam,     b.face_pairs, b.ops64,   b.ops32,   b.ops32lo,
                 b.list_split, b.list_had, b.hflags, b.hflag0, b.hcount, b.sat, b.fcache, b.rows, b.partial, b.scal, b.root, b.status, b.stage_u,
                 b.stage_r, b.dacc, b.node_cache, b.vjp_work, b.host_u, b.host_r, b.fv, b.vsat, b.va, b.wslot, b.vfb, b.vfs, b.vus,
-                b.bslot, b.bstate, b.ihf, b.opsD32, b.ihd, b.nscale};
+                b.bslot, b.bstate, b.ihf, b.opsD32, b.ihd, b.nscale, b.opsP, b.opsE};
   for (void* p : ps) dfree(p);
   if (c->sg.exec) cudaGraphExecDestroy(c->sg.exec);
   if (c->sg.graph) cudaGraphDestroy(c->sg.graph);
@@ -335,6 +335,9 @@ int esplit_upload_mesh(esplit_ctx* c, int n_e, const double* J, const double* La
     dalloc(c, &c->b.opsD32, 0);
     c->opsD_stride = 0;
   }
+  const size_t tensor_rows = d >= 2 ? (size_t)n_e * d * NP : 0;
+  if ((rc = dalloc(c, &c->b.opsP, tensor_rows * ((NP + 1) / 2)))) return rc;
+  if ((rc = dalloc(c, &c->b.opsE, tensor_rows))) return rc;
   c->partial_cap = 0;
   if ((rc = ensure_partial(c))) return rc;
   CK(cudaMemcpy(c->b.J, J, sizeof(double) * n_e * NP, cudaMemcpyHostToDevice));

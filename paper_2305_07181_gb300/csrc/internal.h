@@ -51,6 +51,10 @@ struct Buffers {
   //   k <  d: M_i^T, M_i = H^-1 (Q_x_i/(beta+1) + Q_x_i^T)
   //   k >= d: D_i^T, D_i = H^-1 Q_x_i
   double* ops64 = nullptr;     // [n_e][2d][n_p][n_p]
+  // D_i as 60-bit fixed point, two entries per uint4, and the rows' exponents
+  // (tc64.cuh; triangles and tetrahedra)
+  uint4* opsP = nullptr;       // [n_e][d][n_p][ceil(n_p / 2)]
+  short* opsE = nullptr;       // [n_e][d][n_p]
   float* ops32 = nullptr;      // same, float (nearest)
   float* ops32lo = nullptr;    // same, float remainder ops64 - ops32 (compensated FP32-bulk contractions)
   double* rows = nullptr;      // [n_e][2d][n_p] row sums of the ops64 matrices

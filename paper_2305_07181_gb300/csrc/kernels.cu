@@ -24,6 +24,7 @@
 #include "visc_flux.cuh"
 #include "reduce.cuh"
 #include "bits32.cuh"
+#include "tc64.cuh"
 
 namespace esplit {
 
@@ -149,6 +150,15 @@ int launch_build_ops(esplit_ctx* c, cudaStream_t s) {
   size_t nr = (size_t)c->n_e * 2 * c->dim * c->n_p;
   build_rows_kernel<<<(unsigned)((nr + 255) / 256), 256, 0, s>>>(c->b.ops64, c->n_e, 2 * c->dim, c->b.rows);
   c->launches += 2;
+  if (c->b.opsP) {
+    const size_t nr2 = (size_t)c->n_e * c->dim * c->n_p;
+    const unsigned nb2 = (unsigned)((nr2 + 255) / 256);
+    if (tc::bits_for(c->n_p) == 10)
+      tc::build_packed_kernel<10><<<nb2, 256, 0, s>>>(c->b.ops64, c->n_e, c->dim, c->n_p, c->b.opsP, c->b.opsE);
+    else
+      tc::build_packed_kernel<9><<<nb2, 256, 0, s>>>(c->b.ops64, c->n_e, c->dim, c->n_p, c->b.opsP, c->b.opsE);
+    c->launches++;
+  }
   {
     const size_t nn = (size_t)c->n_e * c->n_p, ns = (size_t)c->n_e * c->n_slot, nt = nn > ns ? nn : ns;
     const unsigned nbt = (unsigned)((nt + 255) / 256);
@@ -558,11 +568,233 @@ int launch_face_bc(esplit_ctx* c, const double* u, double* out, int add, double*
 // nodes (E_i = diag(nu_i) there) and the facet kernel adds it to the facet
 // contributions.
 //
-// Node states, fluxes, entropy variables and the A~_i products are float64 in
-// both precision modes.  T = double: plain float64 contractions.  T = float
-// (FP32-bulk): the contractions act in float32 on the variation inside the
-// element, relative to its node 0, and the node-0 values come back through
-// the float64 row sums of the stored operators,
+// Pointwise work in float64, one node per thread.  Triangles and tetrahedra:
+// the contractions on the tensor cores (tc64.cuh: exact digit products, one
+// rounding; as accurate as a float64 sum or better), so the float64 pipe has
+// only the nodal state, fluxes and A~_i products left.  Lines and 7-node
+// triangles: float64 FMA loops, too short for the tiles.
+// Optional: block partial of sum H w^T r (entropy production, float64).
+// ---------------------------------------------------------------------------
+template <int D, int NP, int EB, bool VISC>
+struct SplitCfg {
+  static constexpr bool TENSOR = D >= 2 && NP > 8;
+  static constexpr int NC = D + 2;
+  static constexpr int THREADS = round32(EB * NP);
+  using S = tc::Shape<D, NP, EB, NC, NC>;  // f_i summed over i, w per direction
+  using SV = tc::Shape<D, NP, EB, NC, 0>;  // F^V_i + a_i/(2H), summed over i
+  static constexpr size_t SMEM =
+      TENSOR ? S::DIG_BYTES + S::RES_BYTES + S::EX_BYTES + EB * sizeof(int)
+             : (size_t)EB * (D + 1) * NC * NP * sizeof(double);
+};
+
+template <int D, int NP, int EB, bool VISC, bool CACHE = false, bool ENT = false>
+__global__ void __launch_bounds__(round32(EB * NP)) split_volume_kernel(
+    const double* __restrict__ u, double* __restrict__ r, const double* __restrict__ ops64,
+    const uint4* __restrict__ opsP, const short* __restrict__ opsE, const double* __restrict__ J,
+    const double* __restrict__ sat, const int* __restrict__ list, int n_list, Phys<double> c64,
+    int* __restrict__ status, double* __restrict__ prod, int visc_heat, const double* __restrict__ nu,
+    const double* __restrict__ ah, double* __restrict__ fvs, double* __restrict__ fcache, int n_slot_total,
+    double* __restrict__ ent_part = nullptr, double* __restrict__ ncache = nullptr,
+    double* __restrict__ wsl = nullptr) {
+  constexpr int NC = D + 2;
+  using Cfg = SplitCfg<D, NP, EB, VISC>;
+  using S = typename Cfg::S;
+  constexpr int THREADS = Cfg::THREADS;
+  extern __shared__ __align__(16) unsigned char split_smem[];
+  const int NS = c_ref.n_slot;
+  int el = threadIdx.x / NP;
+  int m = threadIdx.x - el * NP;
+  int li = blockIdx.x * EB + el;
+  bool active = (el < EB) && (li < n_list);
+  int e = active ? (list ? list[li] : li) : 0;
+  Node<double, D> nd;
+  double vals[S::COLS];  // f_i, then w
+#pragma unroll
+  for (int q = 0; q < S::COLS; ++q) vals[q] = 0.0;
+  if (active) {
+    double uu[NC];
+#pragma unroll
+    for (int q = 0; q < NC; ++q) uu[q] = __ldg(&u[((size_t)e * NC + q) * NP + m]);
+    if (!node_from_u<double, D>(uu, c64, nd)) atomicOr(status, 1);
+    euler_fluxes<D>(nd, uu, vals);
+#pragma unroll
+    for (int q = 0; q < NC; ++q) vals[D * NC + q] = nd.W[q];
+  }
+  double accd[NC], gd[D][NC];  // sum_i D_i f_i and D_i w
+  // shared memory of the tensor path
+  __half* dig = reinterpret_cast<__half*>(split_smem);
+  double* resb = reinterpret_cast<double*>(split_smem + S::DIG_BYTES);
+  int* ex = reinterpret_cast<int*>(split_smem + S::DIG_BYTES + S::RES_BYTES);
+  int* elems = reinterpret_cast<int*>(split_smem + S::DIG_BYTES + S::RES_BYTES + S::EX_BYTES);
+  const int ms = el < EB ? m : 0, els = el < EB ? el : 0;  // in-range slot of the idle lanes
+  if constexpr (Cfg::TENSOR) {
+    if (m == 0 && el < EB) elems[el] = active ? e : -1;
+    tc::zero_padding<S, NP, EB, THREADS>(dig);
+    tc::digitize<S, NP, EB, THREADS>(vals, el < EB, el, m, reinterpret_cast<unsigned*>(resb), ex, dig);
+    __syncthreads();
+    tc::contract<S, D, NP, EB, NC, NC, THREADS>(dig, ex, elems, opsP, opsE, resb);
+    __syncthreads();
+    const double* rs = resb + (size_t)els * S::OUTS * S::NPO + ms;
+#pragma unroll
+    for (int q = 0; q < NC; ++q) accd[q] = rs[q * S::NPO];
+#pragma unroll
+    for (int i = 0; i < D; ++i)
+#pragma unroll
+      for (int q = 0; q < NC; ++q) gd[i][q] = rs[(NC + i * NC + q) * S::NPO];
+  } else {
+    double* sv = reinterpret_cast<double*>(split_smem);  // [EB][COLS][NP]
+    if (active) {
+#pragma unroll
+      for (int q = 0; q < S::COLS; ++q) sv[(el * S::COLS + q) * NP + m] = vals[q];
+    }
+    __syncthreads();
+    const double* op = ops64 + (size_t)e * (2 * D * NP * NP);
+#pragma unroll
+    for (int q = 0; q < NC; ++q) accd[q] = 0.0;
+#pragma unroll
+    for (int i = 0; i < D; ++i)
+#pragma unroll
+      for (int q = 0; q < NC; ++q) gd[i][q] = 0.0;
+    if (active) {
+#pragma unroll
+      for (int i = 0; i < D; ++i)
+#pragma unroll
+        for (int n = 0; n < NP; ++n) {
+          const double dt = __ldg(&op[((D + i) * NP + n) * NP + m]);
+#pragma unroll
+          for (int q = 0; q < NC; ++q) {
+            accd[q] += dt * sv[(el * S::COLS + i * NC + q) * NP + n];
+            gd[i][q] += dt * sv[(el * S::COLS + D * NC + q) * NP + n];
+          }
+        }
+    }
+  }
+  double hw = 0.0, ent_s = 0.0, ent_a = 0.0;
+  const int sl = c_ref.node_slot[ms];
+  double res[NC], Fp[D][NC], Hm = 0.0;
+  if (active) {
+    const JvpPrep<double> jp = jvp_prep<double, D>(nd, c64);
+    if constexpr (ENT) {
+      // entropy of u_n for the relaxation step (the entropy kernel's outputs):
+      // S_H = beta q p, and the per-node values its evaluation passes reuse
+      const size_t nn = (size_t)n_list * NP, g = (size_t)e * NP + m;
+      const double sH = c64.beta * nd.q * nd.p;
+      ncache[g] = sH;
+      ncache[nn + g] = nd.ir;
+      ncache[2 * nn + g] = jp.itheta * nd.ir;  // 1/p
+      const double Hm0 = c_ref.H[m] * __ldg(&J[(size_t)e * NP + m]);
+      ent_s = Hm0 * sH;
+      ent_a = Hm0 * fabs(sH);
+    }
+    if constexpr (CACHE) {
+      // nodal quantities of the facet nodes for the facet kernel that runs after
+      // this one (it then needs no logarithm, exponential or division for them)
+      if (sl >= 0) {
+        const size_t S_ = (size_t)n_slot_total, ix = (size_t)e * NS + sl;
+        fcache[0 * S_ + ix] = nd.rho;
+        fcache[1 * S_ + ix] = nd.ir;
+        fcache[2 * S_ + ix] = nd.p;
+        fcache[3 * S_ + ix] = nd.e;
+        fcache[4 * S_ + ix] = nd.q;
+        fcache[5 * S_ + ix] = nd.lnq;
+        fcache[6 * S_ + ix] = nd.lnp;
+        fcache[7 * S_ + ix] = jp.iq;
+        fcache[8 * S_ + ix] = jp.itheta * nd.ir;  // 1/p
+#pragma unroll
+        for (int i = 0; i < D; ++i) fcache[(9 + i) * S_ + ix] = nd.V[i];
+      }
+    }
+    double nonc[NC];
+    dflux_dw_sum<D>(nd, jp, c64, -c64.inv_bp1, gd, nonc);
+    Hm = c_ref.H[m] * __ldg(&J[(size_t)e * NP + m]);
+    const double kf = c64.beta * c64.inv_bp1;
+#pragma unroll
+    for (int q = 0; q < NC; ++q) {
+      // the facet contributions include H^-1 sum_i E_i f_i (added by the facet kernel)
+      res[q] = nonc[q] - kf * accd[q];
+      if (!CACHE && sl >= 0) res[q] += __ldg(&sat[((size_t)e * NC + q) * NS + sl]);
+    }
+    if constexpr (VISC) {
+      // viscous flux from the gradients just formed (gd = D_i w), plus the
+      // folded BO lift a/(2H) at the facet nodes; F^V kept for the flux jump
+      visc_flux<double, D>(nd, c64, visc_heat, gd, Fp);
+      if (sl >= 0 && wsl) {
+        // entropy variables at the facet slot, for the flux-jump kernel's
+        // share of the entropy production
+#pragma unroll
+        for (int q = 0; q < NC; ++q) wsl[((size_t)e * NC + q) * NS + sl] = nd.W[q];
+      }
+      if (sl >= 0) {
+#pragma unroll
+        for (int i = 0; i < D; ++i)
+#pragma unroll
+          for (int q = 0; q < NC; ++q) {
+            size_t ix = (((size_t)e * D + i) * NC + q) * NS + sl;
+            fvs[ix] = Fp[i][q];
+            Fp[i][q] += 0.5 * __ldg(&ah[ix]);
+          }
+      }
+    }
+  }
+  if constexpr (VISC) {
+    // sum_i D_i (F^V_i + a_i/(2H)) - sum_i nu_i a_i/(2H^2) at the facet nodes
+    using SV = typename Cfg::SV;
+    static_assert(SV::DIG_BYTES <= S::DIG_BYTES && SV::RES_BYTES <= S::RES_BYTES && SV::EX_BYTES <= S::EX_BYTES,
+                  "the second contraction fits the first one's shared memory");
+    double fvals[SV::COLS];
+#pragma unroll
+    for (int i = 0; i < D; ++i)
+#pragma unroll
+      for (int q = 0; q < NC; ++q) fvals[i * NC + q] = active ? Fp[i][q] : 0.0;
+    __syncthreads();  // every thread has read the first contraction's results
+    // the rows keep the first contraction's stride: their padding is still zero
+    tc::digitize<SV, NP, EB, THREADS>(fvals, el < EB, el, m, reinterpret_cast<unsigned*>(resb), ex, dig);
+    __syncthreads();
+    tc::contract<SV, D, NP, EB, NC, 0, THREADS>(dig, ex, elems, opsP, opsE, resb);
+    __syncthreads();
+    if (active) {
+#pragma unroll
+      for (int q = 0; q < NC; ++q) res[q] += resb[((size_t)el * SV::OUTS + q) * SV::NPO + m];
+      if (sl >= 0) {
+        const double ih = 1.0 / Hm;
+        double nv[D];
+#pragma unroll
+        for (int i = 0; i < D; ++i) nv[i] = __ldg(&nu[((size_t)e * NS + sl) * D + i]);
+#pragma unroll
+        for (int q = 0; q < NC; ++q) {
+          double corr = 0.0;
+#pragma unroll
+          for (int i = 0; i < D; ++i) corr += nv[i] * __ldg(&ah[(((size_t)e * D + i) * NC + q) * NS + sl]);
+          res[q] -= 0.5 * corr * ih;
+        }
+      }
+    }
+  }
+  if (active) {
+#pragma unroll
+    for (int q = 0; q < NC; ++q) r[((size_t)e * NC + q) * NP + m] = res[q];
+    if (prod) {
+#pragma unroll
+      for (int q = 0; q < NC; ++q) hw += nd.W[q] * res[q];
+      hw *= Hm;
+    }
+  }
+  if (prod) {
+    double v[1] = {hw};
+    block_sum_t<1, THREADS>(v, prod + blockIdx.x);
+  }
+  if constexpr (ENT) {
+    __syncthreads();  // the block sum's shared scratch is reused
+    double v2[2] = {ent_s, ent_a};
+    block_sum_t<2, THREADS>(v2, ent_part + 2 * blockIdx.x);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// entropy-split volume kernel of the FP32-bulk setting: the terms of
+// split_volume_kernel with the contractions in float32 on the variation
+// inside the element, relative to its node 0; the node-0 values come back
+// through the float64 row sums of the stored operators,
 //   D_i f_i = D_i (f_i - f_i,0) + f_i,0 (D_i 1),  D_i w = D_i (w - w_0) + w_0 (D_i 1).
 // Operator entries and variations are each held as an unevaluated float32
 // sum hi + lo, and the products are accumulated by the compensated dot
@@ -571,8 +803,7 @@ int launch_face_bc(esplit_ctx* c, const double* u, double* out, int add, double*
 // addition (TwoSum) goes to a second float32 accumulator, together with the
 // cross terms hi*lo.  At low Mach number the energy-flux variation inside an
 // element is ~(E + p)|dV|, hundreds of times the residual, and a plain
-// float32 product would lose that factor.
-// Optional: block partial of sum H w^T r (entropy production, float64).
+// float32 product would lose that factor.  Pointwise work in float64.
 // ---------------------------------------------------------------------------
 template <typename T, int D, int NP, int EB>
 struct SplitSmem {
@@ -597,14 +828,9 @@ __device__ __forceinline__ void dot2_step(float ah, float al, float bh, float bl
   acc = s;
   cmp = __fadd_rn(cmp, __fadd_rn(t, e));
 }
-template <int D, int NP, int EB>
-struct SplitSmem<double, D, NP, EB> {
-  double rf[EB][D][D + 2][NP];
-  double rw[EB][D + 2][NP];
-};
 
 template <typename T, int D, int NP, int EB, bool VISC, bool CACHE = false, bool ENT = false>
-__global__ void __launch_bounds__(EB * NP, (sizeof(T) == 4 && !VISC && D == 2) ? 4 : ((VISC && D == 3) ? 2 : 1)) split_volume_kernel(
+__global__ void __launch_bounds__(EB * NP, (sizeof(T) == 4 && !VISC && D == 2) ? 4 : ((VISC && D == 3) ? 2 : 1)) split_bulk_kernel(
     const double* __restrict__ u, double* __restrict__ r, const T* __restrict__ ops,
     const float* __restrict__ opslo, const double* __restrict__ rows, const double* __restrict__ J,
     const double* __restrict__ sat, const int* __restrict__ list, int n_list, Phys<T> c, Phys<double> c64,
@@ -1065,22 +1291,55 @@ namespace esplit {
 
 template <int NP>
 struct VolCfg {
-  static constexpr int EB_SPLIT = (256 / NP) > 0 ? (256 / NP) : 1;
-  // float64 on triangles: the float64-pipe-bound split kernel holds 2 blocks
-  // of ~250 threads per SM, and the last of n_e / EB_SPLIT blocks leave the
-  // SMs unevenly loaded by up to one block in ~15 (config 2).  Smaller blocks
-  // that fill whole warps make that granularity finer and raise the warps
-  // per SM: n_p = 7 and 18, 126 threads (4-5 blocks per SM; measured at 18:
-  // 0.506 -> 0.490 ms per launch); n_p = 12, 192 threads (6 full warps, 3
-  // blocks per SM; 0.285 -> 0.270 ms); n_p = 27, 189 threads (6 warps, 3
-  // blocks per SM; 0.973 -> 0.952 ms).
-  static constexpr int EB_SPLIT64_2D = NP == 7 ? 18 : NP == 12 ? 16 : NP == 18 ? 7 : NP == 27 ? 7 : EB_SPLIT;
+  // split volume kernel: blocks of about 128 threads that fill their warps
+  // (126 of 128 threads at n_p = 7 and 18, 120 at 12, 189 of 192 at 27, 125 at
+  // 25, 116 of 128 at 58, 156 of 160 at 78), so that several blocks share an
+  // SM and one block's tensor phase runs beside another's float64 phase
+  static constexpr int EB_SPLIT = NP == 7 ? 18 : NP == 12 ? 10 : NP == 18 ? 7 : NP == 27 ? 7 : NP == 25 ? 5
+                                  : NP > 32 ? 2 : 128 / NP;
+  static constexpr int EB_BULK = (256 / NP) > 0 ? (256 / NP) : 1;
   // larger operators (tetrahedra of degree 3 and 4): the pair contributions
   // pass through shared memory in chunks of HAD_KC pair offsets, which leaves
   // room for more elements per block
   static constexpr int EB_HAD = NP > 32 ? ((256 / NP) > 0 ? (256 / NP) : 1) : ((128 / NP) > 0 ? (128 / NP) : 1);
   static constexpr int HAD_KC = NP > 32 ? 8 : NP / 2;
 };
+
+// T = float: the FP32-bulk kernel
+template <typename T, int D, int NP, int EB, bool VISC, bool CACHE, bool ENT>
+static void split_launch(esplit_ctx* c, const double* u, double* r, const double* sat, const int* list, int n_list,
+                         int nb, double* prod, double* ent_part, cudaStream_t s) {
+  const Phys<double> ph = make_phys<double>(c->prm.gam, c->prm.beta, c->prm.R, c->prm.mu, c->prm.Pr);
+  const int heat = VISC ? c->prm.heat_flux : -1;
+  double* fcache = CACHE ? c->b.fcache : nullptr;
+  double* ncache = ENT ? c->b.node_cache : nullptr;
+  double* wsl = VISC && prod ? c->b.wslot : nullptr;
+  const double* va = VISC ? c->b.va : nullptr;
+  double* fv = VISC ? c->b.fv : nullptr;
+  static bool attr_set = false;
+  if constexpr (sizeof(T) == sizeof(double)) {
+    using Cfg = SplitCfg<D, NP, EB, VISC>;
+    auto* kern = split_volume_kernel<D, NP, EB, VISC, CACHE, ENT>;
+    if (!attr_set) {
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
+      cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+      attr_set = true;
+    }
+    kern<<<nb, Cfg::THREADS, Cfg::SMEM, s>>>(u, r, c->b.ops64, c->b.opsP, c->b.opsE, c->b.J, sat, list, n_list, ph,
+                                             c->b.status, prod, heat, c->b.nu, va, fv, fcache, c->n_e * c->n_slot,
+                                             ent_part, ncache, wsl);
+  } else {
+    const Phys<T> ph32 = make_phys<T>(c->prm.gam, c->prm.beta, c->prm.R, c->prm.mu, c->prm.Pr);
+    auto* kern = split_bulk_kernel<T, D, NP, EB, VISC, CACHE, ENT>;
+    if (!attr_set) {  // sized for four blocks per SM (inviscid, 2D) or two (viscous, 3D)
+      cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+      attr_set = true;
+    }
+    kern<<<nb, EB * NP, 0, s>>>(u, r, (const T*)c->b.ops32, c->b.ops32lo, c->b.rows, c->b.J, sat, list, n_list, ph32,
+                                ph, c->b.status, prod, heat, c->b.nu, va, fv, c->b.ops64, fcache,
+                                c->n_e * c->n_slot, ent_part, ncache, wsl);
+  }
+}
 
 template <typename T, int D, int NP>
 static int residual_np(esplit_ctx* c, const double* u, double* r, cudaStream_t s, double* prod, int* n_partial,
@@ -1136,55 +1395,23 @@ static int residual_np(esplit_ctx* c, const double* u, double* r, cudaStream_t s
   const int* lsplit = scheme == ESPLIT_SCHEME_HYBRID ? c->b.list_split : nullptr;
   const int* lhad = scheme == ESPLIT_SCHEME_HYBRID ? c->b.list_had : nullptr;
   if (n_split > 0) {
-    constexpr int EB = (std::is_same<T, double>::value && D == 2) ? VolCfg<NP>::EB_SPLIT64_2D : VolCfg<NP>::EB_SPLIT;
+    constexpr int EB = std::is_same<T, double>::value ? VolCfg<NP>::EB_SPLIT : VolCfg<NP>::EB_BULK;
     int nb = (n_split + EB - 1) / EB;
     ProfScope ps(c, PG_SPLIT, s);
-    // the split kernel also forms the viscous volume terms (it has D_i w)
-    const int S = c->n_e * c->n_slot;
-    {
-      // the float32 variant is sized for four blocks per SM and the 3D viscous
-      // variants for two: ask for the shared memory they need
-      static bool carve_set = false;
-      if (!carve_set) {
-        if (!std::is_same<T, double>::value) {
-          cudaFuncSetAttribute(split_volume_kernel<T, D, NP, EB, false, true>,
-                               cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-          cudaFuncSetAttribute(split_volume_kernel<T, D, NP, EB, false, true, true>,
-                               cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        }
-        cudaFuncSetAttribute(split_volume_kernel<T, D, NP, EB, true>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
-        cudaFuncSetAttribute(split_volume_kernel<T, D, NP, EB, true, false, true>,
-                             cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        carve_set = true;
-      }
-    }
+    double* pp = prod ? prod + np_used : nullptr;
     if (visc && c->ent_part && c->b.node_cache) {
       // first stage of a relaxation step: the kernel also forms the entropy of u_n
-      split_volume_kernel<T, D, NP, EB, true, false, true><<<nb, EB * NP, 0, s>>>(
-          u, r, ops, c->b.ops32lo, c->b.rows, c->b.J, sat, lsplit, n_split, ph, ph64, c->b.status,
-          prod ? prod + np_used : nullptr, c->prm.heat_flux, c->b.nu, c->b.va, c->b.fv, c->b.ops64, nullptr, S,
-          c->ent_part, c->b.node_cache, prod ? c->b.wslot : nullptr);
+      split_launch<T, D, NP, EB, true, false, true>(c, u, r, sat, lsplit, n_split, nb, pp, c->ent_part, s);
       c->ent_n = nb;
     } else if (visc)
-      split_volume_kernel<T, D, NP, EB, true><<<nb, EB * NP, 0, s>>>(
-          u, r, ops, c->b.ops32lo, c->b.rows, c->b.J, sat, lsplit, n_split, ph, ph64, c->b.status,
-          prod ? prod + np_used : nullptr, c->prm.heat_flux, c->b.nu, c->b.va, c->b.fv, c->b.ops64, nullptr, S,
-          nullptr, nullptr, prod ? c->b.wslot : nullptr);
+      split_launch<T, D, NP, EB, true, false, false>(c, u, r, sat, lsplit, n_split, nb, pp, nullptr, s);
     else if (cached && scheme == ESPLIT_SCHEME_SPLIT && c->ent_part && c->b.node_cache) {
-      split_volume_kernel<T, D, NP, EB, false, true, true><<<nb, EB * NP, 0, s>>>(
-          u, r, ops, c->b.ops32lo, c->b.rows, c->b.J, sat, lsplit, n_split, ph, ph64, c->b.status,
-          prod ? prod + np_used : nullptr, -1, nullptr, nullptr, nullptr, nullptr, c->b.fcache, S, c->ent_part,
-          c->b.node_cache);
+      split_launch<T, D, NP, EB, false, true, true>(c, u, r, sat, lsplit, n_split, nb, pp, c->ent_part, s);
       c->ent_n = nb;
     } else if (cached)
-      split_volume_kernel<T, D, NP, EB, false, true><<<nb, EB * NP, 0, s>>>(
-          u, r, ops, c->b.ops32lo, c->b.rows, c->b.J, sat, lsplit, n_split, ph, ph64, c->b.status,
-          prod ? prod + np_used : nullptr, -1, nullptr, nullptr, nullptr, nullptr, c->b.fcache, S);
+      split_launch<T, D, NP, EB, false, true, false>(c, u, r, sat, lsplit, n_split, nb, pp, nullptr, s);
     else
-      split_volume_kernel<T, D, NP, EB, false><<<nb, EB * NP, 0, s>>>(
-          u, r, ops, c->b.ops32lo, c->b.rows, c->b.J, sat, lsplit, n_split, ph, ph64, c->b.status,
-          prod ? prod + np_used : nullptr, -1, nullptr, nullptr, nullptr, nullptr, nullptr, S);
+      split_launch<T, D, NP, EB, false, false, false>(c, u, r, sat, lsplit, n_split, nb, pp, nullptr, s);
     c->launches++;
     np_used += nb;
   }

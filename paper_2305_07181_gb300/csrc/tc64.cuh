@@ -1,0 +1,402 @@
+// Float64 operator contractions  out[c][m] = sum_n D_i[m][n] x[c][n]  of one
+// element on the fp16 tensor cores, by error-free slicing (the integer form of
+// the Ozaki scheme: Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012).
+//
+// What bounds it, and why: the float64 pipe of GB300 runs 1.68 FMAs per clock
+// and SM, one warp instruction in ~19 clocks, while everything else (integer,
+// float32, warp-level tensor instructions) runs 40 to 1000 times faster.  A
+// float64 FMA loop over the operators therefore spends ~3/4 of the volume
+// kernel on the contractions.  Here they take no float64 instruction at all:
+//   * every row of D_i and every column of x becomes fixed point: a signed
+//     integer of 6 BITS bits times a power of two taken from the row's or the
+//     column's largest entry, cut into 6 signed digits of BITS bits, each exact
+//     in fp16;
+//   * products of digits are sums of integers below 2^24, exact in the float32
+//     accumulators of mma.sync (m16n8k16); digit pairs (j, a) of one weight
+//     level j + a share accumulators;
+//   * the levels are added up as 64-bit integers and rounded once to float64.
+// Digit width: BITS = 10 up to 32 nodes (60 bits: quantisation 2^-60 of the
+// largest entry, far below a float64 rounding), 9 above (54 bits; a digit
+// product sum over 80 nodes and three pairs stays below 2^24).  Levels up to
+// 3 (BITS 10) are exact; of level 4 on (2^-58 of the largest product) at most
+// the last bits round.  Omitted: digit pairs of level > 6, below 2^-59.
+// The result is closer to the exact sum than n_p float64 FMAs are.
+//
+// Tile: the 16 rows of the A operand are 8 columns of x times 2 consecutive
+// digits, the 8 columns of the B operand 8 rows m of D_i, so both digits'
+// accumulators of an output (c, m) sit in one thread.  12 products (14 for
+// BITS 9) of a 16 x 8 x 16 tile cover the 24 digit pairs that matter.  D_i is
+// stored as 60-bit integers, two entries in 16 bytes, digits laid out so that
+// one shift-and-mask step gives the fp16 pair of a digit (half the bytes of
+// pre-cut fp16 digits; the cutting hides behind the float64 pointwise work of
+// the other blocks of the SM).
+//
+// Columns whose largest entry is below 2^-958 count as zero; a column or row
+// with a non-finite entry gives NaN, as a sum over it would.
+#pragma once
+
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace esplit {
+namespace tc {
+
+constexpr int NONFINITE = 1 << 14;  // exponent marker: the column or row holds an Inf or NaN
+
+__host__ __device__ constexpr int bits_for(int np) { return np <= 32 ? 10 : 9; }
+__host__ __device__ constexpr int pairs_for(int np) { return (np + 1) / 2; }
+
+// power-of-two exponent (biased, from the high words) of the largest entry:
+// every entry is below 0.998 2^(E - 1022), within the signed digits' range
+__device__ __forceinline__ int exp_of_max(unsigned hi_abs_max) {
+  const int e = (int)((hi_abs_max + 0x1100u) >> 20);
+  return hi_abs_max >= 0x7FF00000u ? NONFINITE : e;
+}
+
+// x as 6 unsigned BITS-bit fields (most significant first from bit 5 BITS),
+// field = digit + 2^(BITS-1), relative to the exponent E of exp_of_max
+template <int BITS>
+__device__ __forceinline__ unsigned long long fixed_fields(double x, int E) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int e = (int)((hi >> 20) & 0x7ffu);
+  const unsigned long long M = ((unsigned long long)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo;
+  constexpr int UP = 6 * BITS - 54;  // 6 (BITS 10) or 0 (BITS 9)
+  const int d = E < 64 ? 63 : min(E - e, 63);
+  // right shift by d, rounded to nearest
+  unsigned long long v = (((M << (UP + 1)) >> (d & 63)) + 1ULL) >> 1;
+  constexpr unsigned long long BIAS =
+      (1ULL << (BITS - 1)) * (((1ULL << (6 * BITS)) - 1ULL) / ((1ULL << BITS) - 1ULL));
+  return (hi >> 31) ? BIAS - v : BIAS + v;
+}
+
+// ---------------------------------------------------------------------------
+// packed operators: opsP[e][i][m][pair] (uint4) holds D_i[m][2 pair], D_i[m][2 pair + 1]
+//   x: digit 0 in bits 0-9, low 6 bits of digit 2 in bits 10-15 (entry 2 pair;
+//      entry 2 pair + 1 in the upper halfword), y: digit 1, high bits of digit 2;
+//   z, w: digits 3, 4, 5 likewise.  opsE[e][i][m]: the row's exponent.
+// ---------------------------------------------------------------------------
+template <int BITS>
+__device__ __forceinline__ void pack_half(unsigned long long b, unsigned& x, unsigned& y, unsigned& z, unsigned& w) {
+  constexpr unsigned MASK = (1u << BITS) - 1u;
+  const unsigned u0 = (unsigned)(b >> (5 * BITS)) & MASK, u1 = (unsigned)(b >> (4 * BITS)) & MASK;
+  const unsigned u2 = (unsigned)(b >> (3 * BITS)) & MASK, u3 = (unsigned)(b >> (2 * BITS)) & MASK;
+  const unsigned u4 = (unsigned)(b >> BITS) & MASK, u5 = (unsigned)b & MASK;
+  x = u0 | ((u2 & 63u) << 10);
+  y = u1 | ((u2 >> 6) << 10);
+  z = u3 | ((u5 & 63u) << 10);
+  w = u4 | ((u5 >> 6) << 10);
+}
+
+// one thread per (element, direction, row); ops64: [e][2d][n][m], D_i at k = d + i
+template <int BITS>
+__global__ void build_packed_kernel(const double* __restrict__ ops64, int n_e, int d, int np,
+                                    uint4* __restrict__ opsP, short* __restrict__ opsE) {
+  const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= (size_t)n_e * d * np) return;
+  const size_t ei = idx / np;
+  const int m = (int)(idx - ei * np);
+  const size_t e = ei / d;
+  const int i = (int)(ei - e * d);
+  const double* op = ops64 + ((e * 2 * d + d + i) * np) * np + m;
+  unsigned mx = 0;
+  for (int n = 0; n < np; ++n) mx = max(mx, (unsigned)__double2hiint(op[(size_t)n * np]) & 0x7FFFFFFFu);
+  const int E = exp_of_max(mx);
+  opsE[idx] = (short)E;
+  const int pairs = pairs_for(np);
+  uint4* out = opsP + idx * pairs;
+  for (int p = 0; p < pairs; ++p) {
+    uint4 a, b;
+    pack_half<BITS>(fixed_fields<BITS>(op[(size_t)(2 * p) * np], E), a.x, a.y, a.z, a.w);
+    const double v1 = 2 * p + 1 < np ? op[(size_t)(2 * p + 1) * np] : 0.0;
+    pack_half<BITS>(fixed_fields<BITS>(v1, E), b.x, b.y, b.z, b.w);
+    out[p] = make_uint4(a.x | (b.x << 16), a.y | (b.y << 16), a.z | (b.z << 16), a.w | (b.w << 16));
+  }
+}
+
+template <int BITS>
+__device__ __forceinline__ unsigned unbias(unsigned fields) {  // two 16-bit fields -> two fp16 digits
+  const unsigned h = (fields & 0x03FF03FFu) | 0x64006400u;     // 1024 + field
+  const unsigned c = BITS == 10 ? 0x66006600u : 0x65006500u;   // 1024 + 2^(BITS-1)
+  unsigned r;
+  asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(h), "r"(c));
+  return r;
+}
+
+template <int BITS>
+__device__ __forceinline__ void unpack(const uint4& q, unsigned (&s)[6]) {
+  s[0] = unbias<BITS>(q.x);
+  s[1] = unbias<BITS>(q.y);
+  s[2] = unbias<BITS>(((q.x >> 10) & 0x003F003Fu) | ((q.y >> 4) & 0x03C003C0u));
+  s[3] = unbias<BITS>(q.z);
+  s[4] = unbias<BITS>(q.w);
+  s[5] = unbias<BITS>(((q.z >> 10) & 0x003F003Fu) | ((q.w >> 4) & 0x03C003C0u));
+}
+
+__device__ __forceinline__ void mma16(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+__device__ __forceinline__ void mma8(float (&c)[4], unsigned a0, unsigned a1, unsigned b0) {
+  asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(b0));
+}
+
+__device__ __forceinline__ void ldm4(unsigned (&r)[4], unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+
+__device__ __forceinline__ void ldm2(unsigned& r0, unsigned& r1, unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];"
+               : "=r"(r0), "=r"(r1)
+               : "r"(addr)
+               : "memory");
+}
+
+// Sizes of one block's contraction over EB elements of NP nodes.  Columns per
+// element and direction: NF columns that differ by direction and whose results
+// are summed over the directions (f_i -> sum_i D_i f_i), and NW columns shared
+// by the directions, one result each (w -> D_i w).
+template <int D, int NP, int EB, int NF, int NW>
+struct Shape {
+  static constexpr int BITS = bits_for(NP);
+  static constexpr int KP = (NP + 7) / 8 * 8;          // nodes padded to the tile
+  static constexpr int K16 = KP / 16;                  // 16-node tiles, then one of 8 if KP % 16
+  static constexpr bool K8 = KP % 16 != 0;
+  static constexpr int NT = (NP + 7) / 8;              // tiles of 8 output rows
+  // 32-bit words of a digit row: an odd multiple of 4, so that the eight rows
+  // an ldmatrix reads fall in different banks
+  static constexpr int NPW = (KP / 2) % 8 == 4 ? KP / 2 : KP / 2 + 4;
+  static constexpr int COLS = D * NF + NW;             // distinct columns of x
+  static constexpr int MB = (NF + NW + 7) / 8;         // row blocks of 8 columns per direction
+  static constexpr int OUTS = NF + D * NW;             // results per node
+  static constexpr int NPO = (NP + 3) / 8 * 8 + 4;     // row stride of the results (doubles; an odd multiple of 4)
+  static constexpr int NPH = NP | 1;                   // row stride of the high words (odd)
+  static constexpr int T = BITS == 10 ? 6 : 7;         // accumulator tiles
+  // unit of the 64-bit level sums, 2^-UNIT of the digit products' unit: the
+  // sum over NP nodes and D directions stays below 2^63
+  static constexpr int UNIT = BITS == 10 ? (D == 3 ? 62 : 61) : 51;
+  static constexpr size_t DIG_BYTES = (size_t)EB * 6 * COLS * NPW * 4;
+  static constexpr size_t OUT_BYTES = (size_t)EB * OUTS * NPO * 8;
+  static constexpr size_t HI_BYTES = (size_t)EB * COLS * NPH * 4;
+  static constexpr size_t RES_BYTES = OUT_BYTES > HI_BYTES ? OUT_BYTES : HI_BYTES;
+  static constexpr size_t EX_BYTES = (size_t)(EB * COLS + 3) / 4 * 16;
+};
+
+// Sum of the weight levels of one output, in units of 2^UNIT digit-product
+// units: t[k], b[k] the accumulators of level k (even digit of the pair) and
+// k + 1 (odd digit).  Integer sums of at most 2^24 convert exactly.
+template <int BITS, int UNIT, int NP, int T>
+__device__ __forceinline__ long long level_sum(const float (&t)[T], const float (&b)[T]) {
+  // floats whose two parts may together exceed 2^24 are converted one by one
+  const int i0 = __float2int_rn(t[0]);
+  const int i1 = __float2int_rn(t[1] + b[0]);
+  if constexpr (BITS == 10) {
+    const int i2 = NP <= 21 ? __float2int_rn(t[2] + b[1]) : __float2int_rn(t[2]) + __float2int_rn(b[1]);
+    const int i3 = __float2int_rn(t[3]) + __float2int_rn(b[2]);
+    const float low = (t[4] + b[3]) + ((t[5] + b[4]) + b[5] * 0x1p-10f) * 0x1p-10f;
+    const int il = __float2int_rn(low * (UNIT == 62 ? 0.25f : 0.5f));
+    const long long hi = (long long)i0 * (1 << 20) + ((long long)i1 * (1 << 10) + i2);
+    return (hi << (80 - UNIT)) + ((long long)i3 * (1 << (70 - UNIT)) + il);
+  } else {
+    const int i2 = __float2int_rn(t[2] + b[1]);
+    const int i3 = __float2int_rn(t[3]) + __float2int_rn(b[2]);
+    const int i4 = __float2int_rn(t[4]) + __float2int_rn(b[3]);
+    const float low = (t[5] + b[4]) + ((t[6] + b[5]) + b[6] * 0x1p-9f) * 0x1p-9f;
+    const int il = __float2int_rn(low * 0x1p-6f);
+    const long long hi = (long long)i0 * (1 << 18) + ((long long)i1 * (1 << 9) + i2);
+    return (hi << 21) + ((long long)i3 * (1 << 12) + ((long long)i4 * 8 + il));
+  }
+}
+
+// v 2^(E - shift) rounded to nearest, E the sum of the two exponents of
+// exp_of_max; NaN for a non-finite marker, zero below the normal range
+template <int BITS, int UNIT>
+__device__ __forceinline__ double level_value(long long v, int E) {
+  // x = a 2^(Ex - 1022 - TOT) with TOT = 6 BITS - 1 bits: v has the unit
+  // 2^(UNIT - 2 TOT + E - 2044)
+  constexpr int SH = UNIT - 2 * (6 * BITS - 1) - 2044;
+  const unsigned sgn = (unsigned)((unsigned long long)v >> 63) << 31;
+  const unsigned long long u = (unsigned long long)(v < 0 ? -v : v);
+  const int lz = __clzll((long long)u);
+  const unsigned long long n = u << (lz & 63);
+  const unsigned long long r = (n >> 11) + ((n >> 10) & 1ULL);  // 53 bits, rounded (a carry goes to the exponent)
+  const int ef = 63 - lz + 1023 + SH + E;                       // biased exponent
+  unsigned long long bits = r + ((unsigned long long)(unsigned)(ef - 1) << 52);
+  if (ef >= 2046) bits = E >= NONFINITE ? 0x7FF8000000000000ULL : 0x7FF0000000000000ULL;
+  if (ef <= 0 || u == 0) bits = E >= NONFINITE ? 0x7FF8000000000000ULL : 0ULL;
+  return __longlong_as_double((long long)(bits | ((unsigned long long)sgn << 32)));
+}
+
+// v (COLS values of node m of element el) -> shared digit rows.  Three steps
+// with block barriers between them: high words out, column maxima, digits.
+// Every thread of the block calls it; `on`: the thread owns a node.
+template <class S, int NP, int EB, int THREADS>
+__device__ __forceinline__ void digitize(const double (&v)[S::COLS], bool on, int el, int m, unsigned* hiw, int* ex,
+                                         __half* dig) {
+  constexpr int COLS = S::COLS;
+  if (on) {
+#pragma unroll
+    for (int c = 0; c < COLS; ++c)
+      hiw[(el * COLS + c) * S::NPH + m] = (unsigned)__double2hiint(v[c]) & 0x7FFFFFFFu;
+  }
+  __syncthreads();
+  for (int j = threadIdx.x; j < EB * COLS; j += THREADS) {
+    unsigned mx = 0;
+#pragma unroll 6
+    for (int n = 0; n < NP; ++n) mx = max(mx, hiw[j * S::NPH + n]);
+    ex[j] = exp_of_max(mx);
+  }
+  __syncthreads();
+  if (on) {
+    unsigned short* row = reinterpret_cast<unsigned short*>(dig) + (size_t)el * 6 * COLS * (2 * S::NPW) + m;
+    constexpr unsigned MASK = (1u << S::BITS) - 1u;
+#pragma unroll
+    for (int c = 0; c < COLS; ++c) {
+      const unsigned long long b = fixed_fields<S::BITS>(v[c], ex[el * COLS + c]);
+#pragma unroll
+      for (int s = 0; s < 6; s += 2) {
+        const unsigned ua = (unsigned)(b >> ((5 - s) * S::BITS)) & MASK, ub = (unsigned)(b >> ((4 - s) * S::BITS)) & MASK;
+        const unsigned h = unbias<S::BITS>(ua | (ub << 16));
+        row[(s * COLS + c) * (2 * S::NPW)] = (unsigned short)h;
+        row[((s + 1) * COLS + c) * (2 * S::NPW)] = (unsigned short)(h >> 16);
+      }
+    }
+  }
+}
+
+// zero digits of the padding nodes (NP .. KP - 1) of every row of the block
+template <class S, int NP, int EB, int THREADS>
+__device__ __forceinline__ void zero_padding(__half* dig) {
+  if constexpr (S::KP > NP) {
+    constexpr int W = S::KP - NP;
+    unsigned short* d = reinterpret_cast<unsigned short*>(dig);
+    for (int j = threadIdx.x; j < EB * 6 * S::COLS * W; j += THREADS) {
+      const int row = j / W, k = j - row * W;
+      d[row * (2 * S::NPW) + NP + k] = 0;
+    }
+  }
+}
+
+// The contraction of the block's elements: warps take (element, tile of 8
+// rows) tasks, all directions each.  elems: element index of slot el or -1.
+// Results: res[el][k][m], k < NF the sums over the directions, then
+// NF + i NW + q for column q of direction i.
+template <class S, int D, int NP, int EB, int NF, int NW, int THREADS>
+__device__ __forceinline__ void contract(const __half* dig, const int* ex, const int* elems,
+                                         const uint4* __restrict__ opsP, const short* __restrict__ opsE, double* res) {
+  constexpr int BITS = S::BITS, MB = S::MB, T = S::T, COLS = S::COLS;
+  constexpr int PAIRS = pairs_for(NP);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int g = lane >> 2, t4 = lane & 3;
+  const unsigned dig0 = (unsigned)__cvta_generic_to_shared(dig);
+  for (int task = warp; task < EB * S::NT; task += THREADS / 32) {
+    const int el = task / S::NT, nt = task - el * S::NT;
+    const int e = elems[el];
+    if (e < 0) continue;
+    const int mrow = nt * 8 + g;  // row of D_i this lane loads
+    const bool mon = mrow < NP;
+    const int mo = nt * 8 + 2 * t4;  // first of the two rows of this lane's results
+    long long fs[MB][2];
+    int fE[MB][2];
+#pragma unroll 1
+    for (int i = 0; i < D; ++i) {
+      const uint4* dp = opsP + (((size_t)e * D + i) * NP + (mon ? mrow : 0)) * PAIRS;
+      const short* de = opsE + ((size_t)e * D + i) * NP;
+      // ldmatrix row addresses: matrices 0, 2 hold digit 2a, 1, 3 digit 2a + 1
+      unsigned addr[MB];
+#pragma unroll
+      for (int mb = 0; mb < MB; ++mb) {
+        int c = mb * 8 + (lane & 7);
+        if (c >= NF + NW) c = NF + NW - 1;
+        const int col = c < NF ? i * NF + c : D * NF + (c - NF);
+        addr[mb] = dig0 + (((el * 6 + ((lane >> 3) & 1)) * COLS + col) * S::NPW) * 4 + (lane >> 4) * 16;
+      }
+      float acc[MB][T][4];
+#pragma unroll
+      for (int mb = 0; mb < MB; ++mb)
+#pragma unroll
+        for (int k = 0; k < T; ++k)
+#pragma unroll
+          for (int r = 0; r < 4; ++r) acc[mb][k][r] = 0.0f;
+#pragma unroll
+      for (int kt = 0; kt < S::K16; ++kt) {
+        uint4 qa = make_uint4(0u, 0u, 0u, 0u), qb = qa;
+        if (mon) {
+          if (kt * 8 + t4 < PAIRS) qa = __ldg(&dp[kt * 8 + t4]);
+          if (kt * 8 + 4 + t4 < PAIRS) qb = __ldg(&dp[kt * 8 + 4 + t4]);
+        }
+        unsigned b0[6], b1[6];
+        unpack<BITS>(qa, b0);
+        unpack<BITS>(qb, b1);
+#pragma unroll
+        for (int mb = 0; mb < MB; ++mb)
+#pragma unroll
+          for (int a = 0; a < 3; ++a) {
+            unsigned A[4];
+            ldm4(A, addr[mb] + (2 * a * COLS * S::NPW) * 4 + kt * 32);
+#pragma unroll
+            for (int j = 0; j < 6; ++j)
+              if (j + 2 * a < T) mma16(acc[mb][j + 2 * a], A, b0[j], b1[j]);
+          }
+      }
+      if constexpr (S::K8) {
+        constexpr int kt = S::K16;
+        uint4 qa = make_uint4(0u, 0u, 0u, 0u);
+        if (mon && kt * 8 + t4 < PAIRS) qa = __ldg(&dp[kt * 8 + t4]);
+        unsigned b0[6];
+        unpack<BITS>(qa, b0);
+#pragma unroll
+        for (int mb = 0; mb < MB; ++mb)
+#pragma unroll
+          for (int a = 0; a < 3; ++a) {
+            unsigned A0, A1;
+            ldm2(A0, A1, addr[mb] - (lane >> 4) * 16 + (2 * a * COLS * S::NPW) * 4 + kt * 32);
+#pragma unroll
+            for (int j = 0; j < 6; ++j)
+              if (j + 2 * a < T) mma8(acc[mb][j + 2 * a], A0, A1, b0[j]);
+          }
+      }
+      // levels -> 64-bit sums -> float64, two rows of one column per lane
+#pragma unroll
+      for (int mb = 0; mb < MB; ++mb) {
+        const int c = mb * 8 + g;
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          float tt[T], bb[T];
+#pragma unroll
+          for (int k = 0; k < T; ++k) {
+            tt[k] = acc[mb][k][r];
+            bb[k] = acc[mb][k][2 + r];
+          }
+          long long J = level_sum<BITS, S::UNIT, NP, T>(tt, bb);
+          const int col = c < NF ? i * NF + c : D * NF + (c - NF);
+          const bool live = c < NF + NW && mo + r < NP;
+          int E = live ? ex[el * COLS + col] + (int)__ldg(&de[mo + r]) : 0;
+          if (NF > 0 && c < NF) {  // align with the sum over the directions so far
+            if (i > 0) {
+              const int Em = max(E, fE[mb][r]);
+              J = (J >> min(Em - E, 63)) + (fs[mb][r] >> min(Em - fE[mb][r], 63));
+              E = Em;
+            }
+            fs[mb][r] = J;
+            fE[mb][r] = E;
+          }
+          if (live && (c >= NF || i == D - 1)) {
+            const int k = c < NF ? c : NF + i * NW + (c - NF);
+            res[((size_t)el * S::OUTS + k) * S::NPO + mo + r] = level_value<BITS, S::UNIT>(J, E);
+          }
+        }
+      }
+    }
+  }
+}
+
+}  // namespace tc
+}  // namespace esplit
