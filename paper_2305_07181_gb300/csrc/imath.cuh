@@ -5,7 +5,7 @@
 // float64 log and exp (fmath.cuh) take 17 and 14 float64 instructions; these
 // take none, ~60 integer and float32 instructions each, which hide behind the
 // float64 work around them.  Numbers are fixed point, 64-bit integers of
-// 2^-57: absolute error of the logarithm below 2^-55.8 whatever its size, so a
+// 2^-57: absolute error of the logarithm below 2^-55.5 whatever its size, so a
 // power formed from it (q = rho^a p^b) is good to a few 2^-55 relative, while
 // a float64 logarithm of size 2 alone carries 2^-53 into the exponential.
 //
@@ -110,7 +110,7 @@ IM_FN double exp_fixed(long long X) {
   return __longlong_as_double((long long)(m + ((unsigned long long)(1023 + (N >> 9) - lz) << 52)));
 }
 
-// X 2^-57 as a float64, rounded to nearest
+// X 2^-57 as a float64, rounded to nearest (ties away from zero)
 IM_FN double to_double(long long X) {
   const unsigned long long u = (unsigned long long)(X < 0 ? -X : X);
   const int lz = __clzll((long long)u);

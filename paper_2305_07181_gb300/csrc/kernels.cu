@@ -1584,8 +1584,9 @@ __global__ void __launch_bounds__(256) entropy_kernel(const double* __restrict__
     const double y = 1.0 / (rho * P);
     const double ir = P * y, ip = (rho * rho) * y, p = P * ir;
     // S_H = beta rho (p rho^-gam)^(1/(alpha+gam)) = beta q p, log q = a_q log rho + b_q log p
-    const double lnq = c.a_q * fm::log(rho) + c.b_q * fm::log(p);
-    const double sH = c.beta * fm::exp(lnq) * p;
+    double lnp, lnq, q;
+    node_logs(rho, p, c, lnp, lnq, q);
+    const double sH = c.beta * q * p;
     double H = c_ref.H[m] * __ldg(&J[e * NP + m]);
     v[0] = H * sH;
     v[1] = H * fabs(sH);

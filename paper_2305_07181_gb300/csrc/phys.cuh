@@ -8,8 +8,11 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <type_traits>
+
 #include "dual.cuh"
 #include "fmath.cuh"
+#include "imath.cuh"
 
 namespace esplit {
 
@@ -33,6 +36,10 @@ struct Phys {
   // Taylor coefficients of g(eps) = ((1+eps)^r - 1)/(r eps) for r = r1, r2
   // (c_0 = 1, c_k = c_(k-1) (r - k)/(k + 1)), used by exp_avg
   T ser1[16], ser2[16];
+  // a_q, b_q, r1, r2 in units of 2^-60 for the fixed-point logarithms
+  // (imath.cuh); im_ok: all below 8 in size
+  long long a60, b60, r160, r260;
+  int im_ok;
 };
 
 template <typename T>
@@ -60,6 +67,15 @@ __host__ inline Phys<T> make_phys(double gam, double beta, double R, double mu, 
   c.kappa = (T)(mu * gam * R / ((gam - 1.0) * Pr));
   c.R = (T)R;
   double r1 = -gam / alpha, r2 = (1.0 - gam) / alpha;
+  const double pw[4] = {alpha / (alpha + gam), (1.0 - alpha - gam) / (alpha + gam), r1, r2};
+  c.im_ok = 1;
+  for (int k = 0; k < 4; ++k)
+    if (!(fabs(pw[k]) < 8.0)) c.im_ok = 0;
+  const double sc = c.im_ok ? 1152921504606846976.0 : 0.0;  // 2^60
+  c.a60 = (long long)(pw[0] * sc);
+  c.b60 = (long long)(pw[1] * sc);
+  c.r160 = (long long)(pw[2] * sc);
+  c.r260 = (long long)(pw[3] * sc);
   double a1 = 1.0, a2 = 1.0;
   for (int k = 0; k < 16; ++k) {
     if (k > 0) {
@@ -105,6 +121,26 @@ __device__ __forceinline__ bool t_finite_bits(const Dual<N>& x) {
   return t_finite_bits(x.v);
 }
 
+// 1/d by the cubic iteration y0 (1 + e + e^2), e = 1 - d y0 (Chebyshev's
+// method), from the hardware's 20-bit estimate: three float64 FMAs, where the
+// division takes about nine float64 instructions.  The error before the last
+// rounding is e^3 < 2^-57 relative.  Subnormal d gives a NaN where the
+// division gives a huge value: such states are not physical (t_positive
+// passes them, the logarithms then fail) or columns of no weight.
+__device__ __forceinline__ double rcp64(double d) {
+  double y0;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(d));
+  const double e = fma(-d, y0, 1.0);
+  return fma(y0, fma(e, e, e), y0);
+}
+template <typename T>
+__device__ __forceinline__ T t_rcp(const T& d) {
+  if constexpr (std::is_same<T, double>::value)
+    return rcp64(d);
+  else
+    return T(1) / d;
+}
+
 // Nodal state: primitives, q = z_1 of Eq. (45) (= -W_nc), Harten entropy
 // variables W of Eq. (25).
 template <typename T, int D>
@@ -114,6 +150,30 @@ struct Node {
   T ir;        // 1/rho
   T W[D + 2];
 };
+
+// log p, log q and q = rho^a_q p^b_q: in fixed point (imath.cuh) inside its
+// domain, which holds every ordinary state; the float64 functions otherwise.
+__device__ __forceinline__ void node_logs(double rho, double p, const Phys<double>& c, double& lnp, double& lnq,
+                                          double& q) {
+  long long lr, lp, la, lb;
+  if (c.im_ok && im::log_fixed(rho, lr) && im::log_fixed(p, lp) && im::mul_q60(lr, c.a60, la) &&
+      im::mul_q60(lp, c.b60, lb)) {
+    lnp = im::to_double(lp);
+    lnq = im::to_double(la + lb);
+    q = im::exp_fixed(la + lb);
+  } else {
+    lnp = t_log(p);
+    lnq = c.a_q * t_log(rho) + c.b_q * lnp;
+    q = t_exp(lnq);
+  }
+}
+
+// exp(r l) for a power r (r60: in units of 2^-60) and a logarithm l
+__device__ __forceinline__ double pow_from_log(double l, double r, long long r60, const Phys<double>& c) {
+  long long L, X;
+  if (c.im_ok && im::from_double(l, L) && im::mul_q60(L, r60, X)) return im::exp_fixed(X);
+  return t_exp(r * l);
+}
 
 // Returns false for a non-physical state (rho <= 0, p <= 0 or NaN).
 template <typename T, int D, typename C>
@@ -130,9 +190,13 @@ __device__ __forceinline__ bool node_from_u(const T* u, const C& c, Node<T, D>& 
   n.e = u[D + 1];
   n.p = c.gm1 * (n.e - T(0.5) * n.rho * n.v2);
   bool ok = t_positive(n.rho) && t_positive(n.p) && t_finite_bits(n.e);
-  n.lnp = t_log(n.p);
-  n.lnq = c.a_q * t_log(n.rho) + c.b_q * n.lnp;
-  n.q = t_exp(n.lnq);
+  if constexpr (std::is_same<T, double>::value) {
+    node_logs(n.rho, n.p, c, n.lnp, n.lnq, n.q);
+  } else {
+    n.lnp = t_log(n.p);
+    n.lnq = c.a_q * t_log(n.rho) + c.b_q * n.lnp;
+    n.q = t_exp(n.lnq);
+  }
   n.W[0] = n.q * (c.w1c * n.p * ir - T(0.5) * n.v2);
 #pragma unroll
   for (int i = 0; i < D; ++i) n.W[1 + i] = n.q * n.V[i];
@@ -329,8 +393,13 @@ __device__ __forceinline__ void dU_dW_apply(const Node<T, D>& n, const JvpPrep<T
 // dissipation: P1 = z_1^r1 = q^r1, P2 = z_nc^r2 = p^r2.
 template <typename T, int D, typename C>
 __device__ __forceinline__ void z_powers(const Node<T, D>& n, const C& c, T& P1, T& P2) {
-  P1 = t_exp(c.r1 * n.lnq);
-  P2 = t_exp(c.r2 * n.lnp);
+  if constexpr (std::is_same<T, double>::value) {
+    P1 = pow_from_log(n.lnq, c.r1, c.r160, c);
+    P2 = pow_from_log(n.lnp, c.r2, c.r260, c);
+  } else {
+    P1 = t_exp(c.r1 * n.lnq);
+    P2 = t_exp(c.r2 * n.lnp);
+  }
 }
 
 // Exponential average of Eq. (47), {u^(r-1)}_e = (a^r - b^r)/(r (a - b)),
