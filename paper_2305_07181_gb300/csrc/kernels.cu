@@ -585,10 +585,19 @@ struct SplitCfg {
   static constexpr size_t SMEM =
       TENSOR ? S::DIG_BYTES + S::RES_BYTES + S::EX_BYTES + EB * sizeof(int)
              : (size_t)EB * (D + 1) * NC * NP * sizeof(double);
+  // Resident blocks to compile for.  The phases are chains of dependent
+  // instructions on different pipes, so warps in flight decide: 24 warps per
+  // SM (80 registers, a few spills) on inviscid triangles, 16 (128 registers)
+  // otherwise, as far as shared memory allows.  Measured with the operators
+  // fetched ahead: 18 nodes 5 -> 6 blocks 173 -> 167 us per launch (32,768
+  // triangles), 58 nodes 3 -> 4 blocks 170 -> 160 us (3,072 tetrahedra).
+  static constexpr int BY_SMEM = (int)(233472 / (SMEM + 2048));  // 228 KB per SM; block sums and 1 KB reserved per block
+  static constexpr int BY_REGS = (TENSOR && D == 2 && !VISC ? 768 : D == 2 && !VISC ? 640 : 512) / THREADS;
+  static constexpr int BLOCKS = BY_SMEM < BY_REGS ? BY_SMEM : BY_REGS;
 };
 
 template <int D, int NP, int EB, bool VISC, bool CACHE = false, bool ENT = false>
-__global__ void __launch_bounds__(round32(EB * NP)) split_volume_kernel(
+__global__ void __launch_bounds__(round32(EB * NP), SplitCfg<D, NP, EB, VISC>::BLOCKS) split_volume_kernel(
     const double* __restrict__ u, double* __restrict__ r, const double* __restrict__ ops64,
     const uint4* __restrict__ opsP, const short* __restrict__ opsE, const double* __restrict__ J,
     const double* __restrict__ sat, const int* __restrict__ list, int n_list, Phys<double> c64,
@@ -607,6 +616,10 @@ __global__ void __launch_bounds__(round32(EB * NP)) split_volume_kernel(
   int li = blockIdx.x * EB + el;
   bool active = (el < EB) && (li < n_list);
   int e = active ? (list ? list[li] : li) : 0;
+  if constexpr (Cfg::TENSOR) {
+    constexpr unsigned OPB = D * NP * tc::pairs_for(NP) * sizeof(uint4);  // an element's operators
+    if (m == 0 && active) tc::prefetch_l2(opsP + (size_t)e * (OPB / sizeof(uint4)), OPB);
+  }
   Node<double, D> nd;
   double vals[S::COLS];  // f_i, then w
 #pragma unroll

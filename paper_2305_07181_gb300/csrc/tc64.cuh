@@ -176,7 +176,9 @@ struct Shape {
   static constexpr int COLS = D * NF + NW;             // distinct columns of x
   static constexpr int MB = (NF + NW + 7) / 8;         // row blocks of 8 columns per direction
   static constexpr int OUTS = NF + D * NW;             // results per node
-  static constexpr int NPO = (NP + 3) / 8 * 8 + 4;     // row stride of the results (doubles; an odd multiple of 4)
+  // row stride of the results (doubles): an odd multiple of 4 against bank
+  // conflicts, except where the shorter row lets a sixth block on the SM
+  static constexpr int NPO = NP == 18 ? 18 : (NP + 3) / 8 * 8 + 4;
   static constexpr int NPH = NP | 1;                   // row stride of the high words (odd)
   static constexpr int T = BITS == 10 ? 6 : 7;         // accumulator tiles
   // unit of the 64-bit level sums, 2^-UNIT of the digit products' unit: the
@@ -229,8 +231,11 @@ __device__ __forceinline__ double level_value(long long v, int E) {
   const unsigned long long r = (n >> 11) + ((n >> 10) & 1ULL);  // 53 bits, rounded (a carry goes to the exponent)
   const int ef = 63 - lz + 1023 + SH + E;                       // biased exponent
   unsigned long long bits = r + ((unsigned long long)(unsigned)(ef - 1) << 52);
-  if (ef >= 2046) bits = E >= NONFINITE ? 0x7FF8000000000000ULL : 0x7FF0000000000000ULL;
-  if (ef <= 0 || u == 0) bits = E >= NONFINITE ? 0x7FF8000000000000ULL : 0ULL;
+  if ((unsigned)(ef - 1) >= 2045u) {  // overflow, underflow or a non-finite marker
+    bits = ef > 0 ? 0x7FF0000000000000ULL : 0ULL;
+    if (E >= NONFINITE) bits = 0x7FF8000000000000ULL;
+  }
+  if (u == 0 && E < NONFINITE) bits = 0ULL;
   return __longlong_as_double((long long)(bits | ((unsigned long long)sgn << 32)));
 }
 
@@ -284,6 +289,12 @@ __device__ __forceinline__ void zero_padding(__half* dig) {
   }
 }
 
+// asks for bytes [p, p + n) in L2 (p and n multiples of 16): one request of the
+// bulk-copy engine, issued before the pointwise phase whose ~10 us hide it
+__device__ __forceinline__ void prefetch_l2(const void* p, unsigned n) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(n) : "memory");
+}
+
 // The contraction of the block's elements: warps take (element, tile of 8
 // rows) tasks, all directions each.  elems: element index of slot el or -1.
 // Results: res[el][k][m], k < NF the sums over the directions, then
@@ -296,18 +307,33 @@ __device__ __forceinline__ void contract(const __half* dig, const int* ex, const
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t4 = lane & 3;
   const unsigned dig0 = (unsigned)__cvta_generic_to_shared(dig);
+  // operator entries of one (task, direction): two loads per 16-node tile, one
+  // for an 8-node tile; up to 32 nodes the next direction's (or task's) are
+  // issued before the current one's digit sums are added up
+  constexpr int NQ = 2 * S::K16 + (S::K8 ? 1 : 0);
+  constexpr bool AHEAD = NP <= 32;
+  auto fetch = [&](int task, int i, uint4 (&q)[NQ]) {
+#pragma unroll
+    for (int k = 0; k < NQ; ++k) q[k] = make_uint4(0u, 0u, 0u, 0u);
+    if (task >= EB * S::NT) return;
+    const int el = task / S::NT, mrow = (task - el * S::NT) * 8 + g, e = elems[el];
+    if (e < 0 || mrow >= NP) return;
+    const uint4* dp = opsP + (((size_t)e * D + i) * NP + mrow) * PAIRS;
+#pragma unroll
+    for (int k = 0; k < NQ; ++k)
+      if (k * 4 + t4 < PAIRS) q[k] = __ldcs(&dp[k * 4 + t4]);
+  };
+  uint4 qn[NQ];
+  if constexpr (AHEAD) fetch(warp, 0, qn);
   for (int task = warp; task < EB * S::NT; task += THREADS / 32) {
     const int el = task / S::NT, nt = task - el * S::NT;
     const int e = elems[el];
-    if (e < 0) continue;
-    const int mrow = nt * 8 + g;  // row of D_i this lane loads
-    const bool mon = mrow < NP;
+    if (e < 0) continue;             // only behind the last element of the list
     const int mo = nt * 8 + 2 * t4;  // first of the two rows of this lane's results
     long long fs[MB][2];
     int fE[MB][2];
 #pragma unroll 1
     for (int i = 0; i < D; ++i) {
-      const uint4* dp = opsP + (((size_t)e * D + i) * NP + (mon ? mrow : 0)) * PAIRS;
       const short* de = opsE + ((size_t)e * D + i) * NP;
       // ldmatrix row addresses: matrices 0, 2 hold digit 2a, 1, 3 digit 2a + 1
       unsigned addr[MB];
@@ -325,16 +351,18 @@ __device__ __forceinline__ void contract(const __half* dig, const int* ex, const
         for (int k = 0; k < T; ++k)
 #pragma unroll
           for (int r = 0; r < 4; ++r) acc[mb][k][r] = 0.0f;
+      uint4 q[NQ];
+      if constexpr (AHEAD) {
+#pragma unroll
+        for (int k = 0; k < NQ; ++k) q[k] = qn[k];
+      } else {
+        fetch(task, i, q);
+      }
 #pragma unroll
       for (int kt = 0; kt < S::K16; ++kt) {
-        uint4 qa = make_uint4(0u, 0u, 0u, 0u), qb = qa;
-        if (mon) {
-          if (kt * 8 + t4 < PAIRS) qa = __ldg(&dp[kt * 8 + t4]);
-          if (kt * 8 + 4 + t4 < PAIRS) qb = __ldg(&dp[kt * 8 + 4 + t4]);
-        }
         unsigned b0[6], b1[6];
-        unpack<BITS>(qa, b0);
-        unpack<BITS>(qb, b1);
+        unpack<BITS>(q[2 * kt], b0);
+        unpack<BITS>(q[2 * kt + 1], b1);
 #pragma unroll
         for (int mb = 0; mb < MB; ++mb)
 #pragma unroll
@@ -348,10 +376,8 @@ __device__ __forceinline__ void contract(const __half* dig, const int* ex, const
       }
       if constexpr (S::K8) {
         constexpr int kt = S::K16;
-        uint4 qa = make_uint4(0u, 0u, 0u, 0u);
-        if (mon && kt * 8 + t4 < PAIRS) qa = __ldg(&dp[kt * 8 + t4]);
         unsigned b0[6];
-        unpack<BITS>(qa, b0);
+        unpack<BITS>(q[NQ - 1], b0);
 #pragma unroll
         for (int mb = 0; mb < MB; ++mb)
 #pragma unroll
@@ -363,6 +389,7 @@ __device__ __forceinline__ void contract(const __half* dig, const int* ex, const
               if (j + 2 * a < T) mma8(acc[mb][j + 2 * a], A0, A1, b0[j]);
           }
       }
+      if constexpr (AHEAD) fetch(i + 1 < D ? task : task + THREADS / 32, i + 1 < D ? i + 1 : 0, qn);
       // levels -> 64-bit sums -> float64, two rows of one column per lane
 #pragma unroll
       for (int mb = 0; mb < MB; ++mb) {
