@@ -718,7 +718,7 @@ __global__ void __launch_bounds__(round32(EB * NP), SplitCfg<D, NP, EB, VISC>::B
       }
     }
     double nonc[NC];
-    dflux_dw_sum<D>(nd, jp, c64, -c64.inv_bp1, gd, nonc);
+    dflux_dw_sum<double, D>(nd, jp, c64, -c64.inv_bp1, gd, nonc);
     Hm = c_ref.H[m] * __ldg(&J[(size_t)e * NP + m]);
     const double kf = c64.beta * c64.inv_bp1;
 #pragma unroll

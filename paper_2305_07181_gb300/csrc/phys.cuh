@@ -286,50 +286,51 @@ __device__ __forceinline__ void euler_fluxes(const Node<double, D>& n, const dou
 // out = s sum_i A~_i g_i (Eq. (19)), g_i = D_i w: dflux_dw summed over the
 // directions before the products with the node's state, so that only the
 // temperature and pressure changes are formed per direction:
-//   Q = sum_i V_i dq_i,  div = sum_i dV_i[i],  adv_j = sum_i V_i dV_i[j],
+//   Q = -sum_i V_i dq_i,  div = sum_i dV_i[i],  adv_j = sum_i V_i dV_i[j],
 //   T = sum_i V_i dtheta_i,  A = sum_i V_i drho_i,
 //   out_0 = A + rho div,  out_j = out_0 V_j + rho adv_j + dp_j,
 //   out_E = gam/(gam-1) sum_i V_i dp_i + (|V|^2/2) A + rho V.adv + (e + p) div,
 //   dtheta_i = (g_i0 + V.g_im + g_iE (W_1/q + |V|^2)) / (w1c q).
 // 48 float64 operations in 2D and 72 in 3D; dflux_dw direction by direction
 // takes 72 and 139.  s is carried by the reciprocal 1/q of the linear terms.
-template <int D, typename C>
-__device__ __forceinline__ void dflux_dw_sum(const Node<double, D>& n, const JvpPrep<double>& jp, const C& c, double s,
-                                             const double (&g)[D][D + 2], double* out) {
+template <typename T, int D, typename C>
+__device__ __forceinline__ void dflux_dw_sum(const Node<T, D>& n, const JvpPrep<T>& jp, const C& c, double s,
+                                             const double (&g)[D][D + 2], T* out) {
   constexpr int NC = D + 2;
-  const double iq = s * jp.iq, k = c.inv_w1c * iq, we = jp.w0q + n.v2, c1 = c.b_q * jp.itheta;
-  const double rt = jp.rq * jp.theta, cp = n.rho - rt * c1, cq = rt * iq;
-  double Q = 0.0, T = 0.0, P = 0.0, tr = 0.0, dp[D], S[D];
+  const T iq = s * jp.iq, k = c.inv_w1c * iq, we = jp.w0q + n.v2, c1 = c.b_q * jp.itheta;
+  const T rt = jp.rq * jp.theta, cp = n.rho - rt * c1, cq = rt * iq;
+  T Q, TT, P, dp[D], S[D];
+  double tr = 0.0;
 #pragma unroll
   for (int i = 0; i < D; ++i) {
-    double t = g[i][0] + g[i][NC - 1] * we;
+    T t = g[i][0] + g[i][NC - 1] * we;
 #pragma unroll
-    for (int j = 0; j < D; ++j) t += n.V[j] * g[i][1 + j];
-    t *= k;
+    for (int j = 0; j < D; ++j) t = t + n.V[j] * g[i][1 + j];
+    t = t * k;
     dp[i] = cp * t - cq * g[i][NC - 1];  // drho theta + rho dtheta, dq = -g_E
     if (i == 0) {
-      Q = -n.V[0] * g[0][NC - 1];
-      T = n.V[0] * t;
+      Q = n.V[0] * g[0][NC - 1];
+      TT = n.V[0] * t;
       P = n.V[0] * dp[0];
       tr = g[0][1];
     } else {
-      Q -= n.V[i] * g[i][NC - 1];
-      T += n.V[i] * t;
-      P += n.V[i] * dp[i];
+      Q = Q + n.V[i] * g[i][NC - 1];
+      TT = TT + n.V[i] * t;
+      P = P + n.V[i] * dp[i];
       tr += g[i][1 + i];
     }
 #pragma unroll
     for (int j = 0; j < D; ++j) S[j] = i == 0 ? n.V[0] * g[0][1 + j] : S[j] + n.V[i] * g[i][1 + j];
   }
-  const double div = iq * (tr - Q);
-  const double A = jp.rq * (iq * Q - c1 * T);
-  const double M = A + n.rho * div;
-  const double riq = n.rho * iq;
-  double va = 0.0;
+  const T div = iq * (Q + tr);  // Q here is sum_i V_i g_iE = -sum_i V_i dq_i
+  const T A = jp.rq * (-(iq * Q) - c1 * TT);
+  const T M = A + n.rho * div;
+  const T riq = n.rho * iq;
+  T va;
   out[0] = M;
 #pragma unroll
   for (int j = 0; j < D; ++j) {
-    const double ra = riq * (S[j] - n.V[j] * Q);  // rho adv_j
+    const T ra = riq * (S[j] + n.V[j] * Q);  // rho adv_j
     va = j == 0 ? n.V[0] * ra : va + n.V[j] * ra;
     out[1 + j] = M * n.V[j] + (ra + dp[j]);
   }

@@ -9,6 +9,7 @@
 #include "phys.cuh"
 #include "visc_flux.cuh"
 #include "reduce.cuh"
+#include "tc64.cuh"
 
 namespace esplit {
 

@@ -411,78 +411,185 @@ __global__ void __launch_bounds__(64) face_vjp_kernel(const double* __restrict__
   }
 }
 
+// Volume part of the reverse.  The transposed operators follow from the
+// forward ones: D_i = H^-1 Q_i and Q_i + Q_i^T = E_i (diagonal, nu_i at the
+// facet nodes) give D_i^T y = E_i (y/H) - H D_i (y/H), so
+//   M_i^T cot = [E_i (cot/H) + beta H D_i (cot/H)] / (beta+1),
+//   wbar = sum_i D_i^T gbar_i = sum_i E_i (gbar_i/H) - H sum_i D_i (gbar_i/H):
+// both contractions are forward ones, on the tensor cores as in the split
+// volume kernel (tc64.cuh), with 2 n_c columns (w, cot/H) and then n_c
+// summed ones; 7-node triangles keep float64 loops.  On the float64 pipe the
+// pointwise part is left.
 template <int D, int NP, int EB>
-__global__ void __launch_bounds__(EB * NP) split_vjp_kernel(const double* __restrict__ u,
-                                                            const double* __restrict__ cot,
-                                                            const double* __restrict__ ops,
-                                                            const double* __restrict__ gsat, int n_e,
-                                                            double* __restrict__ grad, Phys<double> c) {
+struct VjpCfg {
+  static constexpr bool TENSOR = NP > 8;
+  static constexpr int NC = D + 2;
+  static constexpr int THREADS = round32(EB * NP);
+  using S1 = tc::Shape<D, NP, EB, 0, 2 * NC>;
+  using S2 = tc::Shape<D, NP, EB, NC, 0>;
+  static constexpr size_t mx(size_t a, size_t b) { return a > b ? a : b; }
+  static constexpr size_t DIG = mx(S1::DIG_BYTES, S2::DIG_BYTES), RES = mx(S1::RES_BYTES, S2::RES_BYTES);
+  static constexpr size_t EXB = mx(S1::EX_BYTES, S2::EX_BYTES);
+  static constexpr size_t SMEM = TENSOR ? DIG + RES + EXB + EB * sizeof(int) : (size_t)EB * D * NC * NP * 8;
+  static constexpr int BY_SMEM = (int)(233472 / (SMEM + 1024));
+  static constexpr int BY_REGS = (NP > 32 ? 384 : 512) / THREADS;
+  static constexpr int BLOCKS = BY_SMEM < BY_REGS ? BY_SMEM : BY_REGS;
+};
+
+template <int D, int NP, int EB>
+__global__ void __launch_bounds__(round32(EB * NP), VjpCfg<D, NP, EB>::BLOCKS) split_vjp_kernel(
+    const double* __restrict__ u, const double* __restrict__ cot, const double* __restrict__ ops,
+    const uint4* __restrict__ opsP, const short* __restrict__ opsE, const double* __restrict__ J,
+    const double* __restrict__ ihd, const double* __restrict__ nu, const double* __restrict__ gsat, int n_e,
+    double* __restrict__ grad, Phys<double> c) {
   constexpr int NC = D + 2;
-  __shared__ double sw[EB][NC][NP];
-  __shared__ double sv[EB][NC][NP];
-  __shared__ double sgb[EB][D][NC][NP];
+  using Cfg = VjpCfg<D, NP, EB>;
+  using S1 = typename Cfg::S1;
+  using S2 = typename Cfg::S2;
+  constexpr int THREADS = Cfg::THREADS;
+  static_assert(!Cfg::TENSOR || S1::NPW == S2::NPW, "one digit row stride: the padding stays zero");
+  extern __shared__ __align__(16) unsigned char vjp_smem[];
   const int NS = c_ref.n_slot;
-  int el = threadIdx.x / NP;
-  int m = threadIdx.x - el * NP;
-  int e = blockIdx.x * EB + el;
-  bool active = e < n_e;
+  const int el = threadIdx.x / NP;
+  const int m = threadIdx.x - el * NP;
+  const int e = blockIdx.x * EB + el;
+  const bool slot = el < EB, active = slot && e < n_e;
+  const int ms = slot ? m : 0, els = slot ? el : 0;
   Node<double, D> nd;
-  double uu[NC], vv[NC];
+  double vv[NC], x1[2 * NC], ih = 0.0, Hm = 0.0;
+#pragma unroll
+  for (int q = 0; q < NC; ++q) vv[q] = 0.0;
+#pragma unroll
+  for (int q = 0; q < 2 * NC; ++q) x1[q] = 0.0;
   if (active) {
+    if constexpr (Cfg::TENSOR) {
+      constexpr unsigned OPB = D * NP * tc::pairs_for(NP) * sizeof(uint4);
+      if (m == 0) tc::prefetch_l2(opsP + (size_t)e * (OPB / sizeof(uint4)), OPB);
+    }
+    double uu[NC];
+    ih = __ldg(&ihd[(size_t)e * NP + m]);
+    Hm = c_ref.H[m] * __ldg(&J[(size_t)e * NP + m]);
 #pragma unroll
     for (int q = 0; q < NC; ++q) {
       uu[q] = __ldg(&u[((size_t)e * NC + q) * NP + m]);
       vv[q] = __ldg(&cot[((size_t)e * NC + q) * NP + m]);
-      sv[el][q][m] = vv[q];
     }
     node_from_u<double, D>(uu, c, nd);
 #pragma unroll
-    for (int q = 0; q < NC; ++q) sw[el][q][m] = nd.W[q];
+    for (int q = 0; q < NC; ++q) {
+      x1[q] = nd.W[q];
+      x1[NC + q] = vv[q] * ih;
+    }
   }
-  __syncthreads();
-  const double* op = ops + (size_t)(active ? e : 0) * (2 * D * NP * NP);
-  double g[D][NC];
-  if (active) {
+  __half* dig = reinterpret_cast<__half*>(vjp_smem);
+  double* resb = reinterpret_cast<double*>(vjp_smem + Cfg::DIG);
+  int* ex = reinterpret_cast<int*>(vjp_smem + Cfg::DIG + Cfg::RES);
+  int* elems = reinterpret_cast<int*>(vjp_smem + Cfg::DIG + Cfg::RES + Cfg::EXB);
+  double* sx = reinterpret_cast<double*>(vjp_smem);  // float64 loops: [EB][columns][NP]
+  const double* op = ops + (size_t)(active ? e : 0) * (2 * D * NP * NP) + D * NP * NP;
+  double g[D][NC], t[D][NC];  // D_i w, D_i (cot/H)
+  if constexpr (Cfg::TENSOR) {
+    if (m == 0 && slot) elems[el] = active ? e : -1;
+    tc::zero_padding<S1, NP, EB, THREADS>(dig);
+    if constexpr (S2::COLS > S1::COLS) tc::zero_padding<S2, NP, EB, THREADS>(dig);
+    tc::digitize<S1, NP, EB, THREADS>(x1, slot, el, m, reinterpret_cast<unsigned*>(resb), ex, dig);
+    __syncthreads();
+    tc::contract<S1, D, NP, EB, 0, 2 * NC, THREADS>(dig, ex, elems, opsP, opsE, resb);
+    __syncthreads();
+    const double* rs = resb + (size_t)els * S1::OUTS * S1::NPO + ms;
 #pragma unroll
     for (int i = 0; i < D; ++i)
 #pragma unroll
-      for (int q = 0; q < NC; ++q) g[i][q] = 0.0;
-#pragma unroll
-    for (int i = 0; i < D; ++i)
-      for (int n = 0; n < NP; ++n) {
-        double dt = __ldg(&op[((D + i) * NP + n) * NP + m]);  // D_i[m][n]
-#pragma unroll
-        for (int q = 0; q < NC; ++q) g[i][q] += dt * sw[el][q][n];
+      for (int q = 0; q < NC; ++q) {
+        g[i][q] = rs[(i * 2 * NC + q) * S1::NPO];
+        t[i][q] = rs[(i * 2 * NC + NC + q) * S1::NPO];
       }
-    const JvpPrep<double> jp = jvp_prep<double, D>(nd, c);
+    __syncthreads();
+  } else {
+    if (active) {
+#pragma unroll
+      for (int q = 0; q < 2 * NC; ++q) sx[(el * 2 * NC + q) * NP + m] = x1[q];
+    }
+    __syncthreads();
+    if (active) {
+#pragma unroll
+      for (int i = 0; i < D; ++i) {
+#pragma unroll
+        for (int q = 0; q < NC; ++q) g[i][q] = t[i][q] = 0.0;
+#pragma unroll
+        for (int n = 0; n < NP; ++n) {
+          const double dt = __ldg(&op[(i * NP + n) * NP + m]);  // D_i[m][n]
+#pragma unroll
+          for (int q = 0; q < NC; ++q) {
+            g[i][q] += dt * sx[(el * 2 * NC + q) * NP + n];
+            t[i][q] += dt * sx[(el * 2 * NC + NC + q) * NP + n];
+          }
+        }
+      }
+    }
+    __syncthreads();
+  }
+  double x2[S2::COLS];  // gbar_i / H
+#pragma unroll
+  for (int q = 0; q < S2::COLS; ++q) x2[q] = 0.0;
+  JvpPrep<double> jp;
+  if (active) {
+    jp = jvp_prep<double, D>(nd, c);
+    const double sc = -c.inv_bp1 * ih;
 #pragma unroll
     for (int i = 0; i < D; ++i) {
       double a[NC];
       dflux_dw<double, D>(nd, jp, c, i, vv, a);
 #pragma unroll
-      for (int q = 0; q < NC; ++q) sgb[el][i][q][m] = -c.inv_bp1 * a[q];
+      for (int q = 0; q < NC; ++q) x2[i * NC + q] = sc * a[q];
     }
   }
-  __syncthreads();
-  if (!active) return;
-  double fb[D][NC], wb[NC];
+  double wb[NC];  // sum_i D_i (gbar_i / H)
+  if constexpr (Cfg::TENSOR) {
+    tc::digitize<S2, NP, EB, THREADS>(x2, slot, el, m, reinterpret_cast<unsigned*>(resb), ex, dig);
+    __syncthreads();
+    tc::contract<S2, D, NP, EB, NC, 0, THREADS>(dig, ex, elems, opsP, opsE, resb);
+    __syncthreads();
 #pragma unroll
-  for (int q = 0; q < NC; ++q) wb[q] = 0.0;
+    for (int q = 0; q < NC; ++q) wb[q] = resb[((size_t)els * S2::OUTS + q) * S2::NPO + ms];
+  } else {
+    if (active) {
 #pragma unroll
-  for (int i = 0; i < D; ++i)
-#pragma unroll
-    for (int q = 0; q < NC; ++q) fb[i][q] = 0.0;
-#pragma unroll
-  for (int i = 0; i < D; ++i)
-    for (int n = 0; n < NP; ++n) {
-      double mt = __ldg(&op[(i * NP + m) * NP + n]);        // M_i[n][m]
-      double dt = __ldg(&op[((D + i) * NP + m) * NP + n]);  // D_i[n][m]
-#pragma unroll
-      for (int q = 0; q < NC; ++q) {
-        fb[i][q] += mt * sv[el][q][n];
-        wb[q] += dt * sgb[el][i][q][n];
-      }
+      for (int q = 0; q < S2::COLS; ++q) sx[(el * S2::COLS + q) * NP + m] = x2[q];
     }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NC; ++q) wb[q] = 0.0;
+    if (active) {
+#pragma unroll
+      for (int i = 0; i < D; ++i)
+#pragma unroll
+        for (int n = 0; n < NP; ++n) {
+          const double dt = __ldg(&op[(i * NP + n) * NP + m]);
+#pragma unroll
+          for (int q = 0; q < NC; ++q) wb[q] += dt * sx[(el * S2::COLS + i * NC + q) * NP + n];
+        }
+    }
+  }
+  if (!active) return;
+  // fbar_i = M_i^T cot and wbar
+  const int sl = c_ref.node_slot[m];
+  double nv[D];
+#pragma unroll
+  for (int i = 0; i < D; ++i) nv[i] = sl >= 0 ? __ldg(&nu[((size_t)e * NS + sl) * D + i]) : 0.0;
+  const double kH = c.beta * c.inv_bp1 * Hm;
+  double z[NC];
+#pragma unroll
+  for (int q = 0; q < NC; ++q) {
+    double s = 0.0;
+    const double ci = c.inv_bp1 * x1[NC + q];
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      s += nv[i] * x2[i * NC + q];
+      t[i][q] = nv[i] * ci + kH * t[i][q];
+    }
+    z[q] = s - Hm * wb[q];
+  }
   // pointwise part.  With A~_i = dF_i/dW symmetric and dW/du the symmetric
   // Hessian of the entropy,
   //   (dF_i/du)^T fb_i = (dW/du) A~_i fb_i,   (dw/du)^T wb = (dW/du) wb,
@@ -492,14 +599,9 @@ __global__ void __launch_bounds__(EB * NP) split_vjp_kernel(const double* __rest
   // A~_i g_i along W in the single direction cot_m (a one-direction dual
   // number, the state moved by (dU/dW) cot_m):
   //   grad_m = (dW/du) [sum_i A~_i fb_i + wb - 1/(beta+1) sum_i d_cot(A~_i g_i)].
-  const JvpPrep<double> jp = jvp_prep<double, D>(nd, c);
-  double z[NC];
-#pragma unroll
-  for (int q = 0; q < NC; ++q) z[q] = wb[q];
-#pragma unroll
-  for (int i = 0; i < D; ++i) {
+  {
     double a[NC];
-    dflux_dw<double, D>(nd, jp, c, i, fb[i], a);
+    dflux_dw_sum<double, D>(nd, jp, c, 1.0, t, a);
 #pragma unroll
     for (int q = 0; q < NC; ++q) z[q] += a[q];
   }
@@ -508,13 +610,15 @@ __global__ void __launch_bounds__(EB * NP) split_vjp_kernel(const double* __rest
     double du[NC];
     dU_dW_apply<double, D>(nd, jp, c, vv, du);
     // the nodal quantities A~_i depends on, with their tangent along du in
-    // closed form (no logarithm or exponential on the duals):
+    // closed form (no logarithm, exponential or division on the duals):
     //   drho = du_0, dV = (du_m - V drho)/rho, dv2 = 2 V.dV, de = du_E,
     //   dp = (gam-1)(de - (drho v2 + rho dv2)/2), dq = q (a_q drho/rho + b_q dp/p)
+    // and those of jvp_prep: d(1/q) = -dq/q^2, dtheta = (dp - theta drho)/rho, ...
     Node<T1, D> n1;
+    JvpPrep<T1> j1;
     {
-      const double drho = du[0];
-      double dv2 = 0.0;
+      const double drho = du[0], ip = jp.itheta * jp.ir;
+      double hv2 = 0.0;  // V.dV
       n1.rho = T1(nd.rho);
       n1.rho.d[0] = drho;
 #pragma unroll
@@ -522,35 +626,34 @@ __global__ void __launch_bounds__(EB * NP) split_vjp_kernel(const double* __rest
         const double dVj = (du[1 + j] - nd.V[j] * drho) * nd.ir;
         n1.V[j] = T1(nd.V[j]);
         n1.V[j].d[0] = dVj;
-        dv2 += 2.0 * nd.V[j] * dVj;
+        hv2 += nd.V[j] * dVj;
       }
       const double de = du[NC - 1];
-      const double dp = c.gm1 * (de - 0.5 * (drho * nd.v2 + nd.rho * dv2));
+      const double dp = c.gm1 * (de - (0.5 * drho * nd.v2 + nd.rho * hv2));
       n1.v2 = T1(nd.v2);
-      n1.v2.d[0] = dv2;
-      n1.e = T1(nd.e);
-      n1.e.d[0] = de;
-      n1.p = T1(nd.p);
-      n1.p.d[0] = dp;
-      n1.ir = T1(nd.ir);
-      n1.ir.d[0] = -nd.ir * nd.ir * drho;
-      n1.q = T1(nd.q);
-      n1.q.d[0] = nd.q * (c.a_q * drho * nd.ir + c.b_q * dp * (jp.itheta * nd.ir));
+      n1.v2.d[0] = 2.0 * hv2;
+      const double lq = c.a_q * drho * nd.ir + c.b_q * dp * ip;  // dq/q
+      const double dth = (dp - jp.theta * drho) * nd.ir;
+      j1.iq = T1(jp.iq);
+      j1.iq.d[0] = -jp.iq * lq;
+      j1.theta = T1(jp.theta);
+      j1.theta.d[0] = dth;
+      j1.itheta = T1(jp.itheta);
+      j1.itheta.d[0] = -jp.itheta * jp.itheta * dth;
+      j1.w0q = T1(jp.w0q);
+      j1.w0q.d[0] = c.w1c * dth - hv2;
+      j1.rq = T1(jp.rq);
+      j1.rq.d[0] = c.inv_apb * drho;
+      j1.ep = T1(jp.ep);
+      j1.ep.d[0] = de + dp;
     }
-    const JvpPrep<T1> j1 = jvp_prep<T1, D>(n1, c);
+    T1 dF[NC];
+    dflux_dw_sum<T1, D>(n1, j1, c, -c.inv_bp1, g, dF);
 #pragma unroll
-    for (int i = 0; i < D; ++i) {
-      T1 gi[NC], dF[NC];
-#pragma unroll
-      for (int q = 0; q < NC; ++q) gi[q] = T1(g[i][q]);
-      dflux_dw<T1, D>(n1, j1, c, i, gi, dF);
-#pragma unroll
-      for (int q = 0; q < NC; ++q) z[q] -= c.inv_bp1 * dF[q].d[0];
-    }
+    for (int q = 0; q < NC; ++q) z[q] += dF[q].d[0];
   }
   double gr[NC];
   dW_dU_apply<double, D>(nd, jp, c, z, gr);
-  int sl = c_ref.node_slot[m];
 #pragma unroll
   for (int cc = 0; cc < NC; ++cc) {
     if (sl >= 0) gr[cc] += __ldg(&gsat[((size_t)e * NC + cc) * NS + sl]);
@@ -570,10 +673,20 @@ static int vjp_np(esplit_ctx* c, const double* u, const double* cot, double* gra
     c->launches++;
   }
   {
-    constexpr int EB = (128 / NP) > 0 ? (128 / NP) : 1;
+    // blocks that fill their warps, as the split volume kernel's
+    constexpr int EB = NP == 7 ? 18 : NP == 12 ? 10 : NP == 18 || NP == 27 ? 7 : NP == 25 ? 5 : 2;
+    using Cfg = VjpCfg<D, NP, EB>;
     int nb = (c->n_e + EB - 1) / EB;
     ProfScope ps(c, PG_SPLIT, s);
-    split_vjp_kernel<D, NP, EB><<<nb, EB * NP, 0, s>>>(u, cot, c->b.ops64, c->b.sat, c->n_e, grad, ph);
+    auto* kern = split_vjp_kernel<D, NP, EB>;
+    static bool attr_set = false;
+    if (!attr_set) {
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
+      cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+      attr_set = true;
+    }
+    kern<<<nb, Cfg::THREADS, Cfg::SMEM, s>>>(u, cot, c->b.ops64, c->b.opsP, c->b.opsE, c->b.J, c->b.ihd, c->b.nu,
+                                             c->b.sat, c->n_e, grad, ph);
     c->launches++;
   }
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
