@@ -260,22 +260,20 @@ __global__ void __launch_bounds__(128) face_kernel(const double* __restrict__ u,
     znode<T, D>(nk, c, zk);
     znode<T, D>(nv, c, zv);
     znode_recips<T, D>(zk);
-    PairAvg<T, D> a;
-    pair_avg<T, D>(zk, zv, c, a);
-    sy_flux_dir<T, D>(a, c, nuv, G);
+    PairSums<D> a;
+    pair_sums<D>(zk, zv, &nk.W[1], &nv.W[1], c, a);
+    sy_flux2<D>(a, nuv, G);
     if (dissipation) {
       const double* ns = nscale + (size_t)pr.x * (D + 1);  // |nu|, nu/|nu| of slot (k, s)
-      const T b = (T)__ldg(&ns[0]);
-      T nh[D];
+      double nh[D], dw[NC];
 #pragma unroll
-      for (int i = 0; i < D; ++i) nh[i] = (T)__ldg(&ns[1 + i]);
-      T dw[NC], out[NC];
+      for (int i = 0; i < D; ++i) nh[i] = __ldg(&ns[1 + i]);
 #pragma unroll
       for (int q = 0; q < NC; ++q) dw[q] = nk.W[q] - nv.W[q];
-      diss_apply<T, D>(a, c, nh, dw, out);
-#pragma unroll
-      for (int q = 0; q < NC; ++q) G[q] += T(0.5) * b * out[q];
+      diss_add2<D>(a, c, nh, dw, __ldg(&ns[0]), G);
     }
+#pragma unroll
+    for (int q = 0; q < NC; ++q) G[q] *= 0.5;
   }
   const double ihk = __ldg(&ihd[(size_t)k * NP + m]), ihv = __ldg(&ihd[(size_t)v * NP + n]);
   double ek[NC], ev[NC];
@@ -329,16 +327,16 @@ __global__ void __launch_bounds__(128) face_kernel(const double* __restrict__ u,
 // inviscid, float64): the same terms as face_kernel (two-point flux,
 // dissipation, the facet part nu . f / H of the split volume term), with the
 // nodal quantities of both sides read from the cache the volume kernels wrote
-// (rho, 1/rho, p, e, q, log q, log p, 1/q, 1/p, V) instead of recomputed, and
+// (rho, W_1, p, e, q, log q, log p, 1/q, 1/p, V) instead of recomputed, and
 // the result added into r.  The
 // entropy production of the facet terms, w . H sat = w_k . (nu f_k - G) +
 // w_v . (G - nu f_v), goes to block partials after the volume kernel's.
 // ---------------------------------------------------------------------------
 template <int D>
 __device__ __forceinline__ void node_from_cache(const double* __restrict__ fc, size_t S, size_t ix,
-                                                const Phys<double>& c, Node<double, D>& n, double& iq, double& ip) {
+                                                Node<double, D>& n, double& iq, double& ip) {
   n.rho = __ldg(&fc[0 * S + ix]);
-  n.ir = __ldg(&fc[1 * S + ix]);
+  n.W[0] = __ldg(&fc[1 * S + ix]);
   n.p = __ldg(&fc[2 * S + ix]);
   n.e = __ldg(&fc[3 * S + ix]);
   n.q = __ldg(&fc[4 * S + ix]);
@@ -346,15 +344,11 @@ __device__ __forceinline__ void node_from_cache(const double* __restrict__ fc, s
   n.lnp = __ldg(&fc[6 * S + ix]);
   iq = __ldg(&fc[7 * S + ix]);
   ip = __ldg(&fc[8 * S + ix]);
-  n.v2 = 0.0;
 #pragma unroll
   for (int i = 0; i < D; ++i) {
     n.V[i] = __ldg(&fc[(9 + i) * S + ix]);
-    n.v2 += n.V[i] * n.V[i];
+    n.W[1 + i] = n.q * n.V[i];
   }
-  n.W[0] = n.q * (c.w1c * n.p * n.ir - 0.5 * n.v2);
-#pragma unroll
-  for (int i = 0; i < D; ++i) n.W[1 + i] = n.q * n.V[i];
   n.W[D + 1] = -n.q;
 }
 
@@ -379,32 +373,28 @@ __global__ void __launch_bounds__(128) face_cached_kernel(double* __restrict__ r
     int m = c_ref.slot_node[s], n = c_ref.slot_node[s2];
     Node<double, D> nk, nv;
     double iqk, ipk, iqv, ipv;
-    node_from_cache<D>(fc, S, (size_t)pr.x, c, nk, iqk, ipk);
-    node_from_cache<D>(fc, S, (size_t)pr.y, c, nv, iqv, ipv);
+    node_from_cache<D>(fc, S, (size_t)pr.x, nk, iqk, ipk);
+    node_from_cache<D>(fc, S, (size_t)pr.y, nv, iqv, ipv);
     ZNode<double, D> zk, zv;
     znode<double, D>(nk, c, zk);
     znode<double, D>(nv, c, zv);
     zk.iq = iqk;
     zk.ip = ipk;
-    PairAvg<double, D> a;
-    pair_avg<double, D>(zk, zv, c, a);
+    PairSums<D> a;
+    pair_sums<D>(zk, zv, &nk.W[1], &nv.W[1], c, a);
     double nuv[D];
 #pragma unroll
     for (int i = 0; i < D; ++i) nuv[i] = __ldg(&nu[((size_t)k * NS + s) * D + i]);
-    double G[NC];
-    sy_flux_dir<double, D>(a, c, nuv, G);
+    double G2[NC];  // twice the flux and the dissipation
+    sy_flux2<D>(a, nuv, G2);
     if (dissipation) {
       const double* ns = nscale + (size_t)pr.x * (D + 1);  // |nu|, nu/|nu| of slot (k, s)
-      const double b = __ldg(&ns[0]);
-      double nh[D];
+      double nh[D], dw[NC];
 #pragma unroll
       for (int i = 0; i < D; ++i) nh[i] = __ldg(&ns[1 + i]);
-      double dw[NC], out[NC];
 #pragma unroll
       for (int q = 0; q < NC; ++q) dw[q] = nk.W[q] - nv.W[q];
-      diss_apply<double, D>(a, c, nh, dw, out);
-#pragma unroll
-      for (int q = 0; q < NC; ++q) G[q] += 0.5 * b * out[q];
+      diss_add2<D>(a, c, nh, dw, __ldg(&ns[0]), G2);
     }
     // the facet part nu . f / H of the split volume term, for split-form sides
     // (ef_mode 1: both, 2: sides whose hybrid flag is 0, 0: none)
@@ -416,7 +406,7 @@ __global__ void __launch_bounds__(128) face_cached_kernel(double* __restrict__ r
     const double ihk = __ldg(&ihd[(size_t)k * NP + m]), ihv = __ldg(&ihd[(size_t)v * NP + n]);
 #pragma unroll
     for (int q = 0; q < NC; ++q) {
-      double gk = ek[q] - G[q], gv = G[q] - ev[q];
+      const double gk = ek[q] - 0.5 * G2[q], gv = 0.5 * G2[q] - ev[q];
       r[((size_t)k * NC + q) * NP + m] += gk * ihk;
       r[((size_t)v * NC + q) * NP + n] += gv * ihv;
       hw += nk.W[q] * gk + nv.W[q] * gv;
@@ -474,8 +464,9 @@ __global__ void __launch_bounds__(128) face_bc_kernel(const double* __restrict__
     const double b = sqrt(b2);
 #pragma unroll
     for (int i = 0; i < D; ++i) nh[i] = nuv[i] / b;
-    double G[NC], dw[NC], o[NC];
+    double G[NC], dw[NC];
     if constexpr (FLUX == 1) {
+      double o[NC];
       IRNode<double, D> ik, ib;
       ir_node<double, D>(nk, ik);
       ir_node<double, D>(nb, ib);
@@ -497,16 +488,16 @@ __global__ void __launch_bounds__(128) face_bc_kernel(const double* __restrict__
       znode<double, D>(nk, c, zk);
       znode<double, D>(nb, c, zb);
       znode_recips<double, D>(zk);
-      PairAvg<double, D> av;
-      pair_avg<double, D>(zk, zb, c, av);
-      sy_flux_dir<double, D>(av, c, nuv, G);
+      PairSums<D> av;
+      pair_sums<D>(zk, zb, &nk.W[1], &nb.W[1], c, av);
+      sy_flux2<D>(av, nuv, G);
       if (dissipation) {
 #pragma unroll
         for (int q = 0; q < NC; ++q) dw[q] = nk.W[q] - nb.W[q];
-        diss_apply<double, D>(av, c, nh, dw, o);
-#pragma unroll
-        for (int q = 0; q < NC; ++q) G[q] += 0.5 * b * o[q];
+        diss_add2<D>(av, c, nh, dw, b, G);
       }
+#pragma unroll
+      for (int q = 0; q < NC; ++q) G[q] *= 0.5;
     }
     double ek[NC];
 #pragma unroll
@@ -705,7 +696,7 @@ __global__ void __launch_bounds__(round32(EB * NP), SplitCfg<D, NP, EB, VISC>::B
       if (sl >= 0) {
         const size_t S_ = (size_t)n_slot_total, ix = (size_t)e * NS + sl;
         fcache[0 * S_ + ix] = nd.rho;
-        fcache[1 * S_ + ix] = nd.ir;
+        fcache[1 * S_ + ix] = nd.W[0];
         fcache[2 * S_ + ix] = nd.p;
         fcache[3 * S_ + ix] = nd.e;
         fcache[4 * S_ + ix] = nd.q;
@@ -989,7 +980,7 @@ __global__ void __launch_bounds__(EB * NP, (sizeof(T) == 4 && !VISC && D == 2) ?
       if (sl0 >= 0) {
         const size_t S = (size_t)n_slot_total, ix = (size_t)e * NS + sl0;
         fcache[0 * S + ix] = nd.rho;
-        fcache[1 * S + ix] = nd.ir;
+        fcache[1 * S + ix] = nd.W[0];
         fcache[2 * S + ix] = nd.p;
         fcache[3 * S + ix] = nd.e;
         fcache[4 * S + ix] = nd.q;
@@ -1155,7 +1146,7 @@ __global__ void __launch_bounds__(EB * NP) hadamard_volume_kernel(
         if (fcache && sl0 >= 0) {
           const size_t S = (size_t)n_slot_total, ix = (size_t)e * NS + sl0;
           fcache[0 * S + ix] = nd.rho;
-          fcache[1 * S + ix] = nd.ir;
+          fcache[1 * S + ix] = nd.W[0];
           fcache[2 * S + ix] = nd.p;
           fcache[3 * S + ix] = nd.e;
           fcache[4 * S + ix] = nd.q;
@@ -1245,14 +1236,32 @@ __global__ void __launch_bounds__(EB * NP) hadamard_volume_kernel(
           zn.P1 = zz[(D + 2) * NP + n];
           zn.P2 = zz[(D + 3) * NP + n];
           zn.v2 = zz[(D + 4) * NP + n];
-          PairAvg<T, D> a;
-          pair_avg<T, D>(zm, zn, c, a);
-          sy_flux_dir<T, D>(a, c, Smn, G);
+          if constexpr (sizeof(T) == sizeof(double)) {
+            double qVm[D], qVn[D];
+#pragma unroll
+            for (int i = 0; i < D; ++i) {
+              qVm[i] = zm.q * zm.V[i];
+              qVn[i] = zn.q * zn.V[i];
+            }
+            PairSums<D> a;
+            pair_sums<D>(zm, zn, qVm, qVn, c64, a);
+            sy_flux2<D>(a, Smn, G);
+          } else {
+            PairAvg<T, D> a;
+            pair_avg<T, D>(zm, zn, c, a);
+            sy_flux_dir<T, D>(a, c, Smn, G);
+#pragma unroll
+            for (int q = 0; q < NC; ++q) G[q] *= T(2);
+          }
+        }
+        if constexpr (FLUX == 1) {
+#pragma unroll
+          for (int q = 0; q < NC; ++q) G[q] *= T(2);
         }
 #pragma unroll
-        for (int q = 0; q < NC; ++q) {
-          acc[q] -= T(2) * G[q] * iHm;
-          gout[(k - k0) * NC + q] = T(2) * G[q];
+        for (int q = 0; q < NC; ++q) {  // G: twice the two-point flux
+          acc[q] -= G[q] * iHm;
+          gout[(k - k0) * NC + q] = G[q];
         }
       }
     }

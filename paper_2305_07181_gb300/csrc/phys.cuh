@@ -40,6 +40,9 @@ struct Phys {
   // (imath.cuh); im_ok: all below 8 in size
   long long a60, b60, r160, r260;
   int im_ok;
+  // ser1, ser2: c_0 .. c_6 in units of 2^-62, c_7 .. c_12 in float32 (exp_avg_pair)
+  long long s1[7], s2[7];
+  float t1[6], t2[6];
 };
 
 template <typename T>
@@ -76,6 +79,7 @@ __host__ inline Phys<T> make_phys(double gam, double beta, double R, double mu, 
   c.b60 = (long long)(pw[1] * sc);
   c.r160 = (long long)(pw[2] * sc);
   c.r260 = (long long)(pw[3] * sc);
+  if (!(r1 > 0.0 && r1 < 1.0 && r2 > 0.0 && r2 < 1.0)) c.im_ok = 0;
   double a1 = 1.0, a2 = 1.0;
   for (int k = 0; k < 16; ++k) {
     if (k > 0) {
@@ -84,6 +88,14 @@ __host__ inline Phys<T> make_phys(double gam, double beta, double R, double mu, 
     }
     c.ser1[k] = (T)a1;
     c.ser2[k] = (T)a2;
+    if (k < 7) {  // |c_k| <= 1 for exponents in (0, 1); exp_avg_pair is not used otherwise
+      const double u62 = 4611686018427387904.0;
+      c.s1[k] = fabs(a1) <= 1.0 ? (long long)(a1 * u62) : 0;
+      c.s2[k] = fabs(a2) <= 1.0 ? (long long)(a2 * u62) : 0;
+    } else if (k < 13) {
+      c.t1[k - 7] = (float)a1;
+      c.t2[k - 7] = (float)a2;
+    }
   }
   return c;
 }
@@ -179,7 +191,7 @@ __device__ __forceinline__ double pow_from_log(double l, double r, long long r60
 template <typename T, int D, typename C>
 __device__ __forceinline__ bool node_from_u(const T* u, const C& c, Node<T, D>& n) {
   n.rho = u[0];
-  T ir = T(1) / n.rho;
+  T ir = t_rcp(n.rho);
   n.ir = ir;
   n.v2 = T(0);
 #pragma unroll
@@ -229,7 +241,7 @@ template <typename T, int D, typename C>
 __device__ __forceinline__ JvpPrep<T> jvp_prep(const Node<T, D>& n, const C& c) {
   JvpPrep<T> j;
   // one division for 1/q and rho/p: y = 1/(q p), 1/q = p y, 1/p = q y
-  const T y = T(1) / (n.q * n.p);
+  const T y = t_rcp(n.q * n.p);
   j.iq = n.p * y;
   j.ir = n.ir;
   j.theta = n.p * j.ir;
@@ -481,8 +493,8 @@ __device__ __forceinline__ void znode(const Node<T, D>& n, const C& c, ZNode<T, 
 // the reciprocals the exponential averages of a pair need (side k only)
 template <typename T, int D>
 __device__ __forceinline__ void znode_recips(ZNode<T, D>& z) {
-  z.iq = T(1) / z.q;
-  z.ip = T(1) / z.p;
+  z.iq = t_rcp(z.q);
+  z.ip = t_rcp(z.p);
 }
 
 // Pair averages shared by the Sjogreen-Yee flux (Eq. (48)) and the
@@ -522,7 +534,7 @@ __device__ __forceinline__ void pair_avg(const ZNode<T, D>& k, const ZNode<T, D>
 // sum_i nu_i F*_i(U_k, U_v) (Eq. (48)) for a direction vector nu.
 template <typename T, int D, typename C>
 __device__ __forceinline__ void sy_flux_dir(const PairAvg<T, D>& a, const C& c, const T* nu, T* F) {
-  T inv_den = T(1) / (a.A1 * a.E1);
+  T inv_den = t_rcp(a.A1 * a.E1);
   T mn = T(0);
 #pragma unroll
   for (int i = 0; i < D; ++i) mn += nu[i] * a.qV[i];
@@ -531,6 +543,150 @@ __device__ __forceinline__ void sy_flux_dir(const PairAvg<T, D>& a, const C& c, 
 #pragma unroll
   for (int j = 0; j < D; ++j) F[1 + j] = mn * a.Va[j] + nu[j] * a.pa;
   F[D + 1] = mn * (c.gam_gm1 * a.A2 * a.E2 + a.ke);
+}
+
+// 1/sqrt(x) by the cubic iteration r0 (1 + e/2 + 3 e^2/8), e = 1 - x r0^2,
+// from the hardware's 19-bit estimate (error before the last rounding < 2^-57)
+__device__ __forceinline__ double rsqrt64(double x) {
+  double r0;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(x));
+  const double e = fma(-(x * r0), r0, 1.0);
+  return fma(r0 * e, fma(e, 0.375, 0.5), r0);
+}
+
+// Exponential average of Eq. (47) as exp_avg, float64, the series in fixed
+// point: Horner's rule on 64-bit integers for c_0 .. c_6 and in float32 for
+// c_7 .. c_12 (below 2^-30 of the sum), ~110 integer instructions instead of
+// 12 float64 ones (which cost ~900 clocks of the pipe).
+__device__ __forceinline__ double exp_avg_pair(double a, double b, double ar, double br, double r, double ia,
+                                               const double* coef, const long long* s62, const float* tail, int ok) {
+  const double eps = (b - a) * ia;
+  const unsigned long long bits = (unsigned long long)__double_as_longlong(eps);
+  const int e = (int)(bits >> 52) & 0x7ff;
+  if (!fm::abs_below(eps, 0x3FA999999999999AULL)) return (ar - br) / (r * (a - b));  // 0.05
+  if (!ok) {
+    double sum = coef[ExpAvgCfg<double>::NTERMS - 1];
+#pragma unroll
+    for (int k = ExpAvgCfg<double>::NTERMS - 2; k >= 0; --k) sum = sum * eps + coef[k];
+    return ar * ia * sum;
+  }
+  // eps = M 2^(e - 1075) in units of 2^-66: e <= 1018, a shift of at most 9
+  const unsigned long long M = (bits & 0xFFFFFFFFFFFFFULL) | 0x10000000000000ULL;
+  const int sh = 1018 - e;
+  const unsigned long long mag = sh > 62 ? 0ULL : ((M << 9) >> sh);
+  const long long x = (bits >> 63) ? -(long long)mag : (long long)mag;
+  const float xf = __int2float_rn((int)(x >> 32)) * 0x1p-34f;
+  float t = tail[5];
+#pragma unroll
+  for (int k = 4; k >= 0; --k) t = t * xf + tail[k];
+  long long s = (long long)__float2int_rn(t * 0x1p30f) << 32;
+#pragma unroll
+  for (int k = 6; k >= 0; --k) s = s62[k] + (__mul64hi(s, x) >> 2);
+  // s is in (0.9, 1.1): two binades, the leading bit 61 or 62
+  const int lz = __clzll(s);
+  const unsigned long long n = (unsigned long long)s << lz;
+  const unsigned long long m = (n >> 11) + ((n >> 10) & 1ULL);
+  const double sum = __longlong_as_double((long long)(m + ((unsigned long long)(1023 - lz) << 52)));
+  return ar * ia * sum;
+}
+
+// Two-point quantities of a node pair in float64, as sums instead of means
+// (twice PairAvg's fields, the halves cancel in the flux and its doubled
+// result): the Sjogreen-Yee flux and the dissipation of Eqs. (48) and (69)
+// with the fewest float64 operations.
+//   dn = {P1}' E1 (= 2 A1 E1), idn = 1/dn, h2 = 2 [gam/(gam-1) A2 E2 + ke],
+//   ke = sum {V_j}^2 - {sum V_j^2}/2 = V_k . V_v / 2.
+template <int D>
+struct PairSums {
+  double dn, idn, E1, E2, Sq, Sp, SqV[D], SV[D], h2;
+};
+
+// qVk, qVv: q V of the two sides
+template <int D, typename C>
+__device__ __forceinline__ void pair_sums(const ZNode<double, D>& k, const ZNode<double, D>& v, const double* qVk,
+                                          const double* qVv, const C& c, PairSums<D>& a) {
+  a.E1 = exp_avg_pair(k.p, v.p, k.P2, v.P2, c.r2, k.ip, c.ser2, c.s2, c.t2, c.im_ok);
+  a.E2 = exp_avg_pair(k.q, v.q, k.P1, v.P1, c.r1, k.iq, c.ser1, c.s1, c.t1, c.im_ok);
+  a.dn = (k.P1 + v.P1) * a.E1;
+  a.idn = rcp64(a.dn);
+  a.Sq = k.q + v.q;
+  a.Sp = k.p + v.p;
+  a.h2 = c.gam_gm1 * (k.P2 + v.P2) * a.E2;
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    a.SqV[i] = qVk[i] + qVv[i];
+    a.SV[i] = k.V[i] + v.V[i];
+    a.h2 += k.V[i] * v.V[i];
+  }
+}
+
+// 2 sum_i nu_i F*_i(U_k, U_v) (Eq. (48)) for a direction vector nu
+template <int D>
+__device__ __forceinline__ void sy_flux2(const PairSums<D>& a, const double* nu, double* G2) {
+  double mn = 0.0;
+#pragma unroll
+  for (int i = 0; i < D; ++i) mn = i == 0 ? nu[0] * a.SqV[0] : mn + nu[i] * a.SqV[i];
+  mn *= a.idn;
+  G2[0] = mn + mn;
+#pragma unroll
+  for (int j = 0; j < D; ++j) G2[1 + j] = mn * a.SV[j] + nu[j] * a.Sp;
+  G2[D + 1] = mn * a.h2;
+}
+
+// out += b X^ |Lambda_n| S^ X^T dw (Eq. (69), unit normal n) at the
+// intermediate state: the terms of diss_apply with the two acoustic columns
+// taken together,
+//   y0 = (c_0 . dw) l_0, y-+ = (base -+ s) l-+,  base = dw_0 + V.dw_m + H dw_E,
+//   s = a (n.dw_m + vn dw_E),
+//   out = [y- + y+ + y0, V out_0 + a (y+ - y-) n, H (y- + y+) + vn a (y+ - y-) + |V|^2/2 y0]
+// plus the printed tangential columns.  theta/(2 gam) = idn / a^2 and
+// 1/(z1 E1 E2), 1/z1 come from one reciprocal, a and 1/a from one rsqrt.
+template <int D, typename C>
+__device__ __forceinline__ void diss_add2(const PairSums<D>& p, const C& c, const double* n, const double* dw,
+                                          double b, double* out) {
+  constexpr int NC = D + 2;
+  const double E12 = p.E1 * p.E2, y = rcp64(p.Sq * E12);
+  const double iSq = E12 * y, eta = 2.0 * y;
+  double V[D], vn = 0.0, h = 0.0, ndm = 0.0, base = dw[0];
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    V[i] = p.SqV[i] * iSq;
+    vn = i == 0 ? V[0] * n[0] : vn + V[i] * n[i];
+    h = i == 0 ? V[0] * V[0] : h + V[i] * V[i];
+    ndm = i == 0 ? n[0] * dw[1] : ndm + n[i] * dw[1 + i];
+    base += V[i] * dw[1 + i];
+  }
+  h *= 0.5;
+  const double x = (0.5 * c.gam) * p.Sp * p.dn * iSq;  // a^2 = gam p^ / rho^
+  const double ia = rsqrt64(x), ah = x * ia;
+  const double kac = b * p.idn * (ia * ia);            // b theta / (2 gam)
+  const double Hh = x * c.inv_gm1 + h, e = dw[NC - 1];
+  const double s = ah * (ndm + vn * e);
+  const double avn = fabs(vn);
+  const double y0 = (base + h * e) * (avn * (2.0 * c.gam * c.s_en) * kac);
+  base += Hh * e;
+  const double ym = (base - s) * (fabs(vn - ah) * kac), yp = (base + s) * (fabs(vn + ah) * kac);
+  const double sp = ym + yp, sd = ah * (yp - ym), o0 = sp + y0;
+  out[0] += o0;
+  double oE = Hh * sp + (h * y0 + vn * sd);
+#pragma unroll
+  for (int i = 0; i < D; ++i) out[1 + i] += V[i] * o0 + sd * n[i];
+  if constexpr (D >= 2) {  // (0, n2, -n1, 0, V1 n2 - V2 n1)
+    const double l = avn * eta * b;
+    const double c2 = V[0] * n[1] - V[1] * n[0];
+    const double t = (n[1] * dw[1] - n[0] * dw[2] + c2 * e) * l;
+    out[1] += n[1] * t;
+    out[2] -= n[0] * t;
+    oE += c2 * t;
+    if constexpr (D == 3) {  // (0, -n3, 0, n1, V3 n1 - V1 n3)
+      const double c3 = V[2] * n[0] - V[0] * n[2];
+      const double t3 = (n[0] * dw[3] - n[2] * dw[1] + c3 * e) * l;
+      out[1] -= n[2] * t3;
+      out[3] += n[0] * t3;
+      oE += c3 * t3;
+    }
+  }
+  out[NC - 1] += oE;
 }
 
 // X^ |Lambda_n| S^ X^T dw of Eq. (69) at the intermediate state (Eqs.
@@ -678,7 +834,7 @@ template <typename T, int D, typename C>
 __device__ __forceinline__ void ir_avg(const IRNode<T, D>& k, const IRNode<T, D>& v, const C& c, IRAvg<T, D>& a) {
   T a1 = T(0.5) * (k.z1 + v.z1), an = T(0.5) * (k.zn + v.zn);
   T L1 = log_mean<T>(k.z1, v.z1, k.l1, v.l1), Ln = log_mean<T>(k.zn, v.zn, k.ln, v.ln);
-  T ia1 = T(1) / a1;
+  T ia1 = t_rcp(a1);
   a.vv = T(0);
 #pragma unroll
   for (int i = 0; i < D; ++i) {
