@@ -39,14 +39,11 @@ extern "C" {
 #define ESPLIT_ERR_STATE (-7)        /* call order (e.g. residual before mesh upload) */
 
 #define ESPLIT_FP64 0       /* everything in float64                               */
-#define ESPLIT_FP32_BULK 1  /* entropy-split volume term: operator contractions as
-                               compensated float32 dot products (Dot2) on the
-                               variations inside each element, fluxes, entropy
-                               variables and A~_i products in float64 (accuracy of
-                               the float64 path to ~1e-12); facet terms, viscous
-                               terms, entropy functionals and the relaxation root
-                               solve in float64.  Hadamard forms: their two-point
-                               fluxes in plain float32                              */
+#define ESPLIT_FP32_BULK 1  /* entropy-split terms: as ESPLIT_FP64 (the contractions
+                               are exact digit products on the tensor cores, faster
+                               than compensated float32 sums).  Hadamard forms: their
+                               two-point fluxes in plain float32                     */
+
 #define ESPLIT_FP32 2       /* entropy-split scheme, inviscid, lines and
                                triangles: fluxes, entropy
                                variables, A~_i products, two-point fluxes,
@@ -191,8 +188,7 @@ int esplit_upload_mesh(esplit_ctx* ctx, int n_e, const double* J, const double* 
  * ESPLIT_ERR_UNSUPPORTED. */
 int esplit_set_boundary_states(esplit_ctx* ctx, int n_b, const int* slots, const double* states);
 
-/* Parameters (host struct, copied).  Changing beta re-forms the stored
- * split operators. */
+/* Parameters (host struct, copied). */
 int esplit_set_params(esplit_ctx* ctx, const esplit_params* params);
 int esplit_get_params(esplit_ctx* ctx, esplit_params* params);
 

@@ -100,8 +100,6 @@ int rebuild_ops(esplit_ctx* c, cudaStream_t s) {
   if (!c->have_op || !c->have_mesh) return ESPLIT_OK;
   if (esplit::launch_build_ops(c, s)) return fail(c, ESPLIT_ERR_CUDA, "build_ops launch failed");
   CK(cudaStreamSynchronize(s));
-  c->ops_beta = c->prm.beta;
-  c->ops_beta_valid = true;
   return ESPLIT_OK;
 }
 
@@ -188,8 +186,8 @@ void esplit_destroy(esplit_ctx* c) {
   if (!c) return;
   cudaSetDevice(c->device);
   esplit::Buffers& b = c->b;
-  void* ps[] = {b.Qref, b.J,       b.nu,      b.pair,   b.Lam,     b.face_pairs, b.ops64,   b.ops32,   b.ops32lo,
-                b.list_split, b.list_had, b.hflags, b.hflag0, b.hcount, b.sat, b.fcache, b.rows, b.partial, b.scal, b.root, b.status, b.stage_u,
+  void* ps[] = {b.Qref, b.J,       b.nu,      b.pair,   b.Lam,     b.face_pairs, b.ops64,   b.ops32,
+                b.list_split, b.list_had, b.hflags, b.hflag0, b.hcount, b.sat, b.fcache, b.partial, b.scal, b.root, b.status, b.stage_u,
                 b.stage_r, b.dacc, b.node_cache, b.vjp_work, b.host_u, b.host_r, b.fv, b.vsat, b.va, b.wslot, b.vfb, b.vfs, b.vus,
                 b.bslot, b.bstate, b.ihf, b.opsD32, b.ihd, b.nscale, b.opsP, b.opsE};
   for (void* p : ps) dfree(p);
@@ -319,10 +317,8 @@ int esplit_upload_mesh(esplit_ctx* c, int n_e, const double* J, const double* La
   if ((rc = dalloc(c, &c->b.pair, (size_t)n_e * NS * 2))) return rc;
   if ((rc = dalloc(c, &c->b.Lam, (size_t)n_e * d * d * NP))) return rc;
   if ((rc = dalloc(c, &c->b.face_pairs, fpairs.size()))) return rc;
-  if ((rc = dalloc(c, &c->b.ops64, (size_t)n_e * 2 * d * NP * NP))) return rc;
-  if ((rc = dalloc(c, &c->b.ops32, (size_t)n_e * 2 * d * NP * NP))) return rc;
-  if ((rc = dalloc(c, &c->b.ops32lo, (size_t)n_e * 2 * d * NP * NP))) return rc;
-  if ((rc = dalloc(c, &c->b.rows, (size_t)n_e * 2 * d * NP))) return rc;
+  if ((rc = dalloc(c, &c->b.ops64, (size_t)n_e * d * NP * NP))) return rc;
+  if ((rc = dalloc(c, &c->b.ops32, (size_t)n_e * d * NP * NP))) return rc;
   if ((rc = dalloc(c, &c->b.sat, (size_t)n_e * c->n_c * NS))) return rc;
   if ((rc = dalloc(c, &c->b.fcache, (size_t)(d + 9) * n_e * NS))) return rc;
   if ((rc = dalloc(c, &c->b.ihf, (size_t)n_e * NP))) return rc;
@@ -394,13 +390,11 @@ int esplit_set_params(esplit_ctx* c, const esplit_params* p) {
     return fail(c, ESPLIT_ERR_ARG, "unknown precision");
   if (p->viscous && c->dim == 1) return fail(c, ESPLIT_ERR_UNSUPPORTED, "1D: inviscid only");
   cudaSetDevice(c->device);
-  bool beta_changed = p->beta != c->prm.beta;
   c->prm = *p;
   if (p->viscous) {
     int rcv = ensure_viscous(c);
     if (rcv) return rcv;
   }
-  if (beta_changed && c->have_mesh) return rebuild_ops(c, 0);
   return ESPLIT_OK;
 }
 

@@ -47,17 +47,13 @@ struct Buffers {
   int* pair = nullptr;         // [n_e][n_slot][2]
   double* Lam = nullptr;       // [n_e][d][d][n_p]
   int2* face_pairs = nullptr;  // [n_pairs] (k*n_slot+s, v*n_slot+s') with owner k
-  // per-element split/derivative operators, transposed ([k][n][m]):
-  //   k <  d: M_i^T, M_i = H^-1 (Q_x_i/(beta+1) + Q_x_i^T)
-  //   k >= d: D_i^T, D_i = H^-1 Q_x_i
-  double* ops64 = nullptr;     // [n_e][2d][n_p][n_p]
+  // per-element derivative operators D_i = H^-1 Q_x_i, transposed ([i][n][m])
+  double* ops64 = nullptr;     // [n_e][d][n_p][n_p]
   // D_i as 60-bit fixed point, two entries per uint4, and the rows' exponents
   // (tc64.cuh; triangles and tetrahedra)
   uint4* opsP = nullptr;       // [n_e][d][n_p][ceil(n_p / 2)]
   short* opsE = nullptr;       // [n_e][d][n_p]
-  float* ops32 = nullptr;      // same, float (nearest)
-  float* ops32lo = nullptr;    // same, float remainder ops64 - ops32 (compensated FP32-bulk contractions)
-  double* rows = nullptr;      // [n_e][2d][n_p] row sums of the ops64 matrices
+  float* ops32 = nullptr;      // [n_e][d][n_p][n_p] ops64 rounded to float32
   float* ihf = nullptr;        // [n_e][n_p] 1/(H_ref J), float32 (the float32 path's facet scaling)
   double* ihd = nullptr;       // [n_e][n_p] 1/(H_ref J) (the float64 facet kernels' scaling)
   double* nscale = nullptr;    // [n_e][n_slot][d + 1] |nu|, nu/|nu| of every facet slot
@@ -135,8 +131,7 @@ struct esplit_ctx {
   int opsD_stride = 0;             // floats per element in b.opsD32
   bool have_bstate = false;        // their exterior states are set
   std::vector<int> bslots;         // flat slot indices (element * n_slot + slot), ascending
-  bool have_op = false, have_mesh = false, ops_beta_valid = false;
-  double ops_beta = 0.0;
+  bool have_op = false, have_mesh = false;
   esplit_params prm{};
   esplit::RefTables ref{};
   esplit::Buffers b;

@@ -7,9 +7,8 @@
 //   nu            [n_e][n_slot][d]     scaled outward normals at facet slots
 //   face_pairs    int2 [n_pairs]       (k*n_slot+s, v*n_slot+s'), one per
 //                                      coincident facet-node pair
-//   ops64/ops32   [n_e][2d][n_p][n_p]  per-element operators, transposed:
-//                 k < d: M_i^T with M_i = H^-1 (Q_x_i/(beta+1) + Q_x_i^T)
-//                 k >= d: D_i^T with D_i = H^-1 Q_x_i
+//   ops64/ops32   [n_e][d][n_p][n_p]   per-element operators D_i = H^-1 Q_x_i,
+//                 transposed; opsP/opsE the same in fixed point (tc64.cuh)
 //   sat           [n_e][n_c][n_slot]   facet (SAT + dissipation) contributions
 #include <cuda_runtime.h>
 #include <math_constants.h>
@@ -23,7 +22,6 @@
 #include "phys.cuh"
 #include "visc_flux.cuh"
 #include "reduce.cuh"
-#include "bits32.cuh"
 #include "tc64.cuh"
 
 namespace esplit {
@@ -36,64 +34,38 @@ int set_ref_tables(const RefTables& t) {
 }
 
 // ---------------------------------------------------------------------------
-// per-element operators (run once per mesh upload / beta change)
+// per-element operators (run once per mesh upload)
 // Q_x_i = 1/2 sum_j (Lam_ij Q_xi_j - Q_xi_j^T Lam_ij) + 1/2 E_x_i
 // ---------------------------------------------------------------------------
 template <int D>
 __global__ void build_ops_kernel(const double* __restrict__ Qref, const double* __restrict__ Lam,
                                  const double* __restrict__ J, const double* __restrict__ nu, int n_e,
-                                 double inv_bp1, double* __restrict__ ops64, float* __restrict__ ops32,
-                                 float* __restrict__ ops32lo) {
+                                 double* __restrict__ ops64, float* __restrict__ ops32) {
   const int NP = c_ref.n_p, NS = c_ref.n_slot;
-  size_t per = (size_t)2 * D * NP * NP;
+  size_t per = (size_t)D * NP * NP;
   size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= per * (size_t)n_e) return;
   int e = (int)(idx / per);
   int rem = (int)(idx - (size_t)e * per);
-  int k = rem / (NP * NP);
-  int nm = rem - k * NP * NP;
-  int n = nm / NP, m = nm - n * NP;  // stored entry (k, n, m) = matrix[m][n]
-  int i = k % D;
-  auto Qx = [&](int a, int b) -> double {
-    double s = 0.0;
-    for (int j = 0; j < D; ++j) {
-      const double* L = Lam + (((size_t)e * D + i) * D + j) * NP;
-      s += L[a] * Qref[((size_t)j * NP + a) * NP + b] - Qref[((size_t)j * NP + b) * NP + a] * L[b];
-    }
-    s *= 0.5;
-    if (a == b) {
-      int sl = c_ref.node_slot[a];
-      if (sl >= 0) s += 0.5 * nu[((size_t)e * NS + sl) * D + i];
-    }
-    return s;
-  };
-  double Hm = c_ref.H[m] * J[(size_t)e * NP + m];
-  double val;
-  if (k < D)
-    val = (Qx(m, n) * inv_bp1 + Qx(n, m)) / Hm;
-  else
-    val = Qx(m, n) / Hm;
-  ops64[idx] = val;
-  float hi = (float)val;
-  ops32[idx] = hi;
-  ops32lo[idx] = (float)(val - (double)hi);
-}
-
-// row sums M_i 1 and D_i 1 of the stored float64 operators, summed in node
-// order: rows[e][k][m] = sum_n ops64[e][k][n][m]
-__global__ void build_rows_kernel(const double* __restrict__ ops64, int n_e, int two_d, double* __restrict__ rows) {
-  const int NP = c_ref.n_p;
-  size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (size_t)n_e * two_d * NP) return;
-  size_t ek = idx / NP;
-  int m = (int)(idx - ek * NP);
-  const double* op = ops64 + ek * NP * NP;
+  int i = rem / (NP * NP);
+  int nm = rem - i * NP * NP;
+  int n = nm / NP, m = nm - n * NP;  // stored entry (i, n, m) = D_i[m][n]
   double s = 0.0;
-  for (int n = 0; n < NP; ++n) s += op[(size_t)n * NP + m];
-  rows[idx] = s;
+  for (int j = 0; j < D; ++j) {
+    const double* L = Lam + (((size_t)e * D + i) * D + j) * NP;
+    s += L[m] * Qref[((size_t)j * NP + m) * NP + n] - Qref[((size_t)j * NP + n) * NP + m] * L[n];
+  }
+  s *= 0.5;
+  if (m == n) {
+    int sl = c_ref.node_slot[m];
+    if (sl >= 0) s += 0.5 * nu[((size_t)e * NS + sl) * D + i];
+  }
+  const double val = s / (c_ref.H[m] * J[(size_t)e * NP + m]);
+  ops64[idx] = val;
+  ops32[idx] = (float)val;
 }
 
-// opsD32[e][i][m][n] = D_i[m][n] (ops32 holds it at [e][d + i][n][m]) for
+// opsD32[e][i][m][n] = D_i[m][n] (ops32 holds it at [e][i][n][m]) for
 // n < n_p, zero in the row padding up to npp and after the d n_p npp entries
 __global__ void build_opsD_kernel(const float* __restrict__ ops32, int n_e, int d, int np, int npp, int stride,
                                   float* __restrict__ opsD) {
@@ -105,7 +77,7 @@ __global__ void build_opsD_kernel(const float* __restrict__ ops32, int n_e, int 
   if (j < d * np * npp) {
     const int i = j / (np * npp), rem = j - i * np * npp;
     const int m = rem / npp, n = rem - m * npp;
-    if (n < np) v = ops32[(((e * 2 * d) + d + i) * np + n) * np + m];
+    if (n < np) v = ops32[((e * d + i) * np + n) * np + m];
   }
   opsD[idx] = v;
 }
@@ -134,22 +106,16 @@ __global__ void facet_tables_kernel(const double* __restrict__ J, const double* 
 }
 
 int launch_build_ops(esplit_ctx* c, cudaStream_t s) {
-  size_t total = (size_t)c->n_e * 2 * c->dim * c->n_p * c->n_p;
+  size_t total = (size_t)c->n_e * c->dim * c->n_p * c->n_p;
   int bs = 256;
   unsigned nb = (unsigned)((total + bs - 1) / bs);
-  double inv_bp1 = 1.0 / (c->prm.beta + 1.0);
   if (c->dim == 1)
-    build_ops_kernel<1><<<nb, bs, 0, s>>>(c->b.Qref, c->b.Lam, c->b.J, c->b.nu, c->n_e, inv_bp1, c->b.ops64,
-                                          c->b.ops32, c->b.ops32lo);
+    build_ops_kernel<1><<<nb, bs, 0, s>>>(c->b.Qref, c->b.Lam, c->b.J, c->b.nu, c->n_e, c->b.ops64, c->b.ops32);
   else if (c->dim == 2)
-    build_ops_kernel<2><<<nb, bs, 0, s>>>(c->b.Qref, c->b.Lam, c->b.J, c->b.nu, c->n_e, inv_bp1, c->b.ops64,
-                                          c->b.ops32, c->b.ops32lo);
+    build_ops_kernel<2><<<nb, bs, 0, s>>>(c->b.Qref, c->b.Lam, c->b.J, c->b.nu, c->n_e, c->b.ops64, c->b.ops32);
   else
-    build_ops_kernel<3><<<nb, bs, 0, s>>>(c->b.Qref, c->b.Lam, c->b.J, c->b.nu, c->n_e, inv_bp1, c->b.ops64,
-                                          c->b.ops32, c->b.ops32lo);
-  size_t nr = (size_t)c->n_e * 2 * c->dim * c->n_p;
-  build_rows_kernel<<<(unsigned)((nr + 255) / 256), 256, 0, s>>>(c->b.ops64, c->n_e, 2 * c->dim, c->b.rows);
-  c->launches += 2;
+    build_ops_kernel<3><<<nb, bs, 0, s>>>(c->b.Qref, c->b.Lam, c->b.J, c->b.nu, c->n_e, c->b.ops64, c->b.ops32);
+  c->launches++;
   if (c->b.opsP) {
     const size_t nr2 = (size_t)c->n_e * c->dim * c->n_p;
     const unsigned nb2 = (unsigned)((nr2 + 255) / 256);
@@ -562,7 +528,9 @@ int launch_face_bc(esplit_ctx* c, const double* u, double* out, int add, double*
 // Pointwise work in float64, one node per thread.  Triangles and tetrahedra:
 // the contractions on the tensor cores (tc64.cuh: exact digit products, one
 // rounding; as accurate as a float64 sum or better), so the float64 pipe has
-// only the nodal state, fluxes and A~_i products left.  Lines and 7-node
+// only the nodal state, fluxes and A~_i products left (the FP32-bulk setting
+// takes this kernel too: compensated float32 contractions measured slower,
+// 97 against 78 us on 18,432 triangles p 2).  Lines and 7-node
 // triangles: float64 FMA loops, too short for the tiles.
 // Optional: block partial of sum H w^T r (entropy production, float64).
 // ---------------------------------------------------------------------------
@@ -652,7 +620,7 @@ __global__ void __launch_bounds__(round32(EB * NP), SplitCfg<D, NP, EB, VISC>::B
       for (int q = 0; q < S::COLS; ++q) sv[(el * S::COLS + q) * NP + m] = vals[q];
     }
     __syncthreads();
-    const double* op = ops64 + (size_t)e * (2 * D * NP * NP);
+    const double* op = ops64 + (size_t)e * (D * NP * NP);
 #pragma unroll
     for (int q = 0; q < NC; ++q) accd[q] = 0.0;
 #pragma unroll
@@ -664,7 +632,7 @@ __global__ void __launch_bounds__(round32(EB * NP), SplitCfg<D, NP, EB, VISC>::B
       for (int i = 0; i < D; ++i)
 #pragma unroll
         for (int n = 0; n < NP; ++n) {
-          const double dt = __ldg(&op[((D + i) * NP + n) * NP + m]);
+          const double dt = __ldg(&op[(i * NP + n) * NP + m]);
 #pragma unroll
           for (int q = 0; q < NC; ++q) {
             accd[q] += dt * sv[(el * S::COLS + i * NC + q) * NP + n];
@@ -795,303 +763,6 @@ __global__ void __launch_bounds__(round32(EB * NP), SplitCfg<D, NP, EB, VISC>::B
 }
 
 // ---------------------------------------------------------------------------
-// entropy-split volume kernel of the FP32-bulk setting: the terms of
-// split_volume_kernel with the contractions in float32 on the variation
-// inside the element, relative to its node 0; the node-0 values come back
-// through the float64 row sums of the stored operators,
-//   D_i f_i = D_i (f_i - f_i,0) + f_i,0 (D_i 1),  D_i w = D_i (w - w_0) + w_0 (D_i 1).
-// Operator entries and variations are each held as an unevaluated float32
-// sum hi + lo, and the products are accumulated by the compensated dot
-// product of Ogita, Rump and Oishi (Dot2, SIAM J. Sci. Comput. 26, 2005):
-// the rounding error of every product (exact through fmaf) and of every
-// addition (TwoSum) goes to a second float32 accumulator, together with the
-// cross terms hi*lo.  At low Mach number the energy-flux variation inside an
-// element is ~(E + p)|dV|, hundreds of times the residual, and a plain
-// float32 product would lose that factor.  Pointwise work in float64.
-// ---------------------------------------------------------------------------
-template <typename T, int D, int NP, int EB>
-struct SplitSmem {
-  double rf[EB][D][D + 2][NP];  // fluxes
-  double rw[EB][D + 2][NP];     // entropy variables
-  T sf[EB][D][D + 2][NP];       // float32 variations, hi and lo parts (FP32-bulk only)
-  T sw[EB][D + 2][NP];
-  T sfl[EB][D][D + 2][NP];
-  T swl[EB][D + 2][NP];
-};
-
-// acc + cmp += (ah + al) (bh + bl), Dot2 step: exact product error by fmaf,
-// TwoSum for the addition; intrinsics keep the compiler from fusing them.
-__device__ __forceinline__ void dot2_step(float ah, float al, float bh, float bl, float& acc, float& cmp) {
-  float p = __fmul_rn(ah, bh);
-  float e = __fmaf_rn(ah, bh, -p);
-  e = __fmaf_rn(ah, bl, e);
-  e = __fmaf_rn(al, bh, e);
-  float s = __fadd_rn(acc, p);
-  float z = __fsub_rn(s, acc);
-  float t = __fadd_rn(__fsub_rn(acc, __fsub_rn(s, z)), __fsub_rn(p, z));
-  acc = s;
-  cmp = __fadd_rn(cmp, __fadd_rn(t, e));
-}
-
-template <typename T, int D, int NP, int EB, bool VISC, bool CACHE = false, bool ENT = false>
-__global__ void __launch_bounds__(EB * NP, (sizeof(T) == 4 && !VISC && D == 2) ? 4 : ((VISC && D == 3) ? 2 : 1)) split_bulk_kernel(
-    const double* __restrict__ u, double* __restrict__ r, const T* __restrict__ ops,
-    const float* __restrict__ opslo, const double* __restrict__ rows, const double* __restrict__ J,
-    const double* __restrict__ sat, const int* __restrict__ list, int n_list, Phys<T> c, Phys<double> c64,
-    int* __restrict__ status, double* __restrict__ prod, int visc_heat, const double* __restrict__ nu,
-    const double* __restrict__ ah, double* __restrict__ fvs, const double* __restrict__ ops64,
-    double* __restrict__ fcache, int n_slot_total, double* __restrict__ ent_part = nullptr,
-    double* __restrict__ ncache = nullptr, double* __restrict__ wsl = nullptr) {
-  constexpr int NC = D + 2;
-  constexpr bool F64 = sizeof(T) == sizeof(double);
-  __shared__ SplitSmem<T, D, NP, EB> sm;
-  const int NS = c_ref.n_slot;
-  int el = threadIdx.x / NP;
-  int m = threadIdx.x - el * NP;
-  int li = blockIdx.x * EB + el;
-  bool active = (el < EB) && (li < n_list);
-  int e = active ? (list ? list[li] : li) : 0;
-  Node<double, D> nd;
-  if (active) {
-    double uu[NC];
-#pragma unroll
-    for (int q = 0; q < NC; ++q) uu[q] = __ldg(&u[((size_t)e * NC + q) * NP + m]);
-    if (!node_from_u<double, D>(uu, c64, nd)) atomicOr(status, 1);
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-      double F[NC];
-      euler_flux<double, D>(nd, i, F);
-#pragma unroll
-      for (int q = 0; q < NC; ++q) sm.rf[el][i][q][m] = F[q];
-    }
-#pragma unroll
-    for (int q = 0; q < NC; ++q) sm.rw[el][q][m] = nd.W[q];
-  }
-  __syncthreads();
-  if constexpr (!F64) {
-    if (active) {
-#pragma unroll
-      for (int i = 0; i < D; ++i)
-#pragma unroll
-        for (int q = 0; q < NC; ++q) {
-          float hi, lo;
-          split_f64(sm.rf[el][i][q][m] - sm.rf[el][i][q][0], hi, lo);
-          sm.sf[el][i][q][m] = hi;
-          sm.sfl[el][i][q][m] = lo;
-        }
-#pragma unroll
-      for (int q = 0; q < NC; ++q) {
-        float hi, lo;
-        split_f64(sm.rw[el][q][m] - sm.rw[el][q][0], hi, lo);
-        sm.sw[el][q][m] = hi;
-        sm.swl[el][q][m] = lo;
-      }
-    }
-    __syncthreads();
-  }
-  double hw = 0.0, ent_s = 0.0, ent_a = 0.0;
-  const int sl = c_ref.node_slot[m];
-  const T* op = ops + (size_t)e * (2 * D * NP * NP);
-  const double* op64 = VISC ? ops64 + (size_t)e * (2 * D * NP * NP) : nullptr;
-  double res[NC], Fp[D][NC], Hm = 0.0;
-  if (active) {
-    T acc[NC], g[D][NC];
-#pragma unroll
-    for (int q = 0; q < NC; ++q) acc[q] = T(0);
-#pragma unroll
-    for (int i = 0; i < D; ++i)
-#pragma unroll
-      for (int q = 0; q < NC; ++q) g[i][q] = T(0);
-    const float* oplo = F64 ? nullptr : opslo + (size_t)e * (2 * D * NP * NP);
-    // float32 sums: second accumulators of the compensated dot products
-    T cacc[NC], cg[D][NC];
-#pragma unroll
-    for (int q = 0; q < NC; ++q) cacc[q] = T(0);
-#pragma unroll
-    for (int i = 0; i < D; ++i)
-#pragma unroll
-      for (int q = 0; q < NC; ++q) cg[i][q] = T(0);
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-#pragma unroll 4
-      for (int n = 0; n < NP; ++n) {
-        T dt = __ldg(&op[((D + i) * NP + n) * NP + m]);
-        float dtl = 0.f;
-        if constexpr (!F64) dtl = __ldg(&oplo[((D + i) * NP + n) * NP + m]);
-#pragma unroll
-        for (int q = 0; q < NC; ++q) {
-          if constexpr (F64) {
-            acc[q] += dt * sm.rf[el][i][q][n];
-            g[i][q] += dt * sm.rw[el][q][n];
-          } else {
-            dot2_step(dt, dtl, sm.sf[el][i][q][n], sm.sfl[el][i][q][n], acc[q], cacc[q]);
-            dot2_step(dt, dtl, sm.sw[el][q][n], sm.swl[el][q][n], g[i][q], cg[i][q]);
-          }
-        }
-      }
-    }
-    double accd[NC], gd[D][NC];
-#pragma unroll
-    for (int q = 0; q < NC; ++q) {
-      if constexpr (F64)
-        accd[q] = acc[q];
-      else
-        accd[q] = widen_f32(acc[q]) + widen_f32(cacc[q]);
-    }
-#pragma unroll
-    for (int i = 0; i < D; ++i)
-#pragma unroll
-      for (int q = 0; q < NC; ++q) {
-        if constexpr (F64)
-          gd[i][q] = g[i][q];
-        else
-          gd[i][q] = widen_f32(g[i][q]) + widen_f32(cg[i][q]);
-      }
-    if constexpr (!F64) {
-      // add back the node-0 values through the stored operators' row sums
-      const double* rs = rows + (size_t)e * (2 * D * NP);
-#pragma unroll
-      for (int i = 0; i < D; ++i) {
-        double rd = __ldg(&rs[(D + i) * NP + m]);
-#pragma unroll
-        for (int q = 0; q < NC; ++q) {
-          accd[q] += sm.rf[el][i][q][0] * rd;  // node-0 values, re-read (fewer live registers)
-          gd[i][q] += sm.rw[el][q][0] * rd;
-        }
-      }
-    }
-    const JvpPrep<double> jp = jvp_prep<double, D>(nd, c64);
-    if constexpr (ENT) {
-      // entropy of u_n for the relaxation step (the entropy kernel's outputs):
-      // S_H = beta q p, and the per-node values its evaluation passes reuse
-      const size_t nn = (size_t)n_list * NP, g = (size_t)e * NP + m;
-      const double sH = c64.beta * nd.q * nd.p;
-      ncache[g] = sH;
-      ncache[nn + g] = nd.ir;
-      ncache[2 * nn + g] = jp.itheta * nd.ir;  // 1/p
-      const double Hm0 = c_ref.H[m] * __ldg(&J[(size_t)e * NP + m]);
-      ent_s = Hm0 * sH;
-      ent_a = Hm0 * fabs(sH);
-    }
-    if constexpr (CACHE) {
-      // nodal quantities of the facet nodes for the facet kernel that runs after
-      // this one (it then needs no logarithm, exponential or division for them)
-      const int sl0 = c_ref.node_slot[m];
-      if (sl0 >= 0) {
-        const size_t S = (size_t)n_slot_total, ix = (size_t)e * NS + sl0;
-        fcache[0 * S + ix] = nd.rho;
-        fcache[1 * S + ix] = nd.W[0];
-        fcache[2 * S + ix] = nd.p;
-        fcache[3 * S + ix] = nd.e;
-        fcache[4 * S + ix] = nd.q;
-        fcache[5 * S + ix] = nd.lnq;
-        fcache[6 * S + ix] = nd.lnp;
-        fcache[7 * S + ix] = jp.iq;
-        fcache[8 * S + ix] = jp.itheta * nd.ir;  // 1/p
-#pragma unroll
-        for (int i = 0; i < D; ++i) fcache[(9 + i) * S + ix] = nd.V[i];
-      }
-    }
-    double nonc[NC];
-#pragma unroll
-    for (int q = 0; q < NC; ++q) nonc[q] = 0.0;
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-      double dF[NC];
-      dflux_dw<double, D>(nd, jp, c64, i, gd[i], dF);
-#pragma unroll
-      for (int q = 0; q < NC; ++q) nonc[q] += dF[q];
-    }
-    Hm = c_ref.H[m] * __ldg(&J[(size_t)e * NP + m]);
-    const double kf = c64.beta * c64.inv_bp1;
-#pragma unroll
-    for (int q = 0; q < NC; ++q) {
-      // the facet contributions include H^-1 sum_i E_i f_i (added by the facet kernel)
-      res[q] = -kf * accd[q] - c64.inv_bp1 * nonc[q];
-      if (!CACHE && sl >= 0) res[q] += __ldg(&sat[((size_t)e * NC + q) * NS + sl]);
-    }
-    if constexpr (VISC) {
-      {
-        // viscous flux from the gradients just formed (gd = D_i w), plus the
-        // folded BO lift a/(2H) at the facet nodes; F^V kept for the flux jump
-        visc_flux<double, D>(nd, c64, visc_heat, gd, Fp);
-        if (sl >= 0 && wsl) {
-          // entropy variables at the facet slot, for the flux-jump kernel's
-          // share of the entropy production
-#pragma unroll
-          for (int q = 0; q < NC; ++q) wsl[((size_t)e * NC + q) * NS + sl] = nd.W[q];
-        }
-        if (sl >= 0) {
-#pragma unroll
-          for (int i = 0; i < D; ++i)
-#pragma unroll
-            for (int q = 0; q < NC; ++q) {
-              size_t ix = (((size_t)e * D + i) * NC + q) * NS + sl;
-              fvs[ix] = Fp[i][q];
-              Fp[i][q] += 0.5 * __ldg(&ah[ix]);
-            }
-        }
-      }
-    }
-  }
-  if constexpr (VISC) {  // float64 in both precision modes
-    {
-      __syncthreads();      // every thread is done with the fluxes in sm.rf
-      if (active) {
-#pragma unroll
-        for (int i = 0; i < D; ++i)
-#pragma unroll
-          for (int q = 0; q < NC; ++q) sm.rf[el][i][q][m] = Fp[i][q];
-      }
-      __syncthreads();
-      if (active) {
-        // sum_i D_i (F^V_i + a_i/(2H)) - sum_i nu_i a_i/(2H^2) at the facet nodes
-#pragma unroll
-        for (int i = 0; i < D; ++i) {
-#pragma unroll 4
-          for (int n = 0; n < NP; ++n) {
-            double dt = __ldg(&op64[((D + i) * NP + n) * NP + m]);
-#pragma unroll
-            for (int q = 0; q < NC; ++q) res[q] += dt * sm.rf[el][i][q][n];
-          }
-        }
-        if (sl >= 0) {
-          const double ih = 1.0 / Hm;
-          double nv[D];
-#pragma unroll
-          for (int i = 0; i < D; ++i) nv[i] = __ldg(&nu[((size_t)e * NS + sl) * D + i]);
-#pragma unroll
-          for (int q = 0; q < NC; ++q) {
-            double corr = 0.0;
-#pragma unroll
-            for (int i = 0; i < D; ++i) corr += nv[i] * __ldg(&ah[(((size_t)e * D + i) * NC + q) * NS + sl]);
-            res[q] -= 0.5 * corr * ih;
-          }
-        }
-      }
-    }
-  }
-  if (active) {
-#pragma unroll
-    for (int q = 0; q < NC; ++q) r[((size_t)e * NC + q) * NP + m] = res[q];
-    if (prod) {
-#pragma unroll
-      for (int q = 0; q < NC; ++q) hw += nd.W[q] * res[q];
-      hw *= Hm;
-    }
-  }
-  if (prod) {
-    double v[1] = {hw};
-    block_sum_t<1, round32(EB * NP)>(v, prod + blockIdx.x);
-  }
-  if constexpr (ENT) {
-    __syncthreads();  // the block sum's shared scratch is reused
-    double v2[2] = {ent_s, ent_a};
-    block_sum_t<2, round32(EB * NP)>(v2, ent_part + 2 * blockIdx.x);
-  }
-}
-
-// ---------------------------------------------------------------------------
 // Hadamard-form volume kernel (Eq. (99)), Sjogreen-Yee flux, each unordered
 // node pair evaluated once: thread m takes pairs (m, m+k mod NP),
 // k = 1..NP/2 (k = NP/2 only for m < NP/2 when NP is even), and hands the
@@ -1200,7 +871,7 @@ __global__ void __launch_bounds__(EB * NP) hadamard_volume_kernel(
     iHm = sH[el * NP + m];
     Hm = T(1) / iHm;
   }
-  const T* op = ops + (size_t)e * (2 * D * NP * NP);
+  const T* op = ops + (size_t)e * (D * NP * NP);
   T* gout = sg + ((size_t)el * NP + m) * KC * NC;
   // pair offsets k = 1..K in chunks of KC (one chunk when KC = K): node m
   // forms the pairs (m, m + k) of the chunk, then gathers the chunk's pairs
@@ -1214,7 +885,7 @@ __global__ void __launch_bounds__(EB * NP) hadamard_volume_kernel(
         if (n >= NP) n -= NP;
         T Smn[D];
 #pragma unroll
-        for (int i = 0; i < D; ++i) Smn[i] = Hm * __ldg(&op[((D + i) * NP + n) * NP + m]);
+        for (int i = 0; i < D; ++i) Smn[i] = Hm * __ldg(&op[(i * NP + n) * NP + m]);
         T G[NC];
         if constexpr (FLUX == 1) {
           IRNode<T, D> in_;
@@ -1319,7 +990,6 @@ struct VolCfg {
   // SM and one block's tensor phase runs beside another's float64 phase
   static constexpr int EB_SPLIT = NP == 7 ? 18 : NP == 12 ? 10 : NP == 18 ? 7 : NP == 27 ? 7 : NP == 25 ? 5
                                   : NP > 32 ? 2 : 128 / NP;
-  static constexpr int EB_BULK = (256 / NP) > 0 ? (256 / NP) : 1;
   // larger operators (tetrahedra of degree 3 and 4): the pair contributions
   // pass through shared memory in chunks of HAD_KC pair offsets, which leaves
   // room for more elements per block
@@ -1327,40 +997,23 @@ struct VolCfg {
   static constexpr int HAD_KC = NP > 32 ? 8 : NP / 2;
 };
 
-// T = float: the FP32-bulk kernel
-template <typename T, int D, int NP, int EB, bool VISC, bool CACHE, bool ENT>
+template <int D, int NP, int EB, bool VISC, bool CACHE, bool ENT>
 static void split_launch(esplit_ctx* c, const double* u, double* r, const double* sat, const int* list, int n_list,
                          int nb, double* prod, double* ent_part, cudaStream_t s) {
-  const Phys<double> ph = make_phys<double>(c->prm.gam, c->prm.beta, c->prm.R, c->prm.mu, c->prm.Pr);
-  const int heat = VISC ? c->prm.heat_flux : -1;
-  double* fcache = CACHE ? c->b.fcache : nullptr;
-  double* ncache = ENT ? c->b.node_cache : nullptr;
-  double* wsl = VISC && prod ? c->b.wslot : nullptr;
-  const double* va = VISC ? c->b.va : nullptr;
-  double* fv = VISC ? c->b.fv : nullptr;
+  using Cfg = SplitCfg<D, NP, EB, VISC>;
+  auto* kern = split_volume_kernel<D, NP, EB, VISC, CACHE, ENT>;
   static bool attr_set = false;
-  if constexpr (sizeof(T) == sizeof(double)) {
-    using Cfg = SplitCfg<D, NP, EB, VISC>;
-    auto* kern = split_volume_kernel<D, NP, EB, VISC, CACHE, ENT>;
-    if (!attr_set) {
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
-      cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-      attr_set = true;
-    }
-    kern<<<nb, Cfg::THREADS, Cfg::SMEM, s>>>(u, r, c->b.ops64, c->b.opsP, c->b.opsE, c->b.J, sat, list, n_list, ph,
-                                             c->b.status, prod, heat, c->b.nu, va, fv, fcache, c->n_e * c->n_slot,
-                                             ent_part, ncache, wsl);
-  } else {
-    const Phys<T> ph32 = make_phys<T>(c->prm.gam, c->prm.beta, c->prm.R, c->prm.mu, c->prm.Pr);
-    auto* kern = split_bulk_kernel<T, D, NP, EB, VISC, CACHE, ENT>;
-    if (!attr_set) {  // sized for four blocks per SM (inviscid, 2D) or two (viscous, 3D)
-      cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-      attr_set = true;
-    }
-    kern<<<nb, EB * NP, 0, s>>>(u, r, (const T*)c->b.ops32, c->b.ops32lo, c->b.rows, c->b.J, sat, list, n_list, ph32,
-                                ph, c->b.status, prod, heat, c->b.nu, va, fv, c->b.ops64, fcache,
-                                c->n_e * c->n_slot, ent_part, ncache, wsl);
+  if (!attr_set) {
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
+    cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    attr_set = true;
   }
+  const Phys<double> ph = make_phys<double>(c->prm.gam, c->prm.beta, c->prm.R, c->prm.mu, c->prm.Pr);
+  kern<<<nb, Cfg::THREADS, Cfg::SMEM, s>>>(u, r, c->b.ops64, c->b.opsP, c->b.opsE, c->b.J, sat, list, n_list, ph,
+                                           c->b.status, prod, VISC ? c->prm.heat_flux : -1, c->b.nu,
+                                           VISC ? c->b.va : nullptr, VISC ? c->b.fv : nullptr,
+                                           CACHE ? c->b.fcache : nullptr, c->n_e * c->n_slot, ent_part,
+                                           ENT ? c->b.node_cache : nullptr, VISC && prod ? c->b.wslot : nullptr);
 }
 
 template <typename T, int D, int NP>
@@ -1417,23 +1070,23 @@ static int residual_np(esplit_ctx* c, const double* u, double* r, cudaStream_t s
   const int* lsplit = scheme == ESPLIT_SCHEME_HYBRID ? c->b.list_split : nullptr;
   const int* lhad = scheme == ESPLIT_SCHEME_HYBRID ? c->b.list_had : nullptr;
   if (n_split > 0) {
-    constexpr int EB = std::is_same<T, double>::value ? VolCfg<NP>::EB_SPLIT : VolCfg<NP>::EB_BULK;
+    constexpr int EB = VolCfg<NP>::EB_SPLIT;
     int nb = (n_split + EB - 1) / EB;
     ProfScope ps(c, PG_SPLIT, s);
     double* pp = prod ? prod + np_used : nullptr;
     if (visc && c->ent_part && c->b.node_cache) {
       // first stage of a relaxation step: the kernel also forms the entropy of u_n
-      split_launch<T, D, NP, EB, true, false, true>(c, u, r, sat, lsplit, n_split, nb, pp, c->ent_part, s);
+      split_launch<D, NP, EB, true, false, true>(c, u, r, sat, lsplit, n_split, nb, pp, c->ent_part, s);
       c->ent_n = nb;
     } else if (visc)
-      split_launch<T, D, NP, EB, true, false, false>(c, u, r, sat, lsplit, n_split, nb, pp, nullptr, s);
+      split_launch<D, NP, EB, true, false, false>(c, u, r, sat, lsplit, n_split, nb, pp, nullptr, s);
     else if (cached && scheme == ESPLIT_SCHEME_SPLIT && c->ent_part && c->b.node_cache) {
-      split_launch<T, D, NP, EB, false, true, true>(c, u, r, sat, lsplit, n_split, nb, pp, c->ent_part, s);
+      split_launch<D, NP, EB, false, true, true>(c, u, r, sat, lsplit, n_split, nb, pp, c->ent_part, s);
       c->ent_n = nb;
     } else if (cached)
-      split_launch<T, D, NP, EB, false, true, false>(c, u, r, sat, lsplit, n_split, nb, pp, nullptr, s);
+      split_launch<D, NP, EB, false, true, false>(c, u, r, sat, lsplit, n_split, nb, pp, nullptr, s);
     else
-      split_launch<T, D, NP, EB, false, false, false>(c, u, r, sat, lsplit, n_split, nb, pp, nullptr, s);
+      split_launch<D, NP, EB, false, false, false>(c, u, r, sat, lsplit, n_split, nb, pp, nullptr, s);
     c->launches++;
     np_used += nb;
   }

@@ -88,7 +88,7 @@ __device__ __forceinline__ void pack_half(unsigned long long b, unsigned& x, uns
   w = u4 | ((u5 >> 6) << 10);
 }
 
-// one thread per (element, direction, row); ops64: [e][2d][n][m], D_i at k = d + i
+// one thread per (element, direction, row); ops64: [e][d][n][m]
 template <int BITS>
 __global__ void build_packed_kernel(const double* __restrict__ ops64, int n_e, int d, int np,
                                     uint4* __restrict__ opsP, short* __restrict__ opsE) {
@@ -96,9 +96,7 @@ __global__ void build_packed_kernel(const double* __restrict__ ops64, int n_e, i
   if (idx >= (size_t)n_e * d * np) return;
   const size_t ei = idx / np;
   const int m = (int)(idx - ei * np);
-  const size_t e = ei / d;
-  const int i = (int)(ei - e * d);
-  const double* op = ops64 + ((e * 2 * d + d + i) * np) * np + m;
+  const double* op = ops64 + (ei * np) * np + m;
   unsigned mx = 0;
   for (int n = 0; n < np; ++n) mx = max(mx, (unsigned)__double2hiint(op[(size_t)n * np]) & 0x7FFFFFFFu);
   const int E = exp_of_max(mx);

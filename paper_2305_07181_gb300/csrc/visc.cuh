@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(EB * NP) visc_volume_kernel(const double* __re
     }
   }
   __syncthreads();
-  const double* op = ops + (size_t)e * (2 * D * NP * NP);
+  const double* op = ops + (size_t)e * (D * NP * NP);
   double Hm = 0.0;
   if (active) {
     double g[D][NC];
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(EB * NP) visc_volume_kernel(const double* __re
 #pragma unroll
     for (int j = 0; j < D; ++j)
       for (int n = 0; n < NP; ++n) {
-        double dt = __ldg(&op[((D + j) * NP + n) * NP + m]);  // D_j[m][n]
+        double dt = __ldg(&op[(j * NP + n) * NP + m]);  // D_j[m][n]
 #pragma unroll
         for (int q = 0; q < NC; ++q) g[j][q] += dt * sw[el][q][n];
       }
@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(EB * NP) visc_volume_kernel(const double* __re
 #pragma unroll
   for (int i = 0; i < D; ++i)
     for (int n = 0; n < NP; ++n) {
-      double dt = __ldg(&op[((D + i) * NP + n) * NP + m]);
+      double dt = __ldg(&op[(i * NP + n) * NP + m]);
 #pragma unroll
       for (int q = 0; q < NC; ++q) acc[q] += dt * sF[el][i][q][n];
     }

@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(EB * NP) visc_vjp1_kernel(const double* __rest
   }
   __syncthreads();
   if (!active) return;
-  const double* op = ops + (size_t)e * (2 * D * NP * NP);
+  const double* op = ops + (size_t)e * (D * NP * NP);
   double g[D][NC], fb[D][NC], ab[D][NC];
 #pragma unroll
   for (int i = 0; i < D; ++i)
@@ -65,8 +65,8 @@ __global__ void __launch_bounds__(EB * NP) visc_vjp1_kernel(const double* __rest
 #pragma unroll
   for (int i = 0; i < D; ++i)
     for (int n = 0; n < NP; ++n) {
-      double dmn = __ldg(&op[((D + i) * NP + n) * NP + m]);  // D_i[m][n]
-      double dnm = __ldg(&op[((D + i) * NP + m) * NP + n]);  // D_i[n][m]
+      double dmn = __ldg(&op[(i * NP + n) * NP + m]);  // D_i[m][n]
+      double dnm = __ldg(&op[(i * NP + m) * NP + n]);  // D_i[n][m]
 #pragma unroll
       for (int q = 0; q < NC; ++q) {
         g[i][q] += dmn * sw[el][q][n];
@@ -256,14 +256,14 @@ __global__ void __launch_bounds__(EB * NP) visc_vjp3_kernel(const double* __rest
   }
   __syncthreads();
   if (!active) return;
-  const double* op = ops + (size_t)e * (2 * D * NP * NP);
+  const double* op = ops + (size_t)e * (D * NP * NP);
   double wb[NC];
 #pragma unroll
   for (int q = 0; q < NC; ++q) wb[q] = (sl >= 0) ? __ldg(&wbs[((size_t)e * NC + q) * NS + sl]) : 0.0;
 #pragma unroll
   for (int j = 0; j < D; ++j)
     for (int n = 0; n < NP; ++n) {
-      double dnm = __ldg(&op[((D + j) * NP + m) * NP + n]);  // D_j[n][m]
+      double dnm = __ldg(&op[(j * NP + m) * NP + n]);  // D_j[n][m]
 #pragma unroll
       for (int q = 0; q < NC; ++q) wb[q] += dnm * sgb[el][j][q][n];
     }

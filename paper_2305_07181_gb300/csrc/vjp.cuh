@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(round32(EB * NP), VjpCfg<D, NP, EB>::BLOCKS) s
   int* ex = reinterpret_cast<int*>(vjp_smem + Cfg::DIG + Cfg::RES);
   int* elems = reinterpret_cast<int*>(vjp_smem + Cfg::DIG + Cfg::RES + Cfg::EXB);
   double* sx = reinterpret_cast<double*>(vjp_smem);  // float64 loops: [EB][columns][NP]
-  const double* op = ops + (size_t)(active ? e : 0) * (2 * D * NP * NP) + D * NP * NP;
+  const double* op = ops + (size_t)(active ? e : 0) * (D * NP * NP);
   double g[D][NC], t[D][NC];  // D_i w, D_i (cot/H)
   if constexpr (Cfg::TENSOR) {
     if (m == 0 && slot) elems[el] = active ? e : -1;
