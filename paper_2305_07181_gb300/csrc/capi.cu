@@ -666,9 +666,25 @@ static int rrk_enqueue_stages(esplit_ctx* c, const double* u, double dt, cudaStr
   }
   c->ent_part = side ? nullptr : c->b.partial;
   c->ent_n = 0;
+  // where the volume kernels alone read the state they form the stage's from
+  // u_n and the previous residual themselves, and the root solve's first pass
+  // adds the last stage's share of dacc: no stage kernels
+  const bool fused = esplit::stage_in_volume(c);
+  c->stage_last = esplit::StageIn{};
+  if (fused) {
+    c->stage_last.b = B[3] * dt;
+    c->stage_last.dacc = c->b.dacc;
+  }
   for (int i = 0; i < 4; ++i) {
-    const double* Ui = (i == 0) ? u : c->b.stage_u;
+    const double* Ui = (i == 0 || fused) ? u : c->b.stage_u;
+    if (fused && i > 0) {
+      c->stage.a = A[i] * dt;
+      c->stage.b = B[i - 1] * dt;
+      c->stage.dacc = c->b.dacc;
+      c->stage.first = i == 1;
+    }
     rc = residual_impl(c, Ui, c->b.stage_r, s, c->b.partial + off, &np);
+    c->stage = esplit::StageIn{};
     if (i == 0) {
       c->ent_part = nullptr;
       if (rc) return rc;
@@ -687,7 +703,7 @@ static int rrk_enqueue_stages(esplit_ctx* c, const double* u, double dt, cudaStr
     R.out[1 + i] = c->b.scal + 2 + i;
     off += np;
     double a_next = (i < 3) ? A[i + 1] * dt : 0.0;
-    if (esplit::launch_stage(c, u, c->b.stage_r, a_next, B[i] * dt, i == 0, (i < 3) ? c->b.stage_u : nullptr,
+    if (!fused && esplit::launch_stage(c, u, c->b.stage_r, a_next, B[i] * dt, i == 0, (i < 3) ? c->b.stage_u : nullptr,
                              c->b.dacc, n, s))
       return fail(c, ESPLIT_ERR_CUDA, "stage launch");
   }
@@ -993,6 +1009,7 @@ int esplit_rrk_step_vjp(esplit_ctx* c, const double* u, double dt, const double*
   if (!c->b.node_cache) {
     if ((rc = dalloc(c, &c->b.node_cache, 3 * (size_t)c->n_e * c->n_p))) return rc;
   }
+  c->stage_last = esplit::StageIn{};
   double* W = c->b.vjp_work;
   double* Us[3] = {W, W + n, W + 2 * n};                  // U_2, U_3, U_4
   double* Rs[4] = {W + 3 * n, W + 4 * n, W + 5 * n, W + 6 * n};

@@ -13,9 +13,11 @@
 //         2^(j/32) tabulated as a float64 pair.
 //   log1p(x) = log(u + c) with u = 1 + x rounded and c = x - (u - 1) the
 //   rounding error, carried into r; for |x| < 2^-5 directly by its Taylor
-//   series through x^12 (truncation < 2^-63 |x|); expm1 from the exp reduction as
+//   series through x^12 (truncation < 2^-63 |x|), all but two operations of it
+//   in fixed point (imath.cuh); expm1 from the exp reduction as
 //   (2^k T_hi - 1) + 2^k (T_hi p + T_lo) (the first difference is exact where
-//   it cancels), and for |x| < 1/16 by its Taylor series through x^10.
+//   it cancels), and for |x| < 1/16 by its Taylor series through x^10,
+//   in fixed point likewise.
 //   Tables: fmath_tables.h (gen_fmath_tables.py).
 // Domain: finite normal positive arguments for log (log1p: 1 + x normal
 // positive), |x| < 708 for exp/expm1; anything else goes to the CUDA library
@@ -26,6 +28,7 @@
 #pragma once
 
 #include "fmath_tables.h"
+#include "imath.cuh"
 
 namespace esplit {
 namespace fm {
@@ -97,17 +100,7 @@ __device__ __forceinline__ double log(double x) { return log_domain(x) ? log_cor
 
 __device__ __forceinline__ double log1p(double x) {
   if (abs_below(x, BITS_2M5)) {
-    double q = fma(x, LOG_C12, LOG_C11);
-    q = fma(x, q, LOG_C10);
-    q = fma(x, q, LOG_C9);
-    q = fma(x, q, LOG_C8);
-    q = fma(x, q, LOG_C7);
-    q = fma(x, q, LOG_C6);
-    q = fma(x, q, LOG_C5);
-    q = fma(x, q, LOG_C4);
-    q = fma(x, q, LOG_C3);
-    q = fma(x, q, LOG_C2);
-    return fma(x * x, q, x);
+    return fma(-(x * x), im::log1p_tail(x), x);
   }
   const double u = 1.0 + x;
   if (!log_domain(u)) return ::log1p(x);
@@ -143,15 +136,7 @@ __device__ __forceinline__ double exp(double x) {
 
 __device__ __forceinline__ double expm1(double x) {
   if (abs_below(x, BITS_2M4)) {  // Taylor series through x^10 (truncation < 2^-64 |x|)
-    double q = fma(x, EXP_E10, EXP_E9);
-    q = fma(x, q, EXP_E8);
-    q = fma(x, q, EXP_E7);
-    q = fma(x, q, EXP_E6);
-    q = fma(x, q, EXP_E5);
-    q = fma(x, q, EXP_E4);
-    q = fma(x, q, EXP_E3);
-    q = fma(x, q, EXP_E2);
-    return fma(x * x, q, x);
+    return fma(x * x, im::expm1_tail(x), x);
   }
   if (!abs_below(x, BITS_708)) return ::expm1(x);
   int j, k;

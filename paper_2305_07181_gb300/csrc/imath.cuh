@@ -110,6 +110,59 @@ IM_FN double exp_fixed(long long X) {
   return __longlong_as_double((long long)(m + ((unsigned long long)(1023 + (N >> 9) - lz) << 52)));
 }
 
+// |x| < 2^-4 in units of 2^-66, truncated
+IM_FN long long small_to_fixed(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int sh = 1018 - ((int)(b >> 52) & 0x7ff);  // x = M 2^(-57 - sh), M < 2^53
+  const unsigned long long M = (b & 0xFFFFFFFFFFFFFULL) | 0x10000000000000ULL;
+  const unsigned long long v = sh > 62 ? 0ULL : ((M << 9) >> sh);
+  return (b >> 63) ? -(long long)v : (long long)v;
+}
+
+// s 2^-62 as a float64, rounded to nearest, for s > 0
+IM_FN double unit62_to_double(long long s) {
+  const int lz = __clzll(s);
+  const unsigned long long n = (unsigned long long)s << lz;
+  const unsigned long long m = (n >> 11) + ((n >> 10) & 1ULL);
+  return __longlong_as_double((long long)(m + ((unsigned long long)(1023 - lz) << 52)));
+}
+
+// one Horner step s <- c + s x, s and c of unit 2^-62, x of unit 2^-66
+IM_FN long long horner62(long long s, long long x, long long c) { return c + (__mul64hi(s, x) >> 2); }
+
+constexpr long long U62(double v) { return (long long)(v * 4611686018427387904.0); }  // 2^62
+
+// P(x) = (x - log1p x)/x^2 = 1/2 - x/3 + x^2/4 - ..., |x| < 2^-5: terms 0 to 5
+// in 64-bit fixed point, 6 to 10 (below 2^-30 of the sum) in float32
+IM_FN double log1p_tail(double x) {
+  const long long f = small_to_fixed(x);
+  const float y = __int2float_rn((int)(f >> 32)) * 0x1p-34f;
+  const float t = 1.0f / 8 + y * (-1.0f / 9 + y * (1.0f / 10 + y * (-1.0f / 11 + y * (1.0f / 12))));
+  long long s = (long long)__float2int_rn(t * 0x1p30f) << 32;
+  s = horner62(s, f, U62(-1.0 / 7));
+  s = horner62(s, f, U62(1.0 / 6));
+  s = horner62(s, f, U62(-1.0 / 5));
+  s = horner62(s, f, U62(1.0 / 4));
+  s = horner62(s, f, -0x1555555555555555LL);  // 1/3
+  s = horner62(s, f, 1LL << 61);
+  return unit62_to_double(s);
+}
+
+// Q(x) = (expm1 x - x)/x^2 = 1/2 + x/6 + x^2/24 + ..., |x| < 2^-4: terms 0 to 4
+// in 64-bit fixed point, 5 to 8 (below 2^-32 of the sum) in float32
+IM_FN double expm1_tail(double x) {
+  const long long f = small_to_fixed(x);
+  const float y = __int2float_rn((int)(f >> 32)) * 0x1p-34f;
+  const float t = 1.0f / 5040 + y * (1.0f / 40320 + y * (1.0f / 362880 + y * (1.0f / 3628800)));
+  long long s = (long long)__float2int_rn(t * 0x1p32f) << 30;
+  s = horner62(s, f, U62(1.0 / 720));
+  s = horner62(s, f, U62(1.0 / 120));
+  s = horner62(s, f, U62(1.0 / 24));
+  s = horner62(s, f, 0x0AAAAAAAAAAAAAAALL);  // 1/6
+  s = horner62(s, f, 1LL << 61);
+  return unit62_to_double(s);
+}
+
 // X 2^-57 as a float64, rounded to nearest (ties away from zero)
 IM_FN double to_double(long long X) {
   const unsigned long long u = (unsigned long long)(X < 0 ? -X : X);

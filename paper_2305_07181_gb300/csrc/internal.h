@@ -38,6 +38,14 @@ struct RootState {
   unsigned int arrivals;      // blocks of the running evaluation pass that are done
 };
 
+// A Runge-Kutta stage whose state the volume kernels form from u_n and the
+// previous residual (dacc null: the state is given), see stage_state
+struct StageIn {
+  double a = 0.0, b = 0.0;
+  double* dacc = nullptr;
+  int first = 0;
+};
+
 struct Buffers {
   // operators
   double* Qref = nullptr;      // [d][n_p][n_p]
@@ -144,6 +152,9 @@ struct esplit_ctx {
   // partials of H s, H |s| at ent_part) and reports its block count in ent_n
   double* ent_part = nullptr;
   int ent_n = 0;
+  // set by the relaxation step around its stage residuals 2 to 4, and around
+  // the root solve's first pass (the last stage's share of dacc)
+  esplit::StageIn stage, stage_last;
   cudaStream_t last_stream = nullptr;
   // bumped by every change that alters what a step launches (operator, mesh,
   // parameters, hybrid flags); a recorded step graph of another version is stale
@@ -212,6 +223,7 @@ struct StepRecord {
 int launch_step_record(esplit_ctx* c, StepRecord* hist, int* counter, int cap, cudaStream_t s);
 int launch_root_apply(esplit_ctx* c, double* un, const double* d, size_t n, cudaStream_t s);
 int set_ref_tables(const RefTables& t);
+bool stage_in_volume(const esplit_ctx* c);  // the volume kernels can form a stage's state
 bool uses_f32_path(const esplit_ctx* c);  // the residual takes the float32 path (fp32.cu)
 int set_ref_tables_vjp(const RefTables& t);  // the reverse-mode unit's copy (vjp.cu)
 // float32 path of the inviscid split scheme (fp32.cu): its own copy of the

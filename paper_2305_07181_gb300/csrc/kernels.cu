@@ -555,6 +555,21 @@ struct SplitCfg {
   static constexpr int BLOCKS = BY_SMEM < BY_REGS ? BY_SMEM : BY_REGS;
 };
 
+// The state of a Runge-Kutta stage formed where the volume kernels load it:
+// u = u_n + a r_prev, r_prev being the residual buffer's content (each thread
+// reads its own entries before it writes them), and dacc (= or +=) b r_prev.
+// Saves the stage kernel's launch and the stage state's write and read.
+template <int NC>
+__device__ __forceinline__ void stage_state(const StageIn& st, const double* r, size_t ix0, int stride, double* uu) {
+#pragma unroll
+  for (int q = 0; q < NC; ++q) {
+    const size_t ix = ix0 + (size_t)q * stride;
+    const double rq = r[ix];
+    uu[q] += st.a * rq;
+    st.dacc[ix] = st.first ? st.b * rq : st.dacc[ix] + st.b * rq;
+  }
+}
+
 template <int D, int NP, int EB, bool VISC, bool CACHE = false, bool ENT = false>
 __global__ void __launch_bounds__(round32(EB * NP), SplitCfg<D, NP, EB, VISC>::BLOCKS) split_volume_kernel(
     const double* __restrict__ u, double* __restrict__ r, const double* __restrict__ ops64,
@@ -562,7 +577,7 @@ __global__ void __launch_bounds__(round32(EB * NP), SplitCfg<D, NP, EB, VISC>::B
     const double* __restrict__ sat, const int* __restrict__ list, int n_list, Phys<double> c64,
     int* __restrict__ status, double* __restrict__ prod, int visc_heat, const double* __restrict__ nu,
     const double* __restrict__ ah, double* __restrict__ fvs, double* __restrict__ fcache, int n_slot_total,
-    double* __restrict__ ent_part = nullptr, double* __restrict__ ncache = nullptr,
+    StageIn st, double* __restrict__ ent_part = nullptr, double* __restrict__ ncache = nullptr,
     double* __restrict__ wsl = nullptr) {
   constexpr int NC = D + 2;
   using Cfg = SplitCfg<D, NP, EB, VISC>;
@@ -587,6 +602,8 @@ __global__ void __launch_bounds__(round32(EB * NP), SplitCfg<D, NP, EB, VISC>::B
     double uu[NC];
 #pragma unroll
     for (int q = 0; q < NC; ++q) uu[q] = __ldg(&u[((size_t)e * NC + q) * NP + m]);
+    if constexpr (CACHE && !ENT)
+      if (st.dacc) stage_state<NC>(st, r, (size_t)e * NC * NP + m, NP, uu);
     if (!node_from_u<double, D>(uu, c64, nd)) atomicOr(status, 1);
     euler_fluxes<D>(nd, uu, vals);
 #pragma unroll
@@ -775,7 +792,7 @@ __global__ void __launch_bounds__(EB * NP) hadamard_volume_kernel(
     const double* __restrict__ u, double* __restrict__ r, const T* __restrict__ ops,
     const double* __restrict__ J, const double* __restrict__ sat, const int* __restrict__ list, int n_list,
     Phys<T> c, Phys<double> c64, int* __restrict__ status, double* __restrict__ prod,
-    double* __restrict__ fcache = nullptr, int n_slot_total = 0) {
+    double* __restrict__ fcache = nullptr, int n_slot_total = 0, StageIn st = StageIn{}) {
   constexpr int NC = D + 2;
   constexpr int K = NP / 2;
   constexpr int NZ = D + 7;  // q, V[D], p, P1, P2, v2, 1/q, 1/p
@@ -794,6 +811,8 @@ __global__ void __launch_bounds__(EB * NP) hadamard_volume_kernel(
     T uu[NC];
 #pragma unroll
     for (int q = 0; q < NC; ++q) uu[q] = (T)__ldg(&u[((size_t)e * NC + q) * NP + m]);
+    if constexpr (sizeof(T) == sizeof(double) && FLUX == 0)
+      if (st.dacc) stage_state<NC>(st, r, (size_t)e * NC * NP + m, NP, uu);
     if (!node_from_u<T, D>(uu, c, nd)) atomicOr(status, 1);
     T* zz = sz + el * NZ * NP;
     if constexpr (FLUX == 1) {  // Ismail-Roe: z_1, z_nc, their logs, V
@@ -960,13 +979,18 @@ __global__ void __launch_bounds__(EB * NP) hadamard_volume_kernel(
       r[((size_t)e * NC + q) * NP + m] = res[q];
     }
     if (prod) {
-      double u64[NC];
+      if constexpr (sizeof(T) == sizeof(double)) {
 #pragma unroll
-      for (int q = 0; q < NC; ++q) u64[q] = __ldg(&u[((size_t)e * NC + q) * NP + m]);
-      Node<double, D> n64;
-      node_from_u<double, D>(u64, c64, n64);
+        for (int q = 0; q < NC; ++q) hw += nd.W[q] * res[q];
+      } else {
+        double u64[NC];
 #pragma unroll
-      for (int q = 0; q < NC; ++q) hw += n64.W[q] * res[q];
+        for (int q = 0; q < NC; ++q) u64[q] = __ldg(&u[((size_t)e * NC + q) * NP + m]);
+        Node<double, D> n64;
+        node_from_u<double, D>(u64, c64, n64);
+#pragma unroll
+        for (int q = 0; q < NC; ++q) hw += n64.W[q] * res[q];
+      }
       hw *= c_ref.H[m] * __ldg(&J[(size_t)e * NP + m]);
     }
   }
@@ -1012,7 +1036,7 @@ static void split_launch(esplit_ctx* c, const double* u, double* r, const double
   kern<<<nb, Cfg::THREADS, Cfg::SMEM, s>>>(u, r, c->b.ops64, c->b.opsP, c->b.opsE, c->b.J, sat, list, n_list, ph,
                                            c->b.status, prod, VISC ? c->prm.heat_flux : -1, c->b.nu,
                                            VISC ? c->b.va : nullptr, VISC ? c->b.fv : nullptr,
-                                           CACHE ? c->b.fcache : nullptr, c->n_e * c->n_slot, ent_part,
+                                           CACHE ? c->b.fcache : nullptr, c->n_e * c->n_slot, c->stage, ent_part,
                                            ENT ? c->b.node_cache : nullptr, VISC && prod ? c->b.wslot : nullptr);
 }
 
@@ -1113,7 +1137,7 @@ static int residual_np(esplit_ctx* c, const double* u, double* r, cudaStream_t s
       // written instead
       hadamard_volume_kernel<T, D, NP, EB, 0, KC><<<nb, EB * NP, smem, s>>>(
           u, r, ops, c->b.J, nullptr, lhad, n_had, ph, ph64, c->b.status, prod ? prod + np_used : nullptr,
-          c->b.fcache, c->n_e * c->n_slot);
+          c->b.fcache, c->n_e * c->n_slot, c->stage);
     else
       hadamard_volume_kernel<T, D, NP, EB, 0, KC><<<nb, EB * NP, smem, s>>>(
           u, r, ops, c->b.J, sat, lhad, n_had, ph, ph64, c->b.status, prod ? prod + np_used : nullptr);
@@ -1188,6 +1212,16 @@ static bool use_f32_path(const esplit_ctx* c) {
 
 bool uses_f32_path(const esplit_ctx* c) { return use_f32_path(c); }
 
+// whether the residual's volume kernels are the only readers of the state, so
+// that they can form a stage's state themselves: the cached facet path (see
+// residual_np) without boundary facets
+bool stage_in_volume(const esplit_ctx* c) {
+  const int sch = c->prm.scheme;
+  return !use_f32_path(c) && !c->prm.viscous && c->n_bslot == 0 && c->b.fcache &&
+         (sch == ESPLIT_SCHEME_SPLIT ||
+          ((sch == ESPLIT_SCHEME_HYBRID || sch == ESPLIT_SCHEME_HADAMARD) && c->prm.precision == ESPLIT_FP64));
+}
+
 int launch_residual(esplit_ctx* c, const double* u, double* r, cudaStream_t s, double* prod, int* n_partial) {
   if (use_f32_path(c)) return launch_split_f32(c, u, r, s, prod, n_partial, c->b.sat);
   if (c->prm.precision != ESPLIT_FP64) return residual_t<float>(c, u, r, s, prod, n_partial, c->b.sat);
@@ -1256,7 +1290,7 @@ __global__ void __launch_bounds__(256) entropy_kernel(const double* __restrict__
 #pragma unroll
     for (int i = 0; i < D; ++i) mm += uu[1 + i] * uu[1 + i];
     const double P = c.gm1 * (rho * uu[NC - 1] - 0.5 * mm);
-    const double y = 1.0 / (rho * P);
+    const double y = rcp64(rho * P);
     const double ir = P * y, ip = (rho * rho) * y, p = P * ir;
     // S_H = beta rho (p rho^-gam)^(1/(alpha+gam)) = beta q p, log q = a_q log rho + b_q log p
     double lnp, lnq, q;
@@ -1496,7 +1530,7 @@ __device__ __forceinline__ void entropy_change_and_slope(const double* u, const 
     mdm += m * dm;
     dmdm += dm * dm;
   }
-  double ir1 = 1.0 / (rho + drho);  // 1/rho'
+  double ir1 = rcp64(rho + drho);  // 1/rho'
   double dke = 0.5 * ((2.0 * mdm + dmdm) - mm * drho * ir) * ir1;
   double dp = c.gm1 * (dE - dke);
   double l1 = fm::log1p(drho * ir), l2 = fm::log1p(dp * ip);
@@ -1504,7 +1538,7 @@ __device__ __forceinline__ void entropy_change_and_slope(const double* u, const 
   // entropy variables at u' = u + g d (Eq. (25)); q' = s'/(beta p') with
   // s' = s + ds (S_H = beta q p), one division that also gives 1/p'
   double p1 = c.gm1 * (u[NC - 1] - 0.5 * mm * ir) + dp;
-  double ibp1 = 1.0 / (c.beta * p1);
+  double ibp1 = rcp64(c.beta * p1);
   double q1 = (s0 + ds) * ibp1;
   double v2 = 0.0, vd = 0.0;
 #pragma unroll
@@ -1547,11 +1581,13 @@ __device__ void root_update_body(const double* tot, RootState* st);
 // bracket search after 10 halvings or 2 doublings); the hard stop below ends
 // the loop even if that reasoning failed, with status "no root".
 template <int D, bool COND>
-__global__ void __launch_bounds__(256) root_eval_kernel(const double* __restrict__ un, const double* __restrict__ d,
+__global__ void __launch_bounds__(256) root_eval_kernel(const double* __restrict__ un, const double* d,
                                                         const double* __restrict__ J,
                                                         const double* __restrict__ cache, size_t n_nodes,
                                                         Phys<double> c, RootState* __restrict__ st,
-                                                        double* __restrict__ part, cudaGraphConditionalHandle h) {
+                                                        double* __restrict__ part, StageIn add,
+                                                        const double* __restrict__ r_last,
+                                                        cudaGraphConditionalHandle h) {
   if (st->done) {
     if constexpr (COND)
       if (blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(h, 0u);
@@ -1560,6 +1596,7 @@ __global__ void __launch_bounds__(256) root_eval_kernel(const double* __restrict
   constexpr int NC = D + 2;
   const int NP = c_ref.n_p;
   const double ga = st->ga, gb = st->gb;
+  const bool add_last = add.dacc && st->iters == 0;
   size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   if (t < n_nodes) {
@@ -1569,7 +1606,15 @@ __global__ void __launch_bounds__(256) root_eval_kernel(const double* __restrict
 #pragma unroll
     for (int q = 0; q < NC; ++q) {
       size_t ix = (e * NC + q) * NP + m;
-      dd[q] = __ldg(&d[ix]);
+      // the first pass completes d with the last stage's residual (each entry
+      // by the one thread that reads it; the iteration count is advanced by the
+      // block that finishes last)
+      if (add_last) {
+        dd[q] = add.dacc[ix] + add.b * __ldg(&r_last[ix]);
+        add.dacc[ix] = dd[q];
+      } else {
+        dd[q] = d[ix];
+      }
       uu[q] = __ldg(&un[ix]);
     }
     double s0 = __ldg(&cache[t]), ir = __ldg(&cache[n_nodes + t]);
@@ -1783,11 +1828,14 @@ static int root_eval_launch(esplit_ctx* c, const double* un, const double* d, cu
   int nb = (int)((n + 255) / 256);
   Phys<double> ph = make_phys<double>(c->prm.gam, c->prm.beta, c->prm.R, c->prm.mu, c->prm.Pr);
   if (c->dim == 1)
-    root_eval_kernel<1, COND><<<nb, 256, 0, s>>>(un, d, c->b.J, c->b.node_cache, n, ph, c->b.root, c->b.partial, h);
+    root_eval_kernel<1, COND><<<nb, 256, 0, s>>>(un, d, c->b.J, c->b.node_cache, n, ph, c->b.root, c->b.partial, c->stage_last,
+                                                   c->b.stage_r, h);
   else if (c->dim == 2)
-    root_eval_kernel<2, COND><<<nb, 256, 0, s>>>(un, d, c->b.J, c->b.node_cache, n, ph, c->b.root, c->b.partial, h);
+    root_eval_kernel<2, COND><<<nb, 256, 0, s>>>(un, d, c->b.J, c->b.node_cache, n, ph, c->b.root, c->b.partial, c->stage_last,
+                                                   c->b.stage_r, h);
   else
-    root_eval_kernel<3, COND><<<nb, 256, 0, s>>>(un, d, c->b.J, c->b.node_cache, n, ph, c->b.root, c->b.partial, h);
+    root_eval_kernel<3, COND><<<nb, 256, 0, s>>>(un, d, c->b.J, c->b.node_cache, n, ph, c->b.root, c->b.partial, c->stage_last,
+                                                   c->b.stage_r, h);
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }

@@ -561,8 +561,6 @@ __device__ __forceinline__ double rsqrt64(double x) {
 __device__ __forceinline__ double exp_avg_pair(double a, double b, double ar, double br, double r, double ia,
                                                const double* coef, const long long* s62, const float* tail, int ok) {
   const double eps = (b - a) * ia;
-  const unsigned long long bits = (unsigned long long)__double_as_longlong(eps);
-  const int e = (int)(bits >> 52) & 0x7ff;
   if (!fm::abs_below(eps, 0x3FA999999999999AULL)) return (ar - br) / (r * (a - b));  // 0.05
   if (!ok) {
     double sum = coef[ExpAvgCfg<double>::NTERMS - 1];
@@ -570,23 +568,15 @@ __device__ __forceinline__ double exp_avg_pair(double a, double b, double ar, do
     for (int k = ExpAvgCfg<double>::NTERMS - 2; k >= 0; --k) sum = sum * eps + coef[k];
     return ar * ia * sum;
   }
-  // eps = M 2^(e - 1075) in units of 2^-66: e <= 1018, a shift of at most 9
-  const unsigned long long M = (bits & 0xFFFFFFFFFFFFFULL) | 0x10000000000000ULL;
-  const int sh = 1018 - e;
-  const unsigned long long mag = sh > 62 ? 0ULL : ((M << 9) >> sh);
-  const long long x = (bits >> 63) ? -(long long)mag : (long long)mag;
+  const long long x = im::small_to_fixed(eps);
   const float xf = __int2float_rn((int)(x >> 32)) * 0x1p-34f;
   float t = tail[5];
 #pragma unroll
   for (int k = 4; k >= 0; --k) t = t * xf + tail[k];
   long long s = (long long)__float2int_rn(t * 0x1p30f) << 32;
 #pragma unroll
-  for (int k = 6; k >= 0; --k) s = s62[k] + (__mul64hi(s, x) >> 2);
-  // s is in (0.9, 1.1): two binades, the leading bit 61 or 62
-  const int lz = __clzll(s);
-  const unsigned long long n = (unsigned long long)s << lz;
-  const unsigned long long m = (n >> 11) + ((n >> 10) & 1ULL);
-  const double sum = __longlong_as_double((long long)(m + ((unsigned long long)(1023 - lz) << 52)));
+  for (int k = 6; k >= 0; --k) s = im::horner62(s, x, s62[k]);
+  const double sum = im::unit62_to_double(s);
   return ar * ia * sum;
 }
 
