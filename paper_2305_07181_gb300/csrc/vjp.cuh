@@ -21,100 +21,96 @@
 
 namespace esplit {
 
-// X^ |Lambda_n| S^ X^T dw of Eq. (69), as diss_apply, one column of X^ at a
-// time; n and dw may be plain doubles (no derivative parts).
-template <typename T, typename TN, typename TW, int D, typename C>
-__device__ __forceinline__ void diss_apply_cols(const PairAvg<T, D>& a, const C& c, const TN* n, const TW* dw,
-                                                T* out) {
-  constexpr int NC = D + 2;
-  T rho_h = a.z1a / (a.A1 * a.E1);
-  T iz = T(1.0) / a.z1a;
-  T Vh[D];
-  T vh2 = T(0.0), vn = T(0.0);
-#pragma unroll
-  for (int i = 0; i < D; ++i) {
-    Vh[i] = a.qV[i] * iz;
-    vh2 = vh2 + Vh[i] * Vh[i];
-    vn = vn + Vh[i] * n[i];
-  }
-  T p_h = a.pa;
-  T theta = rho_h / (p_h * a.A1 * a.E1);
-  T eta = T(1.0) / (a.z1a * a.E2 * a.E1);
-  T ah = t_sqrt(c.gam * p_h / rho_h);
-  T Hh = ah * ah * c.inv_gm1 + 0.5 * vh2;
-#pragma unroll
-  for (int r = 0; r < NC; ++r) out[r] = T(0.0);
-#pragma unroll
-  for (int k = 0; k < NC; ++k) {
-    T col[NC];
-    T ls;
-    if (k == 0 || k == NC - 1) {
-      const double sg = (k == 0) ? -1.0 : 1.0;
-      col[0] = T(1.0);
-#pragma unroll
-      for (int i = 0; i < D; ++i) col[1 + i] = Vh[i] + sg * (ah * n[i]);
-      col[NC - 1] = Hh + sg * (ah * vn);
-      ls = t_abs(vn + sg * ah) * (c.s_ac * theta);
-    } else if (k == 1) {
-      col[0] = T(1.0);
-#pragma unroll
-      for (int i = 0; i < D; ++i) col[1 + i] = Vh[i];
-      col[NC - 1] = 0.5 * vh2;
-      ls = t_abs(vn) * (c.s_en * theta);
-    } else {
-      // tangential columns as printed: (0, n2, -n1, 0, V1 n2 - V2 n1) and
-      // (0, -n3, 0, n1, V3 n1 - V1 n3) (2D: the first without its 4th row)
-#pragma unroll
-      for (int r = 0; r < NC; ++r) col[r] = T(0.0);
-      if (k == 2) {
-        col[1] = T(n[1]);
-        col[2] = T(-n[0]);
-        col[NC - 1] = Vh[0] * n[1] - Vh[1] * n[0];
-      } else {
-        col[1] = T(-n[D - 1]);
-        col[3] = T(n[0]);
-        col[NC - 1] = Vh[D - 1] * n[0] - Vh[0] * n[D - 1];
-      }
-      ls = t_abs(vn) * eta;
-    }
-    T y = col[0] * dw[0];
-#pragma unroll
-    for (int r = 1; r < NC; ++r) y = y + col[r] * dw[r];
-    y = y * ls;
-#pragma unroll
-    for (int r = 0; r < NC; ++r) out[r] = out[r] + col[r] * y;
-  }
-}
-
 __device__ __forceinline__ double sgn0(double x) { return x > 0.0 ? 1.0 : (x < 0.0 ? -1.0 : 0.0); }
 
-// reverse of exp_avg (Eq. (47)) at the values: E = (ar - br)/(r (a - b)) or
-// ar ia g(eps), eps = (b - a) ia; adds the adjoints of a, b, ar, br, ia for Eb
-__device__ __forceinline__ void exp_avg_rev(double a, double b, double ar, double br, double r, double ia,
-                                            const double* coef, double Eb, double& ab, double& bb, double& arb,
-                                            double& brb, double& iab) {
-  const double eps = (b - a) * ia;
-  if (fabs(eps) >= ExpAvgCfg<double>::EPS_SWITCH) {
-    const double q = 1.0 / (r * (a - b));
-    const double E = (ar - br) * q;
-    arb += Eb * q;
-    brb -= Eb * q;
-    ab -= Eb * E / (a - b);
-    bb += Eb * E / (a - b);
+// exp_avg (Eq. (47)) and its partial derivatives at the values:
+// E = (ar - br)/(r (a - b)) or ar ia g(eps), eps = (b - a) ia, with the series
+// g and g' in fixed point (terms 0 to 6; the rest in float32) as exp_avg_pair
+struct ExpAvgD {
+  double E, Ea, Eb, Ear, Ebr, Eia;
+};
+__device__ __forceinline__ void exp_avg_d(double a, double b, double ar, double br, double r, double ia,
+                                          const double* coef, const long long* s62, const float* tail, int ok,
+                                          ExpAvgD& o) {
+  const double df = b - a, eps = df * ia;
+  if (!fm::abs_below(eps, 0x3FA999999999999AULL)) {  // 0.05
+    const double id = rcp64(a - b), q = id / r;
+    o.E = (ar - br) * q;
+    o.Ear = q;
+    o.Ebr = -q;
+    o.Ea = -o.E * id;
+    o.Eb = -o.Ea;
+    o.Eia = 0.0;
     return;
   }
-  double sv = coef[ExpAvgCfg<double>::NTERMS - 1], dv = 0.0;
+  double sv, dv;
+  if (ok) {
+    const long long x = im::small_to_fixed(eps);
+    const float xf = __int2float_rn((int)(x >> 32)) * 0x1p-34f;
+    float t = tail[5], td = 0.0f;
 #pragma unroll
-  for (int k = ExpAvgCfg<double>::NTERMS - 2; k >= 0; --k) {
-    dv = dv * eps + sv;
-    sv = sv * eps + coef[k];
+    for (int k = 4; k >= 0; --k) {
+      td = td * xf + t;
+      t = t * xf + tail[k];
+    }
+    long long s = (long long)__float2int_rn(t * 0x1p30f) << 32, d = (long long)__float2int_rn(td * 0x1p28f) << 34;
+#pragma unroll
+    for (int k = 6; k >= 0; --k) {
+      d = im::horner62(d, x, s);
+      s = im::horner62(s, x, s62[k]);
+    }
+    sv = im::unit62_to_double(s);
+    // g'(0) = (r - 1)/2 < 0 and stays negative below the switch
+    dv = -im::unit62_to_double(-d);
+  } else {
+    sv = coef[ExpAvgCfg<double>::NTERMS - 1];
+    dv = 0.0;
+#pragma unroll
+    for (int k = ExpAvgCfg<double>::NTERMS - 2; k >= 0; --k) {
+      dv = dv * eps + sv;
+      sv = sv * eps + coef[k];
+    }
   }
-  // E = ar ia sv(eps)
-  arb += Eb * ia * sv;
-  const double epsb = Eb * ar * ia * dv;
-  iab += Eb * ar * sv + epsb * (b - a);
-  bb += epsb * ia;
-  ab -= epsb * ia;
+  o.Ear = ia * sv;
+  o.Ebr = 0.0;
+  o.E = ar * o.Ear;
+  const double w = ar * ia * dv;
+  o.Eb = w * ia;
+  o.Ea = -o.Eb;
+  o.Eia = ar * sv + w * df;
+}
+
+// The pair's averages, the derivatives of its exponential averages, and the
+// reciprocals the reverse sweep multiplies by instead of dividing
+template <int D>
+struct PairRev {
+  PairAvg<double, D> a;
+  ExpAvgD e1, e2;  // E1 (of p), E2 (of q)
+  double iA1, iE1, iE2, iz;
+};
+
+template <int D, typename C>
+__device__ __forceinline__ void pair_rev_prep(const ZNode<double, D>& k, const ZNode<double, D>& v, const C& c,
+                                              PairRev<D>& p) {
+  exp_avg_d(k.p, v.p, k.P2, v.P2, c.r2, k.ip, c.ser2, c.s2, c.t2, c.im_ok, p.e1);
+  exp_avg_d(k.q, v.q, k.P1, v.P1, c.r1, k.iq, c.ser1, c.s1, c.t1, c.im_ok, p.e2);
+  p.a.A1 = 0.5 * (k.P1 + v.P1);
+  p.a.E1 = p.e1.E;
+  p.a.A2 = 0.5 * (k.P2 + v.P2);
+  p.a.E2 = p.e2.E;
+  p.a.z1a = 0.5 * (k.q + v.q);
+  p.a.pa = 0.5 * (k.p + v.p);
+  p.a.ke = 0.0;
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    p.a.qV[i] = 0.5 * (k.q * k.V[i] + v.q * v.V[i]);
+    p.a.Va[i] = 0.5 * (k.V[i] + v.V[i]);
+    p.a.ke += 0.5 * k.V[i] * v.V[i];
+  }
+  p.iA1 = rcp64(p.a.A1);
+  p.iE1 = rcp64(p.a.E1);
+  p.iE2 = rcp64(p.a.E2);
+  p.iz = rcp64(p.a.z1a);
 }
 
 // Adjoints of the nodal quantities of both sides (ZNode fields) for
@@ -125,21 +121,19 @@ __device__ __forceinline__ void exp_avg_rev(double a, double b, double ar, doubl
 // column adjoints (|nu|/2) l_k ((r_k.dw) gb + (r_k.gb) dw), weight adjoints
 // (|nu|/2) (r_k.gb)(r_k.dw).
 template <int D, typename C>
-__device__ __forceinline__ void pair_reverse(const ZNode<double, D>& k, const ZNode<double, D>& v, const C& c,
-                                             const double* nu, int dissipation, double b, const double* n,
+__device__ __forceinline__ void pair_reverse(const ZNode<double, D>& k, const ZNode<double, D>& v,
+                                             const PairRev<D>& pr, const C& c, const double* nu, int dissipation, double b, const double* n,
                                              const double* gb, const double* dw, ZNode<double, D>& kb,
                                              ZNode<double, D>& vb) {
   constexpr int NC = D + 2;
-  // ---- forward (values)
-  PairAvg<double, D> a;
-  pair_avg<double, D>(k, v, c, a);
+  const PairAvg<double, D>& a = pr.a;
+  const double iden = pr.iA1 * pr.iE1;  // 1/(A1 E1)
   double A1b = 0.0, E1b = 0.0, A2b = 0.0, E2b = 0.0, z1ab = 0.0, pab = 0.0, keb = 0.0;
   double qVb[D], Vab[D];
 #pragma unroll
   for (int i = 0; i < D; ++i) qVb[i] = Vab[i] = 0.0;
   // ---- two-point flux: s_f = mn C + pa (gb_m . nu)
   {
-    const double den = a.A1 * a.E1, iden = 1.0 / den;
     double mq = 0.0;
 #pragma unroll
     for (int i = 0; i < D; ++i) mq += nu[i] * a.qV[i];
@@ -158,16 +152,15 @@ __device__ __forceinline__ void pair_reverse(const ZNode<double, D>& k, const ZN
     const double mqb = mnb * iden, idenb = mnb * mq;
 #pragma unroll
     for (int i = 0; i < D; ++i) qVb[i] += mqb * nu[i];
-    A1b -= idenb * iden * iden * a.E1;
-    E1b -= idenb * iden * iden * a.A1;
+    A1b -= idenb * iden * pr.iA1;
+    E1b -= idenb * iden * pr.iE1;
     A2b += hb * c.gam_gm1 * a.E2;
     E2b += hb * c.gam_gm1 * a.A2;
     keb += hb;
   }
   // ---- dissipation's averages part
   if (dissipation) {
-    const double rho_h = a.z1a / (a.A1 * a.E1);
-    const double iz = 1.0 / a.z1a;
+    const double iz = pr.iz, rho_h = a.z1a * iden, irho = a.A1 * a.E1 * iz;
     double Vh[D], vh2 = 0.0, vn = 0.0;
 #pragma unroll
     for (int i = 0; i < D; ++i) {
@@ -176,9 +169,10 @@ __device__ __forceinline__ void pair_reverse(const ZNode<double, D>& k, const ZN
       vn += Vh[i] * n[i];
     }
     const double p_h = a.pa;
-    const double theta = rho_h / (p_h * a.A1 * a.E1);
-    const double eta = 1.0 / (a.z1a * a.E2 * a.E1);
-    const double ah = sqrt(c.gam * p_h / rho_h);
+    const double ip_h = rcp64(p_h);
+    const double theta = rho_h * iden * ip_h;
+    const double eta = iz * pr.iE2 * pr.iE1;
+    const double a2 = c.gam * p_h * irho, ah = a2 * rsqrt64(a2);
     const double Hh = ah * ah * c.inv_gm1 + 0.5 * vh2;
     double Vhb[D];
 #pragma unroll
@@ -265,23 +259,20 @@ __device__ __forceinline__ void pair_reverse(const ZNode<double, D>& k, const ZN
     vh2b += 0.5 * Hhb;
 #pragma unroll
     for (int i = 0; i < D; ++i) Vhb[i] += 2.0 * vh2b * Vh[i] + vnb * n[i];
-    double p_hb = ahb * ah / (2.0 * p_h);
-    double rho_hb = -ahb * ah / (2.0 * rho_h);
-    z1ab -= etab * eta / a.z1a;
-    E2b -= etab * eta / a.E2;
-    E1b -= etab * eta / a.E1;
-    rho_hb += thetab * theta / rho_h;
-    p_hb -= thetab * theta / p_h;
-    A1b -= thetab * theta / a.A1;
-    E1b -= thetab * theta / a.E1;
+    const double ah2 = 0.5 * ahb * ah, et = etab * eta, th = thetab * theta;
+    const double p_hb = (ah2 - th) * ip_h;
+    const double rho_hb = (th - ah2) * irho;
+    const double rr = th + rho_hb * rho_h;
+    z1ab -= et * iz;
+    E2b -= et * pr.iE2;
+    E1b -= (et + rr) * pr.iE1;
+    A1b -= rr * pr.iA1;
 #pragma unroll
     for (int i = 0; i < D; ++i) {
       qVb[i] += Vhb[i] * iz;
       z1ab -= Vhb[i] * Vh[i] * iz;
     }
-    z1ab += rho_hb * rho_h / a.z1a;
-    A1b -= rho_hb * rho_h / a.A1;
-    E1b -= rho_hb * rho_h / a.E1;
+    z1ab += rho_hb * iden;
     pab += p_hb;
   }
   // ---- pair averages back to the nodal quantities
@@ -307,8 +298,16 @@ __device__ __forceinline__ void pair_reverse(const ZNode<double, D>& k, const ZN
     kb.q += 0.5 * qVb[i] * k.V[i];
     vb.q += 0.5 * qVb[i] * v.V[i];
   }
-  exp_avg_rev(k.p, v.p, k.P2, v.P2, c.r2, k.ip, c.ser2, E1b, kb.p, vb.p, kb.P2, vb.P2, kb.ip);
-  exp_avg_rev(k.q, v.q, k.P1, v.P1, c.r1, k.iq, c.ser1, E2b, kb.q, vb.q, kb.P1, vb.P1, kb.iq);
+  kb.p += E1b * pr.e1.Ea;
+  vb.p += E1b * pr.e1.Eb;
+  kb.P2 += E1b * pr.e1.Ear;
+  vb.P2 += E1b * pr.e1.Ebr;
+  kb.ip += E1b * pr.e1.Eia;
+  kb.q += E2b * pr.e2.Ea;
+  vb.q += E2b * pr.e2.Eb;
+  kb.P1 += E2b * pr.e2.Ear;
+  vb.P1 += E2b * pr.e2.Ebr;
+  kb.iq += E2b * pr.e2.Eia;
 }
 
 // Reverse of the nodal chain u -> (q, V, p, P1, P2, v2, 1/q, 1/p) at the
@@ -317,9 +316,9 @@ __device__ __forceinline__ void pair_reverse(const ZNode<double, D>& k, const ZN
 //   P1 = q^r1, P2 = p^r2.
 template <int D, typename C>
 __device__ __forceinline__ void node_chain_rev(const Node<double, D>& n, const ZNode<double, D>& z,
-                                               const ZNode<double, D>& zb, const C& c, double* ub) {
+                                               const ZNode<double, D>& zb, const C& c, double iq, double ip,
+                                               double* ub) {
   constexpr int NC = D + 2;
-  const double iq = 1.0 / n.q, ip = 1.0 / n.p;
   const double qb = zb.q + zb.P1 * c.r1 * z.P1 * iq - zb.iq * iq * iq;
   const double pb = zb.p + zb.P2 * c.r2 * z.P2 * ip - zb.ip * ip * ip + qb * n.q * c.b_q * ip;
   double rhob = qb * n.q * c.a_q * n.ir - 0.5 * c.gm1 * n.v2 * pb;
@@ -341,7 +340,9 @@ __device__ __forceinline__ void node_chain_rev(const Node<double, D>& n, const Z
 template <int D>
 __global__ void __launch_bounds__(64) face_vjp_kernel(const double* __restrict__ u, const double* __restrict__ cot,
                                                       const int2* __restrict__ fp, int n_pairs,
-                                                      const double* __restrict__ nu, const double* __restrict__ J,
+                                                      const double* __restrict__ nu,
+                                                      const double* __restrict__ ihd,
+                                                      const double* __restrict__ nscale,
                                                       double* __restrict__ gsat, Phys<double> c, int dissipation) {
   constexpr int NC = D + 2;
   int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -363,20 +364,19 @@ __global__ void __launch_bounds__(64) face_vjp_kernel(const double* __restrict__
   ZNode<double, D> zk, zv;
   znode<double, D>(nk, c, zk);
   znode<double, D>(nv, c, zv);
-  znode_recips<double, D>(zk);
-  double nud[D];
-  double b2 = 0.0;
+  const JvpPrep<double> jk = jvp_prep<double, D>(nk, c), jv = jvp_prep<double, D>(nv, c);
+  const double ipk = jk.itheta * jk.ir, ipv = jv.itheta * jv.ir;
+  zk.iq = jk.iq;
+  zk.ip = ipk;
+  double nud[D], nh[D];
+  const double* ns = nscale + (size_t)pr.x * (D + 1);  // |nu|, nu/|nu| of slot (k, s)
+  const double b = __ldg(&ns[0]);
 #pragma unroll
   for (int i = 0; i < D; ++i) {
     nud[i] = __ldg(&nu[((size_t)k * NS + s) * D + i]);
-    b2 += nud[i] * nud[i];
+    nh[i] = __ldg(&ns[1 + i]);
   }
-  const double b = sqrt(b2);
-  double nh[D];
-#pragma unroll
-  for (int i = 0; i < D; ++i) nh[i] = nud[i] / b;
-  double ihk = 1.0 / (c_ref.H[m] * __ldg(&J[(size_t)k * NP + m]));
-  double ihv = 1.0 / (c_ref.H[n] * __ldg(&J[(size_t)v * NP + n]));
+  const double ihk = __ldg(&ihd[(size_t)k * NP + m]), ihv = __ldg(&ihd[(size_t)v * NP + n]);
   double gb[NC], dw[NC];
 #pragma unroll
   for (int q = 0; q < NC; ++q) {
@@ -387,21 +387,32 @@ __global__ void __launch_bounds__(64) face_vjp_kernel(const double* __restrict__
   // each side's nodal chain; with dissipation also (M gb) . (dw_k - dw_v),
   // M = X^|L|S^X^T symmetric, through the symmetric dW/du of each side
   ZNode<double, D> kb, vb;
-  pair_reverse<D>(zk, zv, c, nud, dissipation, b, nh, gb, dw, kb, vb);
+  PairRev<D> pv;
+  pair_rev_prep<D>(zk, zv, c, pv);
+  pair_reverse<D>(zk, zv, pv, c, nud, dissipation, b, nh, gb, dw, kb, vb);
   double gk[NC], gv[NC];
-  node_chain_rev<D>(nk, zk, kb, c, gk);
-  node_chain_rev<D>(nv, zv, vb, c, gv);
+  node_chain_rev<D>(nk, zk, kb, c, jk.iq, ipk, gk);
+  node_chain_rev<D>(nv, zv, vb, c, jv.iq, ipv, gv);
   if (dissipation) {
-    PairAvg<double, D> ar;
-    pair_avg<double, D>(zk, zv, c, ar);
+    PairSums<D> ps;
+    ps.dn = 2.0 * pv.a.A1 * pv.a.E1;
+    ps.idn = 0.5 * pv.iA1 * pv.iE1;
+    ps.E1 = pv.a.E1;
+    ps.E2 = pv.a.E2;
+    ps.Sq = 2.0 * pv.a.z1a;
+    ps.Sp = 2.0 * pv.a.pa;
+#pragma unroll
+    for (int i = 0; i < D; ++i) ps.SqV[i] = 2.0 * pv.a.qV[i];
     double Mgb[NC], wk[NC], wv[NC];
-    diss_apply_cols<double, double, double, D>(ar, c, nh, gb, Mgb);
-    dW_dU_apply<double, D>(nk, jvp_prep<double, D>(nk, c), c, Mgb, wk);
-    dW_dU_apply<double, D>(nv, jvp_prep<double, D>(nv, c), c, Mgb, wv);
+#pragma unroll
+    for (int q = 0; q < NC; ++q) Mgb[q] = 0.0;
+    diss_add2<D>(ps, c, nh, gb, 0.5 * b, Mgb);  // (|nu|/2) M gb
+    dW_dU_apply<double, D>(nk, jk, c, Mgb, wk);
+    dW_dU_apply<double, D>(nv, jv, c, Mgb, wv);
 #pragma unroll
     for (int cc = 0; cc < NC; ++cc) {
-      gk[cc] += 0.5 * b * wk[cc];
-      gv[cc] -= 0.5 * b * wv[cc];
+      gk[cc] += wk[cc];
+      gv[cc] -= wv[cc];
     }
   }
 #pragma unroll
@@ -668,8 +679,8 @@ static int vjp_np(esplit_ctx* c, const double* u, const double* cot, double* gra
     int bs = 64;
     int nb = (c->n_pairs + bs - 1) / bs;
     ProfScope ps(c, PG_FACE, s);
-    face_vjp_kernel<D><<<nb, bs, 0, s>>>(u, cot, c->b.face_pairs, c->n_pairs, c->b.nu, c->b.J, c->b.sat, ph,
-                                         c->prm.dissipation);
+    face_vjp_kernel<D><<<nb, bs, 0, s>>>(u, cot, c->b.face_pairs, c->n_pairs, c->b.nu, c->b.ihd, c->b.nscale,
+                                         c->b.sat, ph, c->prm.dissipation);
     c->launches++;
   }
   {
