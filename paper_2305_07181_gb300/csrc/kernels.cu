@@ -736,14 +736,36 @@ __global__ void __launch_bounds__(round32(EB * NP), SplitCfg<D, NP, EB, VISC>::B
 #pragma unroll
       for (int q = 0; q < NC; ++q) fvals[i * NC + q] = active ? Fp[i][q] : 0.0;
     __syncthreads();  // every thread has read the first contraction's results
-    // the rows keep the first contraction's stride: their padding is still zero
-    tc::digitize<SV, NP, EB, THREADS>(fvals, el < EB, el, m, reinterpret_cast<unsigned*>(resb), ex, dig);
-    __syncthreads();
-    tc::contract<SV, D, NP, EB, NC, 0, THREADS>(dig, ex, elems, opsP, opsE, resb);
-    __syncthreads();
-    if (active) {
+    if constexpr (Cfg::TENSOR) {
+      // the rows keep the first contraction's stride: their padding is still zero
+      tc::digitize<SV, NP, EB, THREADS>(fvals, el < EB, el, m, reinterpret_cast<unsigned*>(resb), ex, dig);
+      __syncthreads();
+      tc::contract<SV, D, NP, EB, NC, 0, THREADS>(dig, ex, elems, opsP, opsE, resb);
+      __syncthreads();
+      if (active) {
 #pragma unroll
-      for (int q = 0; q < NC; ++q) res[q] += resb[((size_t)el * SV::OUTS + q) * SV::NPO + m];
+        for (int q = 0; q < NC; ++q) res[q] += resb[((size_t)el * SV::OUTS + q) * SV::NPO + m];
+      }
+    } else {
+      double* sv = reinterpret_cast<double*>(split_smem);  // [EB][D NC][NP]
+      if (active) {
+#pragma unroll
+        for (int q = 0; q < D * NC; ++q) sv[(el * D * NC + q) * NP + m] = fvals[q];
+      }
+      __syncthreads();
+      if (active) {
+        const double* op = ops64 + (size_t)e * (D * NP * NP);
+#pragma unroll
+        for (int i = 0; i < D; ++i)
+#pragma unroll
+          for (int n = 0; n < NP; ++n) {
+            const double dt = __ldg(&op[(i * NP + n) * NP + m]);
+#pragma unroll
+            for (int q = 0; q < NC; ++q) res[q] += dt * sv[(el * D * NC + i * NC + q) * NP + n];
+          }
+      }
+    }
+    if (active) {
       if (sl >= 0) {
         const double ih = 1.0 / Hm;
         double nv[D];
