@@ -3,7 +3,7 @@ exponential in imath.cuh, computed with 60-digit decimal arithmetic.
 
   log:  for the 256 intervals of [1, 2), centre c_j = 1 + (j + 1/2)/256:
         r_j = 2^14 / c_j rounded to an integer, and -ln(r_j / 2^14) as an
-        integer multiple of 2^-57 (the entry of the exact r_j, not of c_j);
+        integer multiple of 2^-62 (the entry of the exact r_j, not of c_j);
   exp:  2^(j/512), j = 0..511, as an integer multiple of 2^-62;
   ln 2 and ln 2 / 512 as integers of 2^-57 with the rest in units of 2^-89.
 
@@ -36,6 +36,7 @@ def render() -> str:
 
     split("LN2", ln2)
     split("LN2_512", ln2 / 512)
+    out.append(f"constexpr long long LN2_62 = {fixed(ln2, 62)}LL;  // multiples of 2^-62")
     out.append(f"constexpr int INV_LN2_512 = {fixed(512 / ln2, 20)};  // 512 / ln 2, multiples of 2^-20")
 
     def arr(kind, name, vals, suffix, per):
@@ -47,7 +48,7 @@ def render() -> str:
     r = [int((Decimal(2 ** 14) / (1 + (Decimal(j) + Decimal("0.5")) / 256)).to_integral_value(ROUND_HALF_EVEN))
          for j in range(256)]
     arr("unsigned short", "LOG_R", r, "", 16)
-    arr("long long", "LOG_T", [fixed(-(Decimal(v) / 2 ** 14).ln(), 57) for v in r], "LL", 4)
+    arr("long long", "LOG_T", [fixed(-(Decimal(v) / 2 ** 14).ln(), 62) for v in r], "LL", 4)
     arr("unsigned long long", "EXP_T", [fixed((Decimal(j) / 512 * ln2).exp(), 62) for j in range(512)], "ULL", 4)
     out += ["", "}  // namespace im", "}  // namespace esplit", ""]
     return "\n".join(out)

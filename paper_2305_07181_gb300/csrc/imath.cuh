@@ -14,7 +14,7 @@
 //         product modulo 2^64), |z| < 2^-8.9;
 //         ln x = k ln 2 + T_j + z - z^2 (1/2 - z/3) - z^4 (1/4 - z/5 + z^2/6),
 //         T_j = -ln(r_j / 2^14) tabulated; the last term, below 2^-37, in
-//         float32.
+//         float32.  log_fixed62 the same in units of 2^-62 near 1.
 //   exp:  X = N ln2/512 + r, |r| < 2^-10.5, N = 512 K + j;
 //         exp X = 2^K 2^(j/512) (1 + r + r^2/2 + r^3/6 (1 + r/4 + r^2/20)),
 //         the cubic term, below 2^-34, in float32.
@@ -84,7 +84,25 @@ IM_FN bool log_fixed(double x, long long& L) {
   const float zf = __int2float_rn((int)(a >> 32)) * 0x1p-39f, z2 = zf * zf;
   const int t = __float2int_rn(z2 * z2 * (0.25f + zf * (zf * 0.16666667f - 0.2f)) * 0x1p+57f);
   const long long kl = (long long)k * LN2_HI + (((long long)k * LN2_LO) >> 32);
-  L = kl + IM_LOAD(&LOG_T[j]) + ((z + 256) >> 9) - ((s + (1LL << 18)) >> 19) - t;
+  L = kl + ((IM_LOAD(&LOG_T[j]) + 16) >> 5) + ((z + 256) >> 9) - ((s + (1LL << 18)) >> 19) - t;
+  return true;
+}
+
+// ln x in units of 2^-62 for x in [1/4, 4): absolute error below 2^-59
+IM_FN bool log_fixed62(double x, long long& L) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int k = (int)(b >> 52) - 1023;
+  if ((unsigned)(k + 2) >= 4u) return false;
+  const int j = (int)(b >> 44) & 255;
+  const unsigned long long M = (b & 0xFFFFFFFFFFFFFULL) | 0x10000000000000ULL;
+  const long long z = (long long)(M * (unsigned long long)IM_LOAD(&LOG_R[j]));
+  const long long a = (long long)((unsigned long long)z << 5);
+  const long long h = __mul64hi(a, a);
+  const long long w = (1LL << 61) - __mul64hi(a, 0x2AAAAAAAAAAAABLL);
+  const long long s = __mul64hi(h, w);
+  const float zf = __int2float_rn((int)(a >> 32)) * 0x1p-39f, z2 = zf * zf;
+  const int t = __float2int_rn(z2 * z2 * (0.25f + zf * (zf * 0.16666667f - 0.2f)) * 0x1p+62f);
+  L = (long long)k * LN2_62 + IM_LOAD(&LOG_T[j]) + ((z + 8) >> 4) - ((s + (1LL << 13)) >> 14) - t;
   return true;
 }
 
@@ -163,13 +181,14 @@ IM_FN double expm1_tail(double x) {
   return unit62_to_double(s);
 }
 
-// X 2^-57 as a float64, rounded to nearest (ties away from zero)
+// X 2^-unit as a float64, rounded to nearest (ties away from zero)
+template <int UNIT_ = UNIT>
 IM_FN double to_double(long long X) {
   const unsigned long long u = (unsigned long long)(X < 0 ? -X : X);
   const int lz = __clzll((long long)u);
   const unsigned long long n = u << (lz & 63);
   const unsigned long long m = (n >> 11) + ((n >> 10) & 1ULL);
-  const unsigned long long b = u ? m + ((unsigned long long)(1023 + 63 - UNIT - lz - 1) << 52) : 0ULL;
+  const unsigned long long b = u ? m + ((unsigned long long)(1023 + 63 - UNIT_ - lz - 1) << 52) : 0ULL;
   return __longlong_as_double((long long)(b | (X < 0 ? 0x8000000000000000ULL : 0ULL)));
 }
 

@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(128) face_kernel(const double* __restrict__ u,
     ir_node<T, D>(nk, ik);
     ir_node<T, D>(nv, iv);
     IRAvg<T, D> a;
-    ir_avg<T, D>(ik, iv, c, a);
+    ir_avg_t<T, D>(ik, iv, c, a);
     ir_flux_dir<T, D>(a, c, nuv, G);
     if (dissipation) {
       const double* ns = nscale + (size_t)pr.x * (D + 1);  // |nu|, nu/|nu| of slot (k, s)
@@ -437,7 +437,7 @@ __global__ void __launch_bounds__(128) face_bc_kernel(const double* __restrict__
       ir_node<double, D>(nk, ik);
       ir_node<double, D>(nb, ib);
       IRAvg<double, D> av;
-      ir_avg<double, D>(ik, ib, c, av);
+      ir_avg_t<double, D>(ik, ib, c, av);
       ir_flux_dir<double, D>(av, c, nuv, G);
       if (dissipation) {
         double wk[NC], wb[NC];
@@ -889,7 +889,7 @@ __global__ void __launch_bounds__(EB * NP) hadamard_volume_kernel(
   const T* zz = sz + el * NZ * NP;
   ZNode<T, D> zm;
   IRNode<T, D> im;
-  T iHm = T(0), Hm = T(0);
+  T iHm = T(0), Hf = T(0);
   if (active) {
     if constexpr (FLUX == 1) {
       im.z1 = zz[m];
@@ -910,7 +910,8 @@ __global__ void __launch_bounds__(EB * NP) hadamard_volume_kernel(
       zm.ip = zz[(D + 6) * NP + m];
     }
     iHm = sH[el * NP + m];
-    Hm = T(1) / iHm;
+    // G is twice the two-point flux: sy_flux2 doubles by itself
+    Hf = (FLUX == 0 && sizeof(T) == sizeof(double) ? T(1) : T(2)) / iHm;
   }
   const T* op = ops + (size_t)e * (D * NP * NP);
   T* gout = sg + ((size_t)el * NP + m) * KC * NC;
@@ -926,7 +927,7 @@ __global__ void __launch_bounds__(EB * NP) hadamard_volume_kernel(
         if (n >= NP) n -= NP;
         T Smn[D];
 #pragma unroll
-        for (int i = 0; i < D; ++i) Smn[i] = Hm * __ldg(&op[(i * NP + n) * NP + m]);
+        for (int i = 0; i < D; ++i) Smn[i] = Hf * __ldg(&op[(i * NP + n) * NP + m]);
         T G[NC];
         if constexpr (FLUX == 1) {
           IRNode<T, D> in_;
@@ -937,7 +938,7 @@ __global__ void __launch_bounds__(EB * NP) hadamard_volume_kernel(
 #pragma unroll
           for (int i = 0; i < D; ++i) in_.V[i] = zz[(4 + i) * NP + n];
           IRAvg<T, D> ia;
-          ir_avg<T, D>(im, in_, c, ia);
+          ir_avg_t<T, D>(im, in_, c, ia);
           ir_flux_dir<T, D>(ia, c, Smn, G);
         } else {
           ZNode<T, D> zn;
@@ -962,13 +963,7 @@ __global__ void __launch_bounds__(EB * NP) hadamard_volume_kernel(
             PairAvg<T, D> a;
             pair_avg<T, D>(zm, zn, c, a);
             sy_flux_dir<T, D>(a, c, Smn, G);
-#pragma unroll
-            for (int q = 0; q < NC; ++q) G[q] *= T(2);
           }
-        }
-        if constexpr (FLUX == 1) {
-#pragma unroll
-          for (int q = 0; q < NC; ++q) G[q] *= T(2);
         }
 #pragma unroll
         for (int q = 0; q < NC; ++q) {  // G: twice the two-point flux
