@@ -88,7 +88,9 @@ int opsD_stride_for(int d, int np) {
 }
 
 int ensure_partial(esplit_ctx* c) {
-  size_t need = 8 * ((size_t)c->n_e * c->n_p / 256 + 1) + 4 * ((size_t)c->n_e + 64);
+  // two values per block of the entropy (at most a block per element), then
+  // four stages of up to a block per element and 128 facet pairs
+  size_t need = 8 * ((size_t)c->n_e * c->n_p / 256 + 1) + 8 * ((size_t)c->n_e + 64);
   if (c->partial_cap >= need) return ESPLIT_OK;
   int rc = dalloc(c, &c->b.partial, need);
   if (rc) return rc;

@@ -11,6 +11,7 @@
 namespace esplit {
 
 constexpr int MAX_NP = 80;
+constexpr int SMALL_BLOCKS = 4 * 152;  // short blocks up to four per SM (152 SMs), see split_cached_launch
 
 // row length of the float32 path's staged operators: the smallest multiple of
 // 4 (one 16-byte load) not below n_p whose number of 16-byte chunks is odd, so

@@ -534,11 +534,11 @@ int launch_face_bc(esplit_ctx* c, const double* u, double* out, int add, double*
 // triangles: float64 FMA loops, too short for the tiles.
 // Optional: block partial of sum H w^T r (entropy production, float64).
 // ---------------------------------------------------------------------------
-template <int D, int NP, int EB, bool VISC>
+template <int D, int NP, int EB, bool VISC, int TH = round32(EB * NP)>
 struct SplitCfg {
   static constexpr bool TENSOR = D >= 2 && NP > 8;
   static constexpr int NC = D + 2;
-  static constexpr int THREADS = round32(EB * NP);
+  static constexpr int THREADS = TH;
   using S = tc::Shape<D, NP, EB, NC, NC>;  // f_i summed over i, w per direction
   using SV = tc::Shape<D, NP, EB, NC, 0>;  // F^V_i + a_i/(2H), summed over i
   static constexpr size_t SMEM =
@@ -552,7 +552,8 @@ struct SplitCfg {
   // triangles), 58 nodes 3 -> 4 blocks 170 -> 160 us (3,072 tetrahedra).
   static constexpr int BY_SMEM = (int)(233472 / (SMEM + 2048));  // 228 KB per SM; block sums and 1 KB reserved per block
   static constexpr int BY_REGS = (TENSOR && D == 2 && !VISC ? 768 : D == 2 && !VISC ? 640 : 512) / THREADS;
-  static constexpr int BLOCKS = BY_SMEM < BY_REGS ? BY_SMEM : BY_REGS;
+  // short blocks (small meshes, at most a few per SM): no register pressure
+  static constexpr int BLOCKS = EB * NP <= 32 || EB == 1 ? 2 : BY_SMEM < BY_REGS ? BY_SMEM : BY_REGS;
 };
 
 // The state of a Runge-Kutta stage formed where the volume kernels load it:
@@ -570,8 +571,8 @@ __device__ __forceinline__ void stage_state(const StageIn& st, const double* r, 
   }
 }
 
-template <int D, int NP, int EB, bool VISC, bool CACHE = false, bool ENT = false>
-__global__ void __launch_bounds__(round32(EB * NP), SplitCfg<D, NP, EB, VISC>::BLOCKS) split_volume_kernel(
+template <int D, int NP, int EB, bool VISC, bool CACHE = false, bool ENT = false, int TH = round32(EB * NP)>
+__global__ void __launch_bounds__(TH, SplitCfg<D, NP, EB, VISC, TH>::BLOCKS) split_volume_kernel(
     const double* __restrict__ u, double* __restrict__ r, const double* __restrict__ ops64,
     const uint4* __restrict__ opsP, const short* __restrict__ opsE, const double* __restrict__ J,
     const double* __restrict__ sat, const int* __restrict__ list, int n_list, Phys<double> c64,
@@ -580,7 +581,7 @@ __global__ void __launch_bounds__(round32(EB * NP), SplitCfg<D, NP, EB, VISC>::B
     StageIn st, double* __restrict__ ent_part = nullptr, double* __restrict__ ncache = nullptr,
     double* __restrict__ wsl = nullptr) {
   constexpr int NC = D + 2;
-  using Cfg = SplitCfg<D, NP, EB, VISC>;
+  using Cfg = SplitCfg<D, NP, EB, VISC, TH>;
   using S = typename Cfg::S;
   constexpr int THREADS = Cfg::THREADS;
   extern __shared__ __align__(16) unsigned char split_smem[];
@@ -1038,11 +1039,12 @@ struct VolCfg {
   static constexpr int HAD_KC = NP > 32 ? 8 : NP / 2;
 };
 
-template <int D, int NP, int EB, bool VISC, bool CACHE, bool ENT>
-static void split_launch(esplit_ctx* c, const double* u, double* r, const double* sat, const int* list, int n_list,
-                         int nb, double* prod, double* ent_part, cudaStream_t s) {
-  using Cfg = SplitCfg<D, NP, EB, VISC>;
-  auto* kern = split_volume_kernel<D, NP, EB, VISC, CACHE, ENT>;
+template <int D, int NP, int EB, bool VISC, bool CACHE, bool ENT, int TH = round32(EB * NP)>
+static int split_launch(esplit_ctx* c, const double* u, double* r, const double* sat, const int* list, int n_list,
+                        double* prod, double* ent_part, cudaStream_t s) {
+  using Cfg = SplitCfg<D, NP, EB, VISC, TH>;
+  auto* kern = split_volume_kernel<D, NP, EB, VISC, CACHE, ENT, TH>;
+  const int nb = (n_list + EB - 1) / EB;
   static bool attr_set = false;
   if (!attr_set) {
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
@@ -1055,6 +1057,28 @@ static void split_launch(esplit_ctx* c, const double* u, double* r, const double
                                            VISC ? c->b.va : nullptr, VISC ? c->b.fv : nullptr,
                                            CACHE ? c->b.fcache : nullptr, c->n_e * c->n_slot, c->stage, ent_part,
                                            ENT ? c->b.node_cache : nullptr, VISC && prod ? c->b.wslot : nullptr);
+  return nb;
+}
+
+// The inviscid volume kernel with facet cache for a list of any length.  On
+// small meshes the length of one block's chain decides, not throughput: blocks
+// of as many elements as fill one warp, with the contraction's (element, row
+// tile) tasks spread over up to four warps, while at most four such blocks
+// fall on an SM.  Measured, residual with short and with full blocks:
+// triangles p 3, 512 elements 25.5 and 33.0 us, 968 elements 35.0 and 33.0;
+// tetrahedra p 2, 384 elements 33.0 and 45.3.
+template <int D, int NP, int EB, bool ENT>
+static int split_cached_launch(esplit_ctx* c, const double* u, double* r, const double* sat, const int* list,
+                               int n_list, double* prod, double* ent_part, cudaStream_t s) {
+  if constexpr (D >= 2) {
+    constexpr int EBS = NP < 32 ? 32 / NP : 1;
+    constexpr int TASKS = EBS * ((NP + 7) / 8);
+    constexpr int MIN = round32(EBS * NP), BY_TASKS = 32 * (TASKS < 4 ? TASKS : 4);
+    constexpr int THS = SplitCfg<D, NP, EB, false>::TENSOR && BY_TASKS > MIN ? BY_TASKS : MIN;
+    if ((n_list + EBS - 1) / EBS <= SMALL_BLOCKS)
+      return split_launch<D, NP, EBS, false, true, ENT, THS>(c, u, r, sat, list, n_list, prod, ent_part, s);
+  }
+  return split_launch<D, NP, EB, false, true, ENT>(c, u, r, sat, list, n_list, prod, ent_part, s);
 }
 
 template <typename T, int D, int NP>
@@ -1112,22 +1136,22 @@ static int residual_np(esplit_ctx* c, const double* u, double* r, cudaStream_t s
   const int* lhad = scheme == ESPLIT_SCHEME_HYBRID ? c->b.list_had : nullptr;
   if (n_split > 0) {
     constexpr int EB = VolCfg<NP>::EB_SPLIT;
-    int nb = (n_split + EB - 1) / EB;
+    int nb;
     ProfScope ps(c, PG_SPLIT, s);
     double* pp = prod ? prod + np_used : nullptr;
     if (visc && c->ent_part && c->b.node_cache) {
       // first stage of a relaxation step: the kernel also forms the entropy of u_n
-      split_launch<D, NP, EB, true, false, true>(c, u, r, sat, lsplit, n_split, nb, pp, c->ent_part, s);
+      nb = split_launch<D, NP, EB, true, false, true>(c, u, r, sat, lsplit, n_split, pp, c->ent_part, s);
       c->ent_n = nb;
     } else if (visc)
-      split_launch<D, NP, EB, true, false, false>(c, u, r, sat, lsplit, n_split, nb, pp, nullptr, s);
+      nb = split_launch<D, NP, EB, true, false, false>(c, u, r, sat, lsplit, n_split, pp, nullptr, s);
     else if (cached && scheme == ESPLIT_SCHEME_SPLIT && c->ent_part && c->b.node_cache) {
-      split_launch<D, NP, EB, false, true, true>(c, u, r, sat, lsplit, n_split, nb, pp, c->ent_part, s);
+      nb = split_cached_launch<D, NP, EB, true>(c, u, r, sat, lsplit, n_split, pp, c->ent_part, s);
       c->ent_n = nb;
     } else if (cached)
-      split_launch<D, NP, EB, false, true, false>(c, u, r, sat, lsplit, n_split, nb, pp, nullptr, s);
+      nb = split_cached_launch<D, NP, EB, false>(c, u, r, sat, lsplit, n_split, pp, nullptr, s);
     else
-      split_launch<D, NP, EB, false, false, false>(c, u, r, sat, lsplit, n_split, nb, pp, nullptr, s);
+      nb = split_launch<D, NP, EB, false, false, false>(c, u, r, sat, lsplit, n_split, pp, nullptr, s);
     c->launches++;
     np_used += nb;
   }

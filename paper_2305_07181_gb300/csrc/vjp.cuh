@@ -431,11 +431,11 @@ __global__ void __launch_bounds__(64) face_vjp_kernel(const double* __restrict__
 // volume kernel (tc64.cuh), with 2 n_c columns (w, cot/H) and then n_c
 // summed ones; 7-node triangles keep float64 loops.  On the float64 pipe the
 // pointwise part is left.
-template <int D, int NP, int EB>
+template <int D, int NP, int EB, int TH = round32(EB * NP)>
 struct VjpCfg {
   static constexpr bool TENSOR = NP > 8;
   static constexpr int NC = D + 2;
-  static constexpr int THREADS = round32(EB * NP);
+  static constexpr int THREADS = TH;
   using S1 = tc::Shape<D, NP, EB, 0, 2 * NC>;
   using S2 = tc::Shape<D, NP, EB, NC, 0>;
   static constexpr size_t mx(size_t a, size_t b) { return a > b ? a : b; }
@@ -444,17 +444,17 @@ struct VjpCfg {
   static constexpr size_t SMEM = TENSOR ? DIG + RES + EXB + EB * sizeof(int) : (size_t)EB * D * NC * NP * 8;
   static constexpr int BY_SMEM = (int)(233472 / (SMEM + 1024));
   static constexpr int BY_REGS = (NP > 32 ? 384 : 512) / THREADS;
-  static constexpr int BLOCKS = BY_SMEM < BY_REGS ? BY_SMEM : BY_REGS;
+  static constexpr int BLOCKS = EB * NP <= 32 || EB == 1 ? 2 : BY_SMEM < BY_REGS ? BY_SMEM : BY_REGS;
 };
 
-template <int D, int NP, int EB>
-__global__ void __launch_bounds__(round32(EB * NP), VjpCfg<D, NP, EB>::BLOCKS) split_vjp_kernel(
+template <int D, int NP, int EB, int TH = round32(EB * NP)>
+__global__ void __launch_bounds__(TH, VjpCfg<D, NP, EB, TH>::BLOCKS) split_vjp_kernel(
     const double* __restrict__ u, const double* __restrict__ cot, const double* __restrict__ ops,
     const uint4* __restrict__ opsP, const short* __restrict__ opsE, const double* __restrict__ J,
     const double* __restrict__ ihd, const double* __restrict__ nu, const double* __restrict__ gsat, int n_e,
     double* __restrict__ grad, Phys<double> c) {
   constexpr int NC = D + 2;
-  using Cfg = VjpCfg<D, NP, EB>;
+  using Cfg = VjpCfg<D, NP, EB, TH>;
   using S1 = typename Cfg::S1;
   using S2 = typename Cfg::S2;
   constexpr int THREADS = Cfg::THREADS;
@@ -672,6 +672,21 @@ __global__ void __launch_bounds__(round32(EB * NP), VjpCfg<D, NP, EB>::BLOCKS) s
   }
 }
 
+template <int D, int NP, int EB, int TH>
+static void split_vjp_launch(esplit_ctx* c, const double* u, const double* cot, double* grad, const Phys<double>& ph,
+                             cudaStream_t s) {
+  using Cfg = VjpCfg<D, NP, EB, TH>;
+  auto* kern = split_vjp_kernel<D, NP, EB, TH>;
+  static bool attr_set = false;
+  if (!attr_set) {
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
+    cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    attr_set = true;
+  }
+  kern<<<(c->n_e + EB - 1) / EB, TH, Cfg::SMEM, s>>>(u, cot, c->b.ops64, c->b.opsP, c->b.opsE, c->b.J, c->b.ihd,
+                                                     c->b.nu, c->b.sat, c->n_e, grad, ph);
+}
+
 template <int D, int NP>
 static int vjp_np(esplit_ctx* c, const double* u, const double* cot, double* grad, cudaStream_t s) {
   const Phys<double> ph = make_phys<double>(c->prm.gam, c->prm.beta, c->prm.R, c->prm.mu, c->prm.Pr);
@@ -686,18 +701,14 @@ static int vjp_np(esplit_ctx* c, const double* u, const double* cot, double* gra
   {
     // blocks that fill their warps, as the split volume kernel's
     constexpr int EB = NP == 7 ? 18 : NP == 12 ? 10 : NP == 18 || NP == 27 ? 7 : NP == 25 ? 5 : 2;
-    using Cfg = VjpCfg<D, NP, EB>;
-    int nb = (c->n_e + EB - 1) / EB;
+    constexpr int EBS = NP < 32 ? 32 / NP : 1, TASKS = EBS * ((NP + 7) / 8), MIN = round32(EBS * NP);
+    constexpr int BY_TASKS = 32 * (TASKS < 4 ? TASKS : 4);
+    constexpr int THS = VjpCfg<D, NP, EB>::TENSOR && BY_TASKS > MIN ? BY_TASKS : MIN;
     ProfScope ps(c, PG_SPLIT, s);
-    auto* kern = split_vjp_kernel<D, NP, EB>;
-    static bool attr_set = false;
-    if (!attr_set) {
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
-      cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-      attr_set = true;
-    }
-    kern<<<nb, Cfg::THREADS, Cfg::SMEM, s>>>(u, cot, c->b.ops64, c->b.opsP, c->b.opsE, c->b.J, c->b.ihd, c->b.nu,
-                                             c->b.sat, c->n_e, grad, ph);
+    if ((c->n_e + EBS - 1) / EBS <= SMALL_BLOCKS)  // small meshes: short blocks, as for the split volume kernel
+      split_vjp_launch<D, NP, EBS, THS>(c, u, cot, grad, ph, s);
+    else
+      split_vjp_launch<D, NP, EB, round32(EB * NP)>(c, u, cot, grad, ph, s);
     c->launches++;
   }
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
