@@ -539,8 +539,8 @@ struct SplitCfg {
   static constexpr bool TENSOR = D >= 2 && NP > 8;
   static constexpr int NC = D + 2;
   static constexpr int THREADS = TH;
-  using S = tc::Shape<D, NP, EB, NC, NC>;  // f_i summed over i, w per direction
-  using SV = tc::Shape<D, NP, EB, NC, 0>;  // F^V_i + a_i/(2H), summed over i
+  using S = tc::Shape<D, NP, EB, NC, NC, TH>;  // f_i summed over i, w per direction
+  using SV = tc::Shape<D, NP, EB, NC, 0, TH>;  // F^V_i + a_i/(2H), summed over i
   static constexpr size_t SMEM =
       TENSOR ? S::DIG_BYTES + S::RES_BYTES + S::EX_BYTES + EB * sizeof(int)
              : (size_t)EB * (D + 1) * NC * NP * sizeof(double);
@@ -619,12 +619,11 @@ __global__ void __launch_bounds__(TH, SplitCfg<D, NP, EB, VISC, TH>::BLOCKS) spl
   const int ms = el < EB ? m : 0, els = el < EB ? el : 0;  // in-range slot of the idle lanes
   if constexpr (Cfg::TENSOR) {
     if (m == 0 && el < EB) elems[el] = active ? e : -1;
-    tc::zero_padding<S, NP, EB, THREADS>(dig);
-    tc::digitize<S, NP, EB, THREADS>(vals, el < EB, el, m, reinterpret_cast<unsigned*>(resb), ex, dig);
+    tc::digitize<S, NP, EB, THREADS>(vals, el < EB, el, m, ex, dig);
     __syncthreads();
     tc::contract<S, D, NP, EB, NC, NC, THREADS>(dig, ex, elems, opsP, opsE, resb);
     __syncthreads();
-    const double* rs = resb + (size_t)els * S::OUTS * S::NPO + ms;
+    const double* rs = S::results(dig, resb, els) + ms;
 #pragma unroll
     for (int q = 0; q < NC; ++q) accd[q] = rs[q * S::NPO];
 #pragma unroll
@@ -738,14 +737,13 @@ __global__ void __launch_bounds__(TH, SplitCfg<D, NP, EB, VISC, TH>::BLOCKS) spl
       for (int q = 0; q < NC; ++q) fvals[i * NC + q] = active ? Fp[i][q] : 0.0;
     __syncthreads();  // every thread has read the first contraction's results
     if constexpr (Cfg::TENSOR) {
-      // the rows keep the first contraction's stride: their padding is still zero
-      tc::digitize<SV, NP, EB, THREADS>(fvals, el < EB, el, m, reinterpret_cast<unsigned*>(resb), ex, dig);
+      tc::digitize<SV, NP, EB, THREADS>(fvals, el < EB, el, m, ex, dig);
       __syncthreads();
       tc::contract<SV, D, NP, EB, NC, 0, THREADS>(dig, ex, elems, opsP, opsE, resb);
       __syncthreads();
       if (active) {
 #pragma unroll
-        for (int q = 0; q < NC; ++q) res[q] += resb[((size_t)el * SV::OUTS + q) * SV::NPO + m];
+        for (int q = 0; q < NC; ++q) res[q] += SV::results(dig, resb, el)[q * SV::NPO + m];
       }
     } else {
       double* sv = reinterpret_cast<double*>(split_smem);  // [EB][D NC][NP]

@@ -161,7 +161,7 @@ __device__ __forceinline__ void ldm2(unsigned& r0, unsigned& r1, unsigned addr) 
 // element and direction: NF columns that differ by direction and whose results
 // are summed over the directions (f_i -> sum_i D_i f_i), and NW columns shared
 // by the directions, one result each (w -> D_i w).
-template <int D, int NP, int EB, int NF, int NW>
+template <int D, int NP, int EB, int NF, int NW, int THREADS>
 struct Shape {
   static constexpr int BITS = bits_for(NP);
   static constexpr int KP = (NP + 7) / 8 * 8;          // nodes padded to the tile
@@ -182,10 +182,23 @@ struct Shape {
   // unit of the 64-bit level sums, 2^-UNIT of the digit products' unit: the
   // sum over NP nodes and D directions stays below 2^63
   static constexpr int UNIT = BITS == 10 ? (D == 3 ? 62 : 61) : 51;
-  static constexpr size_t DIG_BYTES = (size_t)EB * 6 * COLS * NPW * 4;
-  static constexpr size_t OUT_BYTES = (size_t)EB * OUTS * NPO * 8;
-  static constexpr size_t HI_BYTES = (size_t)EB * COLS * NPH * 4;
-  static constexpr size_t RES_BYTES = OUT_BYTES > HI_BYTES ? OUT_BYTES : HI_BYTES;
+  static constexpr size_t DIG_EL = (size_t)6 * COLS * NPW * 4, RES_EL = (size_t)OUTS * NPO * 8;  // bytes per element
+  // Where every warp takes the same number of an element's row tiles, the
+  // element's results go over the digits of the element before it (a block
+  // barrier between the elements), the first one's to a region of its own:
+  // 53 instead of 71 KB per block at 25 nodes, four blocks per SM instead of
+  // three (Navier-Stokes kernel, 24,576 tetrahedra: 780 -> 680 us).  Not for
+  // blocks of a few elements, which other limits hold to the same number.
+  static constexpr bool OVER = EB >= 4 && NT % (THREADS / 32) == 0 && RES_EL <= DIG_EL;
+  static constexpr size_t HI_BYTES = (size_t)EB * COLS * NPH * 4;  // the columns' high words, before the digits
+  static constexpr size_t DIG_BYTES = EB * DIG_EL > HI_BYTES ? EB * DIG_EL : (HI_BYTES + 15) / 16 * 16;
+  static constexpr size_t RES_BYTES = OVER ? RES_EL : EB * RES_EL;
+  static __device__ __forceinline__ double* results(void* dig, double* res, int el) {
+    if constexpr (OVER)
+      return el == 0 ? res : reinterpret_cast<double*>(static_cast<unsigned char*>(dig) + (size_t)(el - 1) * DIG_EL);
+    else
+      return res + (size_t)el * OUTS * NPO;
+  }
   static constexpr size_t EX_BYTES = (size_t)(EB * COLS + 3) / 4 * 16;
 };
 
@@ -237,13 +250,14 @@ __device__ __forceinline__ double level_value(long long v, int E) {
   return __longlong_as_double((long long)(bits | ((unsigned long long)sgn << 32)));
 }
 
-// v (COLS values of node m of element el) -> shared digit rows.  Three steps
-// with block barriers between them: high words out, column maxima, digits.
+// v (COLS values of node m of element el) -> shared digit rows, with zero
+// digits for the padding nodes (NP .. KP - 1).  Three steps with block barriers
+// between them: high words out (in the digits' place), column maxima, digits.
 // Every thread of the block calls it; `on`: the thread owns a node.
 template <class S, int NP, int EB, int THREADS>
-__device__ __forceinline__ void digitize(const double (&v)[S::COLS], bool on, int el, int m, unsigned* hiw, int* ex,
-                                         __half* dig) {
+__device__ __forceinline__ void digitize(const double (&v)[S::COLS], bool on, int el, int m, int* ex, __half* dig) {
   constexpr int COLS = S::COLS;
+  unsigned* hiw = reinterpret_cast<unsigned*>(dig);
   if (on) {
 #pragma unroll
     for (int c = 0; c < COLS; ++c)
@@ -257,6 +271,14 @@ __device__ __forceinline__ void digitize(const double (&v)[S::COLS], bool on, in
     ex[j] = exp_of_max(mx);
   }
   __syncthreads();
+  if constexpr (S::KP > NP) {
+    constexpr int W = S::KP - NP;
+    unsigned short* d = reinterpret_cast<unsigned short*>(dig);
+    for (int j = threadIdx.x; j < EB * 6 * COLS * W; j += THREADS) {
+      const int row = j / W, k = j - row * W;
+      d[row * (2 * S::NPW) + NP + k] = 0;
+    }
+  }
   if (on) {
     unsigned short* row = reinterpret_cast<unsigned short*>(dig) + (size_t)el * 6 * COLS * (2 * S::NPW) + m;
     constexpr unsigned MASK = (1u << S::BITS) - 1u;
@@ -274,19 +296,6 @@ __device__ __forceinline__ void digitize(const double (&v)[S::COLS], bool on, in
   }
 }
 
-// zero digits of the padding nodes (NP .. KP - 1) of every row of the block
-template <class S, int NP, int EB, int THREADS>
-__device__ __forceinline__ void zero_padding(__half* dig) {
-  if constexpr (S::KP > NP) {
-    constexpr int W = S::KP - NP;
-    unsigned short* d = reinterpret_cast<unsigned short*>(dig);
-    for (int j = threadIdx.x; j < EB * 6 * S::COLS * W; j += THREADS) {
-      const int row = j / W, k = j - row * W;
-      d[row * (2 * S::NPW) + NP + k] = 0;
-    }
-  }
-}
-
 // asks for bytes [p, p + n) in L2 (p and n multiples of 16): one request of the
 // bulk-copy engine, issued before the pointwise phase whose ~10 us hide it
 __device__ __forceinline__ void prefetch_l2(const void* p, unsigned n) {
@@ -298,7 +307,7 @@ __device__ __forceinline__ void prefetch_l2(const void* p, unsigned n) {
 // Results: res[el][k][m], k < NF the sums over the directions, then
 // NF + i NW + q for column q of direction i.
 template <class S, int D, int NP, int EB, int NF, int NW, int THREADS>
-__device__ __forceinline__ void contract(const __half* dig, const int* ex, const int* elems,
+__device__ __forceinline__ void contract(__half* dig, const int* ex, const int* elems,
                                          const uint4* __restrict__ opsP, const short* __restrict__ opsE, double* res) {
   constexpr int BITS = S::BITS, MB = S::MB, T = S::T, COLS = S::COLS;
   constexpr int PAIRS = pairs_for(NP);
@@ -326,7 +335,8 @@ __device__ __forceinline__ void contract(const __half* dig, const int* ex, const
   for (int task = warp; task < EB * S::NT; task += THREADS / 32) {
     const int el = task / S::NT, nt = task - el * S::NT;
     const int e = elems[el];
-    if (e < 0) continue;             // only behind the last element of the list
+    double* out = S::results(dig, res, el);
+    if (e >= 0) {                    // -1 only behind the last element of the list
     const int mo = nt * 8 + 2 * t4;  // first of the two rows of this lane's results
     long long fs[MB][2];
     int fE[MB][2];
@@ -415,10 +425,17 @@ __device__ __forceinline__ void contract(const __half* dig, const int* ex, const
           }
           if (live && (c >= NF || i == D - 1)) {
             const int k = c < NF ? c : NF + i * NW + (c - NF);
-            res[((size_t)el * S::OUTS + k) * S::NPO + mo + r] = level_value<BITS, S::UNIT>(J, E);
+            out[k * S::NPO + mo + r] = level_value<BITS, S::UNIT>(J, E);
           }
         }
       }
+    }
+    }
+    if constexpr (S::OVER) {
+      // all warps are through with this element's digits before the next
+      // element's results go there (uniform: OVER makes the counts equal)
+      constexpr int PER = S::NT / (THREADS / 32);
+      if ((task / (THREADS / 32) + 1) % PER == 0) __syncthreads();
     }
   }
 }

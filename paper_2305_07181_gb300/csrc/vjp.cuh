@@ -436,8 +436,8 @@ struct VjpCfg {
   static constexpr bool TENSOR = NP > 8;
   static constexpr int NC = D + 2;
   static constexpr int THREADS = TH;
-  using S1 = tc::Shape<D, NP, EB, 0, 2 * NC>;
-  using S2 = tc::Shape<D, NP, EB, NC, 0>;
+  using S1 = tc::Shape<D, NP, EB, 0, 2 * NC, TH>;
+  using S2 = tc::Shape<D, NP, EB, NC, 0, TH>;
   static constexpr size_t mx(size_t a, size_t b) { return a > b ? a : b; }
   static constexpr size_t DIG = mx(S1::DIG_BYTES, S2::DIG_BYTES), RES = mx(S1::RES_BYTES, S2::RES_BYTES);
   static constexpr size_t EXB = mx(S1::EX_BYTES, S2::EX_BYTES);
@@ -458,7 +458,6 @@ __global__ void __launch_bounds__(TH, VjpCfg<D, NP, EB, TH>::BLOCKS) split_vjp_k
   using S1 = typename Cfg::S1;
   using S2 = typename Cfg::S2;
   constexpr int THREADS = Cfg::THREADS;
-  static_assert(!Cfg::TENSOR || S1::NPW == S2::NPW, "one digit row stride: the padding stays zero");
   extern __shared__ __align__(16) unsigned char vjp_smem[];
   const int NS = c_ref.n_slot;
   const int el = threadIdx.x / NP;
@@ -501,13 +500,11 @@ __global__ void __launch_bounds__(TH, VjpCfg<D, NP, EB, TH>::BLOCKS) split_vjp_k
   double g[D][NC], t[D][NC];  // D_i w, D_i (cot/H)
   if constexpr (Cfg::TENSOR) {
     if (m == 0 && slot) elems[el] = active ? e : -1;
-    tc::zero_padding<S1, NP, EB, THREADS>(dig);
-    if constexpr (S2::COLS > S1::COLS) tc::zero_padding<S2, NP, EB, THREADS>(dig);
-    tc::digitize<S1, NP, EB, THREADS>(x1, slot, el, m, reinterpret_cast<unsigned*>(resb), ex, dig);
+    tc::digitize<S1, NP, EB, THREADS>(x1, slot, el, m, ex, dig);
     __syncthreads();
     tc::contract<S1, D, NP, EB, 0, 2 * NC, THREADS>(dig, ex, elems, opsP, opsE, resb);
     __syncthreads();
-    const double* rs = resb + (size_t)els * S1::OUTS * S1::NPO + ms;
+    const double* rs = S1::results(dig, resb, els) + ms;
 #pragma unroll
     for (int i = 0; i < D; ++i)
 #pragma unroll
@@ -557,12 +554,12 @@ __global__ void __launch_bounds__(TH, VjpCfg<D, NP, EB, TH>::BLOCKS) split_vjp_k
   }
   double wb[NC];  // sum_i D_i (gbar_i / H)
   if constexpr (Cfg::TENSOR) {
-    tc::digitize<S2, NP, EB, THREADS>(x2, slot, el, m, reinterpret_cast<unsigned*>(resb), ex, dig);
+    tc::digitize<S2, NP, EB, THREADS>(x2, slot, el, m, ex, dig);
     __syncthreads();
     tc::contract<S2, D, NP, EB, NC, 0, THREADS>(dig, ex, elems, opsP, opsE, resb);
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < NC; ++q) wb[q] = resb[((size_t)els * S2::OUTS + q) * S2::NPO + ms];
+    for (int q = 0; q < NC; ++q) wb[q] = S2::results(dig, resb, els)[q * S2::NPO + ms];
   } else {
     if (active) {
 #pragma unroll
