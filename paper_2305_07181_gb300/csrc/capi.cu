@@ -90,7 +90,8 @@ int opsD_stride_for(int d, int np) {
 int ensure_partial(esplit_ctx* c) {
   // two values per block of the entropy (at most a block per element), then
   // four stages of up to a block per element and 128 facet pairs
-  size_t need = 8 * ((size_t)c->n_e * c->n_p / 256 + 1) + 8 * ((size_t)c->n_e + 64);
+  // (small meshes: up to two blocks per SM of 32 threads and more)
+  size_t need = 8 * ((size_t)c->n_e * c->n_p / 256 + 1) + 8 * ((size_t)c->n_e + 64) + 16384;
   if (c->partial_cap >= need) return ESPLIT_OK;
   int rc = dalloc(c, &c->b.partial, need);
   if (rc) return rc;
@@ -105,13 +106,30 @@ int rebuild_ops(esplit_ctx* c, cudaStream_t s) {
   return ESPLIT_OK;
 }
 
+// the context's small device block: 64 doubles, the root state, the status word
+constexpr size_t kRootOff = 64 * sizeof(double);
+constexpr size_t kStatusOff = kRootOff + (sizeof(esplit::RootState) + 15) / 16 * 16;
+constexpr size_t kStepBytes = kStatusOff + 16;
+
+// copies the block to pinned host memory and waits for it: one round trip
+int read_step(esplit_ctx* c, cudaStream_t s) {
+  CK(cudaMemcpyAsync(c->h_step, c->b.scal, kStepBytes, cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  return ESPLIT_OK;
+}
+
+// the error code of a status word, which is cleared on the device when set
+int status_code(esplit_ctx* c, int h, cudaStream_t s, bool clear) {
+  if (clear && h) CK(cudaMemsetAsync(c->b.status, 0, sizeof(int), s));
+  if (h & 4) return fail(c, ESPLIT_ERR_CUDA, "a kernel's wait for its shared-memory staging timed out");
+  return h ? ESPLIT_ERR_NONPHYSICAL : ESPLIT_OK;
+}
+
 int read_status(esplit_ctx* c, cudaStream_t s, bool clear) {
   int h = 0;
   CK(cudaMemcpyAsync(&h, c->b.status, sizeof(int), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
-  if (clear && h) CK(cudaMemsetAsync(c->b.status, 0, sizeof(int), s));
-  if (h & 4) return fail(c, ESPLIT_ERR_CUDA, "a kernel's wait for its shared-memory staging timed out");
-  return h ? ESPLIT_ERR_NONPHYSICAL : ESPLIT_OK;
+  return status_code(c, h, s, clear);
 }
 
 }  // namespace
@@ -172,14 +190,16 @@ int esplit_create(esplit_ctx** out, int dim, int device) {
   c->prm.heat_flux = 1;
   c->prm.scheme = ESPLIT_SCHEME_SPLIT;
   c->prm.precision = ESPLIT_FP64;
-  if (cudaMalloc((void**)&c->b.status, sizeof(int)) != cudaSuccess ||
-      cudaMalloc((void**)&c->b.root, sizeof(esplit::RootState)) != cudaSuccess ||
-      cudaMalloc((void**)&c->b.scal, 64 * sizeof(double)) != cudaSuccess) {
+  // one allocation, read back by one copy after a step: [scal | root | status]
+  if (cudaMalloc((void**)&c->b.scal, kStepBytes) != cudaSuccess ||
+      cudaMallocHost((void**)&c->h_step, kStepBytes) != cudaSuccess) {
     esplit_destroy(c);
     return ESPLIT_ERR_CUDA;
   }
-  cudaMemset(c->b.status, 0, sizeof(int));
-  cudaMemset(c->b.scal, 0, 64 * sizeof(double));
+  unsigned char* block = reinterpret_cast<unsigned char*>(c->b.scal);
+  c->b.root = reinterpret_cast<esplit::RootState*>(block + kRootOff);
+  c->b.status = reinterpret_cast<int*>(block + kStatusOff);
+  cudaMemset(c->b.scal, 0, kStepBytes);
   *out = c;
   return ESPLIT_OK;
 }
@@ -189,10 +209,11 @@ void esplit_destroy(esplit_ctx* c) {
   cudaSetDevice(c->device);
   esplit::Buffers& b = c->b;
   void* ps[] = {b.Qref, b.J,       b.nu,      b.pair,   b.Lam,     b.face_pairs, b.ops64,   b.ops32,
-                b.list_split, b.list_had, b.hflags, b.hflag0, b.hcount, b.sat, b.fcache, b.partial, b.scal, b.root, b.status, b.stage_u,
+                b.list_split, b.list_had, b.hflags, b.hflag0, b.hcount, b.sat, b.fcache, b.partial, b.scal, b.stage_u,
                 b.stage_r, b.dacc, b.node_cache, b.vjp_work, b.host_u, b.host_r, b.fv, b.vsat, b.va, b.wslot, b.vfb, b.vfs, b.vus,
                 b.bslot, b.bstate, b.ihf, b.opsD32, b.ihd, b.nscale, b.opsP, b.opsE};
   for (void* p : ps) dfree(p);
+  if (c->h_step) cudaFreeHost(c->h_step);
   if (c->sg.exec) cudaGraphExecDestroy(c->sg.exec);
   if (c->sg.graph) cudaGraphDestroy(c->sg.graph);
   if (c->cap_s) cudaStreamDestroy(c->cap_s);
@@ -651,7 +672,7 @@ static int rrk_enqueue_stages(esplit_ctx* c, const double* u, double dt, cudaStr
   // block-partial regions: entropy of u_n (width 2) first, then the four stage
   // productions (width 1); reduced together after the stages
   esplit::ReduceRegions R{};
-  const int ent_cap = (int)std::max<size_t>((size_t)c->n_e * c->n_p / 256 + 1, (size_t)c->n_e);
+  const int ent_cap = (int)std::max<size_t>((size_t)c->n_e * c->n_p / 256 + 2 * esplit::SMS, (size_t)c->n_e);
   int off = 2 * ent_cap;
   // stage 0: the split volume kernel computes the entropy of u_n on the way
   // (entropy-split scheme); otherwise the entropy kernel does.  On the
@@ -729,8 +750,8 @@ int esplit_rrk_step(esplit_ctx* c, double* u, double dt, double* g_out, esplit_s
     if (esplit::launch_root_eval(c, u, c->b.dacc, s))
       return fail(c, ESPLIT_ERR_CUDA, "root launch");
   if (esplit::launch_root_apply(c, u, c->b.dacc, n, s)) return fail(c, ESPLIT_ERR_CUDA, "apply launch");
-  CK(cudaMemcpyAsync(&st, c->b.root, sizeof(st), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
+  if ((rc = read_step(c, s))) return rc;
+  std::memcpy(&st, c->h_step + kRootOff, sizeof(st));
   if (!st.done) {
     for (int it = 2; it < esplit::ROOT_EVALS_MAX; ++it) {
       if (esplit::launch_root_eval(c, u, c->b.dacc, s))
@@ -742,12 +763,14 @@ int esplit_rrk_step(esplit_ctx* c, double* u, double dt, double* g_out, esplit_s
       }
     }
     if (esplit::launch_root_apply(c, u, c->b.dacc, n, s)) return fail(c, ESPLIT_ERR_CUDA, "apply launch");
+    if ((rc = read_step(c, s))) return rc;
+    std::memcpy(&st, c->h_step + kRootOff, sizeof(st));
   }
   double e_stage[4];
-  CK(cudaMemcpyAsync(&st, c->b.root, sizeof(st), cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(e_stage, c->b.scal + 2, 4 * sizeof(double), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
-  int phys = read_status(c, s, true);
+  std::memcpy(e_stage, c->h_step + 2 * sizeof(double), sizeof(e_stage));
+  int h_status;
+  std::memcpy(&h_status, c->h_step + kStatusOff, sizeof(h_status));
+  int phys = status_code(c, h_status, s, true);
   c->last_stream = s;
   int status = phys ? phys : st.status;
   if (g_out) *g_out = st.g;

@@ -11,7 +11,16 @@
 namespace esplit {
 
 constexpr int MAX_NP = 80;
-constexpr int SMALL_BLOCKS = 4 * 152;  // short blocks up to four per SM (152 SMs), see split_cached_launch
+constexpr int SMS = 152;
+// threads per block of the kernels with one thread per node or facet pair: the
+// float64 pipe is shared by an SM's warps, so while there are fewer than `most`
+// threads per SM the warps go to as many SMs as there are
+inline int spread_block(size_t n, int most) {
+  int b = most;
+  while (b > 32 && (n + b - 1) / b < (size_t)SMS) b /= 2;
+  return b;
+}
+constexpr int SMALL_BLOCKS = 4 * SMS;  // short blocks up to four per SM, see split_cached_launch
 
 // row length of the float32 path's staged operators: the smallest multiple of
 // 4 (one 16-byte load) not below n_p whose number of 16-byte chunks is odd, so
@@ -166,6 +175,7 @@ struct esplit_ctx {
   // entropy of u_n runs there beside the stages (fork and join events)
   cudaStream_t side_s = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  unsigned char* h_step = nullptr;                 // pinned copy of [scal | root | status]
   void* hist = nullptr;                            // StepRecord[HIST_CAP] + int counter
   bool prof = false;
   std::vector<esplit::ProfRec> recs;

@@ -1098,7 +1098,7 @@ static int residual_np(esplit_ctx* c, const double* u, double* r, cudaStream_t s
                         std::is_same<T, double>::value)) &&
                       !visc && sat == c->b.sat && c->b.fcache != nullptr;
   if (!cached) {
-    int bs = 128;
+    const int bs = spread_block(c->n_pairs, 128);
     int nb = (c->n_pairs + bs - 1) / bs;
     ProfScope ps(c, PG_FACE, s);
     // facet terms are O(1/h) and cancel against the volume's boundary part:
@@ -1185,7 +1185,7 @@ static int residual_np(esplit_ctx* c, const double* u, double* r, cudaStream_t s
   }
   if (cached) {
     // after both volume kernels (the Hadamard kernel assigns r)
-    int bs = 128;
+    const int bs = spread_block(c->n_pairs, 128);
     int nb = (c->n_pairs + bs - 1) / bs;
     ProfScope ps(c, PG_FACE, s);
     face_cached_kernel<D><<<nb, bs, 0, s>>>(r, c->b.face_pairs, c->n_pairs, c->b.nu, c->b.ihd, c->b.nscale,
@@ -1386,16 +1386,16 @@ __global__ void __launch_bounds__(256) entropy_rate_kernel(const double* __restr
 
 int launch_entropy(esplit_ctx* c, const double* u, cudaStream_t s, int* n_partial, double* cache, double* part) {
   size_t n = (size_t)c->n_e * c->n_p;
-  int nb = (int)((n + 255) / 256);
+  const int bs = spread_block(n, 256), nb = (int)((n + bs - 1) / bs);
   Phys<double> ph = make_phys<double>(c->prm.gam, c->prm.beta, c->prm.R, c->prm.mu, c->prm.Pr);
   ProfScope ps(c, PG_ENTROPY, s);
   double* out = part ? part : c->b.partial;
   if (c->dim == 1)
-    entropy_kernel<1><<<nb, 256, 0, s>>>(u, c->b.J, n, ph, out, cache);
+    entropy_kernel<1><<<nb, bs, 0, s>>>(u, c->b.J, n, ph, out, cache);
   else if (c->dim == 2)
-    entropy_kernel<2><<<nb, 256, 0, s>>>(u, c->b.J, n, ph, out, cache);
+    entropy_kernel<2><<<nb, bs, 0, s>>>(u, c->b.J, n, ph, out, cache);
   else
-    entropy_kernel<3><<<nb, 256, 0, s>>>(u, c->b.J, n, ph, out, cache);
+    entropy_kernel<3><<<nb, bs, 0, s>>>(u, c->b.J, n, ph, out, cache);
   c->launches++;
   *n_partial = nb;
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
@@ -1404,25 +1404,25 @@ int launch_entropy(esplit_ctx* c, const double* u, cudaStream_t s, int* n_partia
 int launch_entropy_rate(esplit_ctx* c, const double* u, const double* r, cudaStream_t s, int* n_partial,
                         double* part, int width) {
   size_t n = (size_t)c->n_e * c->n_p;
-  int nb = (int)((n + 255) / 256);
+  const int bs = spread_block(n, 256), nb = (int)((n + bs - 1) / bs);
   Phys<double> ph = make_phys<double>(c->prm.gam, c->prm.beta, c->prm.R, c->prm.mu, c->prm.Pr);
   ProfScope ps(c, PG_ENTROPY, s);
   if (!part) part = c->b.partial;
   if (c->dim == 1) {
     if (width == 1)
-      entropy_rate_kernel<1, 1><<<nb, 256, 0, s>>>(u, r, c->b.J, n, ph, part);
+      entropy_rate_kernel<1, 1><<<nb, bs, 0, s>>>(u, r, c->b.J, n, ph, part);
     else
-      entropy_rate_kernel<1, 2><<<nb, 256, 0, s>>>(u, r, c->b.J, n, ph, part);
+      entropy_rate_kernel<1, 2><<<nb, bs, 0, s>>>(u, r, c->b.J, n, ph, part);
   } else if (c->dim == 2) {
     if (width == 1)
-      entropy_rate_kernel<2, 1><<<nb, 256, 0, s>>>(u, r, c->b.J, n, ph, part);
+      entropy_rate_kernel<2, 1><<<nb, bs, 0, s>>>(u, r, c->b.J, n, ph, part);
     else
-      entropy_rate_kernel<2, 2><<<nb, 256, 0, s>>>(u, r, c->b.J, n, ph, part);
+      entropy_rate_kernel<2, 2><<<nb, bs, 0, s>>>(u, r, c->b.J, n, ph, part);
   } else {
     if (width == 1)
-      entropy_rate_kernel<3, 1><<<nb, 256, 0, s>>>(u, r, c->b.J, n, ph, part);
+      entropy_rate_kernel<3, 1><<<nb, bs, 0, s>>>(u, r, c->b.J, n, ph, part);
     else
-      entropy_rate_kernel<3, 2><<<nb, 256, 0, s>>>(u, r, c->b.J, n, ph, part);
+      entropy_rate_kernel<3, 2><<<nb, bs, 0, s>>>(u, r, c->b.J, n, ph, part);
   }
   c->launches++;
   *n_partial = nb;
@@ -1864,16 +1864,16 @@ template <bool COND>
 static int root_eval_launch(esplit_ctx* c, const double* un, const double* d, cudaStream_t s,
                             cudaGraphConditionalHandle h) {
   size_t n = (size_t)c->n_e * c->n_p;
-  int nb = (int)((n + 255) / 256);
+  const int bs = spread_block(n, 256), nb = (int)((n + bs - 1) / bs);
   Phys<double> ph = make_phys<double>(c->prm.gam, c->prm.beta, c->prm.R, c->prm.mu, c->prm.Pr);
   if (c->dim == 1)
-    root_eval_kernel<1, COND><<<nb, 256, 0, s>>>(un, d, c->b.J, c->b.node_cache, n, ph, c->b.root, c->b.partial, c->stage_last,
+    root_eval_kernel<1, COND><<<nb, bs, 0, s>>>(un, d, c->b.J, c->b.node_cache, n, ph, c->b.root, c->b.partial, c->stage_last,
                                                    c->b.stage_r, h);
   else if (c->dim == 2)
-    root_eval_kernel<2, COND><<<nb, 256, 0, s>>>(un, d, c->b.J, c->b.node_cache, n, ph, c->b.root, c->b.partial, c->stage_last,
+    root_eval_kernel<2, COND><<<nb, bs, 0, s>>>(un, d, c->b.J, c->b.node_cache, n, ph, c->b.root, c->b.partial, c->stage_last,
                                                    c->b.stage_r, h);
   else
-    root_eval_kernel<3, COND><<<nb, 256, 0, s>>>(un, d, c->b.J, c->b.node_cache, n, ph, c->b.root, c->b.partial, c->stage_last,
+    root_eval_kernel<3, COND><<<nb, bs, 0, s>>>(un, d, c->b.J, c->b.node_cache, n, ph, c->b.root, c->b.partial, c->stage_last,
                                                    c->b.stage_r, h);
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? 0 : -1;

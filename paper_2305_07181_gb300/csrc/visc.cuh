@@ -181,7 +181,7 @@ static void viscous_volume_np(esplit_ctx* c, const double* u, double* r, const i
 // returns the number of block partials written to prod (0 without prod)
 template <int D>
 static int viscous_jump(esplit_ctx* c, double* r, cudaStream_t s, double* prod = nullptr) {
-  int bs = 128;
+  const int bs = spread_block(c->n_pairs, 128);
   int nb = (c->n_pairs + bs - 1) / bs;
   visc_jump_kernel<D><<<nb, bs, 0, s>>>(r, c->b.fv, c->b.face_pairs, c->n_pairs, c->b.nu, c->b.J, c->b.wslot,
                                         prod);

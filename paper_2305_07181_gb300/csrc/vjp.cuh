@@ -688,7 +688,7 @@ template <int D, int NP>
 static int vjp_np(esplit_ctx* c, const double* u, const double* cot, double* grad, cudaStream_t s) {
   const Phys<double> ph = make_phys<double>(c->prm.gam, c->prm.beta, c->prm.R, c->prm.mu, c->prm.Pr);
   {
-    int bs = 64;
+    const int bs = spread_block(c->n_pairs, 64);
     int nb = (c->n_pairs + bs - 1) / bs;
     ProfScope ps(c, PG_FACE, s);
     face_vjp_kernel<D><<<nb, bs, 0, s>>>(u, cot, c->b.face_pairs, c->n_pairs, c->b.nu, c->b.ihd, c->b.nscale,
