@@ -532,6 +532,11 @@ int launch_face_bc(esplit_ctx* c, const double* u, double* out, int add, double*
 // takes this kernel too: compensated float32 contractions measured slower,
 // 97 against 78 us on 18,432 triangles p 2).  Lines and 7-node
 // triangles: float64 FMA loops, too short for the tiles.
+// Measured per launch, float64 loops before and now: 32,768 triangles p 3 490
+// and 163 us, 7,442 triangles p 4 210 and 83, 3,072 tetrahedra p 3 740 and 158,
+// 24,576 tetrahedra p 2 with viscous terms 1,650 and 680.  Bound now by the
+// latency of its phases: float64 pipe ~50 % busy, issue slots 48 %, tensor pipe
+// 17 %, DRAM 15 % (18 nodes).
 // Optional: block partial of sum H w^T r (entropy production, float64).
 // ---------------------------------------------------------------------------
 template <int D, int NP, int EB, bool VISC, int TH = round32(EB * NP)>
@@ -766,7 +771,7 @@ __global__ void __launch_bounds__(TH, SplitCfg<D, NP, EB, VISC, TH>::BLOCKS) spl
     }
     if (active) {
       if (sl >= 0) {
-        const double ih = 1.0 / Hm;
+        const double ih = rcp64(Hm);
         double nv[D];
 #pragma unroll
         for (int i = 0; i < D; ++i) nv[i] = __ldg(&nu[((size_t)e * NS + sl) * D + i]);

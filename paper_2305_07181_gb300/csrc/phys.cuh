@@ -34,6 +34,7 @@ struct Phys {
   T ir_a, ir_b;        // (gam+1)/(2 gam), (gam-1)/(2 gam), times gam/(gam-1)
   T s_ac, s_en;        // S^ entries: 1/(2 gam), (gam-1)(gam+alpha)/(gam alpha), Eq. (76)
   T mu, kappa, R;      // viscosity, conductivity mu gam R/((gam-1) Pr), gas constant
+  T iR, k_T;           // 1/R, (gam-1)/(alpha R)
   // Taylor coefficients of g(eps) = ((1+eps)^r - 1)/(r eps) for r = r1, r2
   // (c_0 = 1, c_k = c_(k-1) (r - k)/(k + 1)), used by exp_avg
   T ser1[16], ser2[16];
@@ -72,6 +73,8 @@ __host__ inline Phys<T> make_phys(double gam, double beta, double R, double mu, 
   c.mu = (T)mu;
   c.kappa = (T)(mu * gam * R / ((gam - 1.0) * Pr));
   c.R = (T)R;
+  c.iR = (T)(1.0 / R);
+  c.k_T = (T)((gam - 1.0) / (alpha * R));
   double r1 = -gam / alpha, r2 = (1.0 - gam) / alpha;
   const double pw[4] = {alpha / (alpha + gam), (1.0 - alpha - gam) / (alpha + gam), r1, r2};
   c.im_ok = 1;

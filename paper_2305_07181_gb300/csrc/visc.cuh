@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(EB * NP) visc_volume_kernel(const double* __re
       for (int q = 0; q < NC; ++q) acc[q] += dt * sF[el][i][q][n];
     }
   if (sl >= 0) {
-    double ih = 1.0 / Hm;
+    double ih = rcp64(Hm);
 #pragma unroll
     for (int q = 0; q < NC; ++q) {
       double corr = 0.0;
@@ -138,8 +138,8 @@ __global__ void __launch_bounds__(128) visc_jump_kernel(double* __restrict__ r, 
     int k = pr.x / NS, s = pr.x - k * NS;
     int v = pr.y / NS, s2 = pr.y - v * NS;
     int m = c_ref.slot_node[s], n = c_ref.slot_node[s2];
-    double ihk = 1.0 / (c_ref.H[m] * __ldg(&J[(size_t)k * NP + m]));
-    double ihv = 1.0 / (c_ref.H[n] * __ldg(&J[(size_t)v * NP + n]));
+    double ihk = rcp64(c_ref.H[m] * __ldg(&J[(size_t)k * NP + m]));
+    double ihv = rcp64(c_ref.H[n] * __ldg(&J[(size_t)v * NP + n]));
     double nuv[D];
 #pragma unroll
     for (int i = 0; i < D; ++i) nuv[i] = __ldg(&nu[((size_t)k * NS + s) * D + i]);

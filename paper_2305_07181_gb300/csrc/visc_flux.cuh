@@ -29,16 +29,26 @@ __device__ __forceinline__ void dT_dW(const Node<T, D>& n, const C& c, T* TW) {
     const T pr = n.p * n.ir;  // p / rho = -1 / v_nc
 #pragma unroll
     for (int q = 0; q < NC - 1; ++q) TW[q] = T(0.0);
-    TW[NC - 1] = pr * pr / c.R;
+    if constexpr (std::is_same<T, double>::value)
+      TW[NC - 1] = pr * pr * c.iR;
+    else
+      TW[NC - 1] = pr * pr / c.R;
     return;
   }
-  T Wn = -n.q;
-  T k = c.gm1 / (c.alpha * c.R * Wn);
-  T T_ = n.p * n.ir / c.R;
+  T k, TiW;  // dT/dW_1 and T / W_nc
+  if constexpr (std::is_same<T, double>::value) {
+    const double iWn = -rcp64(n.q);
+    k = c.k_T * iWn;
+    TiW = n.p * n.ir * c.iR * iWn;
+  } else {
+    T Wn = -n.q;
+    k = c.gm1 / (c.alpha * c.R * Wn);
+    TiW = n.p * n.ir / c.R / Wn;
+  }
   TW[0] = k;
 #pragma unroll
   for (int l = 0; l < D; ++l) TW[1 + l] = k * n.V[l];
-  TW[NC - 1] = -T_ / Wn + S(0.5) * k * n.v2;
+  TW[NC - 1] = -TiW + S(0.5) * k * n.v2;
 }
 
 // F^V_i (i < D) from the entropy-variable gradients g[j] = dW/dx_j:
@@ -53,6 +63,8 @@ __device__ __forceinline__ void visc_flux(const Node<T, D>& n, const C& c, int h
   T iWn;  // 1 / w_nc
   if constexpr (ENT == 1)
     iWn = -(n.p * n.ir);
+  else if constexpr (std::is_same<T, double>::value)
+    iWn = -rcp64(n.q);
   else
     iWn = S(-1.0) / n.q;
   T Lg[D][D];  // Lg[j][l] = dV_l/dx_j
@@ -95,6 +107,8 @@ __device__ __forceinline__ void visc_flux_transpose(const Node<T, D>& n, const C
   T iWn;  // 1 / w_nc
   if constexpr (ENT == 1)
     iWn = -(n.p * n.ir);
+  else if constexpr (std::is_same<T, double>::value)
+    iWn = -rcp64(n.q);
   else
     iWn = S(-1.0) / n.q;
   T cc[D][D];
