@@ -535,8 +535,8 @@ int launch_face_bc(esplit_ctx* c, const double* u, double* out, int add, double*
 // Measured per launch, float64 loops before and now: 32,768 triangles p 3 490
 // and 163 us, 7,442 triangles p 4 210 and 83, 3,072 tetrahedra p 3 740 and 158,
 // 24,576 tetrahedra p 2 with viscous terms 1,650 and 680.  Bound now by the
-// latency of its phases: float64 pipe ~50 % busy, issue slots 48 %, tensor pipe
-// 17 %, DRAM 15 % (18 nodes).
+// latency of its phases: float64 pipe and issue slots 60 % busy, tensor pipe
+// 20 % (18 nodes, 24 warps per SM).
 // Optional: block partial of sum H w^T r (entropy production, float64).
 // ---------------------------------------------------------------------------
 template <int D, int NP, int EB, bool VISC, int TH = round32(EB * NP)>
