@@ -237,16 +237,6 @@ __device__ __forceinline__ bool node_from_u(const T* u, const C& c, Node<T, D>& 
   return ok;
 }
 
-// Euler flux F^{I(i)} of Eq. (5).
-template <typename T, int D>
-__device__ __forceinline__ void euler_flux(const Node<T, D>& n, int i, T* F) {
-  T m = n.rho * n.V[i];
-  F[0] = m;
-#pragma unroll
-  for (int j = 0; j < D; ++j) F[1 + j] = m * n.V[j] + (j == i ? n.p : T(0));
-  F[D + 1] = (n.e + n.p) * n.V[i];
-}
-
 // dF^{I(i)} = A~_i v (Eq. (19)): the change of F_i(U(W)) for a change v of
 // the entropy variables, by the chain rule through (q, V, theta = p/rho, rho):
 //   q = -W_nc, V = W_(1..d)/q, W_1/q = w1c theta - |V|^2/2,
@@ -457,9 +447,6 @@ struct ExpAvgCfg<float> {
   static constexpr int NTERMS = 14;
 };
 
-template <int N>
-struct ExpAvgCfg<Dual<N>> : ExpAvgCfg<double> {};
-
 template <typename T, typename S>
 __device__ __forceinline__ T exp_avg(T a, T b, T ar, T br, S r, T ia, const S* coef) {
   T eps = (b - a) * ia;
@@ -469,26 +456,6 @@ __device__ __forceinline__ T exp_avg(T a, T b, T ar, T br, S r, T ia, const S* c
   T sum = coef[ExpAvgCfg<T>::NTERMS - 1];
 #pragma unroll
   for (int k = ExpAvgCfg<T>::NTERMS - 2; k >= 0; --k) sum = sum * eps + coef[k];  // Horner
-  return ar * ia * sum;
-}
-
-// The same average on dual numbers: the series and its derivative by Horner's
-// rule on the values, then one chain-rule step (d sum = g'(eps) d eps),
-// instead of the series on the duals.
-template <int N, typename S>
-__device__ __forceinline__ Dual<N> exp_avg(const Dual<N>& a, const Dual<N>& b, const Dual<N>& ar,
-                                           const Dual<N>& br, S r, const Dual<N>& ia, const S* coef) {
-  const Dual<N> eps = (b - a) * ia;
-  if (fabs(eps.v) >= ExpAvgCfg<double>::EPS_SWITCH) return (ar - br) / (r * (a - b));
-  double sv = coef[ExpAvgCfg<double>::NTERMS - 1], dv = 0.0;
-#pragma unroll
-  for (int k = ExpAvgCfg<double>::NTERMS - 2; k >= 0; --k) {
-    dv = dv * eps.v + sv;
-    sv = sv * eps.v + coef[k];
-  }
-  Dual<N> sum(sv);
-#pragma unroll
-  for (int i = 0; i < N; ++i) sum.d[i] = dv * eps.d[i];
   return ar * ia * sum;
 }
 
