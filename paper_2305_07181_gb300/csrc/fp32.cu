@@ -432,15 +432,8 @@ static int split_f32_np(esplit_ctx* c, const double* u, double* r, cudaStream_t 
     ProfScope ps(c, PG_SPLIT, s);
     constexpr bool STAGE = true;
     const size_t dyn = STAGE ? (size_t)EB * c->opsD_stride * sizeof(float) : 0;
-    if (STAGE) {
-      // static + dynamic shared memory above 48 KB needs the opt-in
-      static size_t attr_set = 0;
-      if (attr_set < dyn) {
-        cudaFuncSetAttribute(split_volume_f32_kernel<D, NP, EB, STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)dyn);
-        attr_set = dyn;
-      }
-    }
+    // static + dynamic shared memory above 48 KB needs the opt-in
+    if (STAGE && opt_in_smem(c, split_volume_f32_kernel<D, NP, EB, STAGE>, dyn, false)) return -1;
     split_volume_f32_kernel<D, NP, EB, STAGE><<<nb, EB * NP, dyn, s>>>(
         u, r, c->b.opsD32, c->opsD_stride, c->b.ihf, satf, c->n_e, ph, c->b.status,
         prod ? prod + np_used : nullptr);

@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "../../include/esplit.h"
+#include "optin.h"
 
 namespace esplit {
 
@@ -141,6 +142,7 @@ struct StepGraph {
 };
 
 struct esplit_ctx {
+  esplit::OptIn optin;             // kernel attributes set on this context's device
   int dim = 2, device = 0, n_c = 4;
   int n_p = 0, n_fac = 0, n_f = 0, n_slot = 0;
   int n_e = 0, n_pairs = 0;
@@ -183,6 +185,21 @@ struct esplit_ctx {
 };
 
 namespace esplit {
+
+// Allows a kernel `bytes` of dynamic shared memory on the context's device
+// (the current one), and with `carve` asks for the largest shared-memory share
+// of the SM's cache, so that as many blocks fit as the kernel is compiled for.
+// Nonzero when the device refuses.
+template <class Kernel>
+int opt_in_smem(esplit_ctx* c, Kernel* kern, size_t bytes, bool carve) {
+  return c->optin.once(reinterpret_cast<const void*>(kern), [&]() -> int {
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return -1;
+    if (carve && cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                      cudaSharedmemCarveoutMaxShared) != cudaSuccess)
+      return -1;
+    return 0;
+  });
+}
 
 // Brackets one kernel launch with CUDA events on its stream when the
 // context's profiling is enabled (groups listed in include/esplit.h).

@@ -1042,18 +1042,14 @@ struct VolCfg {
   static constexpr int HAD_KC = NP > 32 ? 8 : NP / 2;
 };
 
+// launches the kernel; the number of blocks, or -1 when the device refuses the shared memory
 template <int D, int NP, int EB, bool VISC, bool CACHE, bool ENT, int TH = round32(EB * NP)>
 static int split_launch(esplit_ctx* c, const double* u, double* r, const double* sat, const int* list, int n_list,
                         double* prod, double* ent_part, cudaStream_t s) {
   using Cfg = SplitCfg<D, NP, EB, VISC, TH>;
   auto* kern = split_volume_kernel<D, NP, EB, VISC, CACHE, ENT, TH>;
   const int nb = (n_list + EB - 1) / EB;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
-    cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-    attr_set = true;
-  }
+  if (opt_in_smem(c, kern, Cfg::SMEM, true)) return -1;
   const Phys<double> ph = make_phys<double>(c->prm.gam, c->prm.beta, c->prm.R, c->prm.mu, c->prm.Pr);
   kern<<<nb, Cfg::THREADS, Cfg::SMEM, s>>>(u, r, c->b.ops64, c->b.opsP, c->b.opsE, c->b.J, sat, list, n_list, ph,
                                            c->b.status, prod, VISC ? c->prm.heat_flux : -1, c->b.nu,
@@ -1155,6 +1151,7 @@ static int residual_np(esplit_ctx* c, const double* u, double* r, cudaStream_t s
       nb = split_cached_launch<D, NP, EB, false>(c, u, r, sat, lsplit, n_split, pp, nullptr, s);
     else
       nb = split_launch<D, NP, EB, false, false, false>(c, u, r, sat, lsplit, n_split, pp, nullptr, s);
+    if (nb < 0) return -1;
     c->launches++;
     np_used += nb;
   }
@@ -1162,14 +1159,9 @@ static int residual_np(esplit_ctx* c, const double* u, double* r, cudaStream_t s
     constexpr int EB = VolCfg<NP>::EB_HAD;
     constexpr int KC = VolCfg<NP>::HAD_KC;
     size_t smem = sizeof(T) * ((size_t)EB * (D + 7) * NP + (size_t)EB * NP * KC * (D + 2) + (size_t)EB * NP);
-    static bool attr_set = false;
-    if (!attr_set) {
-      cudaFuncSetAttribute(hadamard_volume_kernel<T, D, NP, EB, 0, KC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem);
-      cudaFuncSetAttribute(hadamard_volume_kernel<T, D, NP, EB, 1, KC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem);
-      attr_set = true;
-    }
+    auto* kern = scheme == ESPLIT_SCHEME_HADAMARD_IR ? hadamard_volume_kernel<T, D, NP, EB, 1, KC>
+                                                     : hadamard_volume_kernel<T, D, NP, EB, 0, KC>;
+    if (opt_in_smem(c, kern, smem, false)) return -1;
     int nb = (n_had + EB - 1) / EB;
     ProfScope ps(c, PG_HAD, s);
     if (scheme == ESPLIT_SCHEME_HADAMARD_IR)

@@ -670,18 +670,14 @@ __global__ void __launch_bounds__(TH, VjpCfg<D, NP, EB, TH>::BLOCKS) split_vjp_k
 }
 
 template <int D, int NP, int EB, int TH>
-static void split_vjp_launch(esplit_ctx* c, const double* u, const double* cot, double* grad, const Phys<double>& ph,
+static int split_vjp_launch(esplit_ctx* c, const double* u, const double* cot, double* grad, const Phys<double>& ph,
                              cudaStream_t s) {
   using Cfg = VjpCfg<D, NP, EB, TH>;
   auto* kern = split_vjp_kernel<D, NP, EB, TH>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
-    cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-    attr_set = true;
-  }
+  if (opt_in_smem(c, kern, Cfg::SMEM, true)) return -1;
   kern<<<(c->n_e + EB - 1) / EB, TH, Cfg::SMEM, s>>>(u, cot, c->b.ops64, c->b.opsP, c->b.opsE, c->b.J, c->b.ihd,
                                                      c->b.nu, c->b.sat, c->n_e, grad, ph);
+  return 0;
 }
 
 template <int D, int NP>
@@ -702,10 +698,11 @@ static int vjp_np(esplit_ctx* c, const double* u, const double* cot, double* gra
     constexpr int BY_TASKS = 32 * (TASKS < 4 ? TASKS : 4);
     constexpr int THS = VjpCfg<D, NP, EB>::TENSOR && BY_TASKS > MIN ? BY_TASKS : MIN;
     ProfScope ps(c, PG_SPLIT, s);
-    if ((c->n_e + EBS - 1) / EBS <= SMALL_BLOCKS)  // small meshes: short blocks, as for the split volume kernel
-      split_vjp_launch<D, NP, EBS, THS>(c, u, cot, grad, ph, s);
-    else
-      split_vjp_launch<D, NP, EB, round32(EB * NP)>(c, u, cot, grad, ph, s);
+    // small meshes: short blocks, as for the split volume kernel
+    const int rc = (c->n_e + EBS - 1) / EBS <= SMALL_BLOCKS
+                       ? split_vjp_launch<D, NP, EBS, THS>(c, u, cot, grad, ph, s)
+                       : split_vjp_launch<D, NP, EB, round32(EB * NP)>(c, u, cot, grad, ph, s);
+    if (rc) return rc;
     c->launches++;
   }
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
