@@ -671,7 +671,7 @@ __global__ void __launch_bounds__(TH, SplitCfg<D, NP, EB, VISC, TH>::BLOCKS) spl
     if constexpr (ENT) {
       // entropy of u_n for the relaxation step (the entropy kernel's outputs):
       // S_H = beta q p, and the per-node values its evaluation passes reuse
-      const size_t nn = (size_t)n_list * NP, g = (size_t)e * NP + m;
+      const size_t nn = (size_t)n_list * NP, g = (size_t)e * NP + m;  // the list is all elements
       const double sH = c64.beta * nd.q * nd.p;
       ncache[g] = sH;
       ncache[nn + g] = nd.ir;
@@ -1138,8 +1138,10 @@ static int residual_np(esplit_ctx* c, const double* u, double* r, cudaStream_t s
     int nb;
     ProfScope ps(c, PG_SPLIT, s);
     double* pp = prod ? prod + np_used : nullptr;
-    if (visc && c->ent_part && c->b.node_cache) {
-      // first stage of a relaxation step: the kernel also forms the entropy of u_n
+    if (visc && scheme == ESPLIT_SCHEME_SPLIT && c->ent_part && c->b.node_cache) {
+      // first stage of a relaxation step: the kernel also forms the entropy of
+      // u_n (split scheme only: in the hybrid one it sees a part of the elements,
+      // and the step takes the entropy kernel)
       nb = split_launch<D, NP, EB, true, false, true>(c, u, r, sat, lsplit, n_split, pp, c->ent_part, s);
       c->ent_n = nb;
     } else if (visc)
