@@ -248,19 +248,25 @@ struct JvpPrep {
   T w0q, rq, ep;  // w1c theta - |V|^2/2, rho/(a_q + b_q), e + p (shared by the directions)
 };
 
+// from 1/q and rho/p
 template <typename T, int D, typename C>
-__device__ __forceinline__ JvpPrep<T> jvp_prep(const Node<T, D>& n, const C& c) {
+__device__ __forceinline__ JvpPrep<T> jvp_prep_from(const Node<T, D>& n, const C& c, const T& iq, const T& itheta) {
   JvpPrep<T> j;
-  // one division for 1/q and rho/p: y = 1/(q p), 1/q = p y, 1/p = q y
-  const T y = t_rcp(n.q * n.p);
-  j.iq = n.p * y;
+  j.iq = iq;
   j.ir = n.ir;
   j.theta = n.p * j.ir;
-  j.itheta = n.rho * (n.q * y);
+  j.itheta = itheta;
   j.w0q = c.w1c * j.theta - T(0.5) * n.v2;
   j.rq = n.rho * c.inv_apb;
   j.ep = n.e + n.p;
   return j;
+}
+
+// one division for 1/q and rho/p: y = 1/(q p), 1/q = p y, 1/p = q y
+template <typename T, int D, typename C>
+__device__ __forceinline__ JvpPrep<T> jvp_prep(const Node<T, D>& n, const C& c) {
+  const T y = t_rcp(n.q * n.p);
+  return jvp_prep_from<T, D>(n, c, n.p * y, n.rho * (n.q * y));
 }
 
 template <typename T, int D, typename C>

@@ -364,9 +364,15 @@ __global__ void __launch_bounds__(64) face_vjp_kernel(const double* __restrict__
   ZNode<double, D> zk, zv;
   znode<double, D>(nk, c, zk);
   znode<double, D>(nv, c, zv);
-  const JvpPrep<double> jk = jvp_prep<double, D>(nk, c), jv = jvp_prep<double, D>(nv, c);
-  const double ipk = jk.itheta * jk.ir, ipv = jv.itheta * jv.ir;
-  zk.iq = jk.iq;
+  // 1/q and 1/p of each side by a reciprocal of its own: as products of one
+  // reciprocal 1/(q p) they carry up to three more roundings into every term of
+  // the nodal chains (relative error of the gradient with dissipation, 3,200
+  // triangles p 1 / 1,296 tetrahedra p 1: 2.71e-15 / 2.46e-15 instead of 2.93e-15 /
+  // 2.64e-15; by divisions 2.75e-15 / 2.45e-15)
+  const double iqk = rcp64(nk.q), ipk = rcp64(nk.p), iqv = rcp64(nv.q), ipv = rcp64(nv.p);
+  const JvpPrep<double> jk = jvp_prep_from<double, D>(nk, c, iqk, nk.rho * ipk);
+  const JvpPrep<double> jv = jvp_prep_from<double, D>(nv, c, iqv, nv.rho * ipv);
+  zk.iq = iqk;
   zk.ip = ipk;
   double nud[D], nh[D];
   const double* ns = nscale + (size_t)pr.x * (D + 1);  // |nu|, nu/|nu| of slot (k, s)
@@ -391,8 +397,8 @@ __global__ void __launch_bounds__(64) face_vjp_kernel(const double* __restrict__
   pair_rev_prep<D>(zk, zv, c, pv);
   pair_reverse<D>(zk, zv, pv, c, nud, dissipation, b, nh, gb, dw, kb, vb);
   double gk[NC], gv[NC];
-  node_chain_rev<D>(nk, zk, kb, c, jk.iq, ipk, gk);
-  node_chain_rev<D>(nv, zv, vb, c, jv.iq, ipv, gv);
+  node_chain_rev<D>(nk, zk, kb, c, iqk, ipk, gk);
+  node_chain_rev<D>(nv, zv, vb, c, iqv, ipv, gv);
   if (dissipation) {
     PairSums<D> ps;
     ps.dn = 2.0 * pv.a.A1 * pv.a.E1;
