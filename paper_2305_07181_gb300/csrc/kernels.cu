@@ -533,7 +533,7 @@ int launch_face_bc(esplit_ctx* c, const double* u, double* out, int add, double*
 // 97 against 78 us on 18,432 triangles p 2).  Lines and 7-node
 // triangles: float64 FMA loops, too short for the tiles.
 // Measured per launch, float64 loops before and now: 32,768 triangles p 3 490
-// and 163 us, 7,442 triangles p 4 210 and 83, 3,072 tetrahedra p 3 740 and 158,
+// and 163 us, 7,442 triangles p 4 210 and 83, 3,072 tetrahedra p 3 740 and 177,
 // 24,576 tetrahedra p 2 with viscous terms 1,650 and 680.  Bound now by the
 // latency of its phases: float64 pipe and issue slots 60 % busy, tensor pipe
 // 20 % (18 nodes, 24 warps per SM).
@@ -554,7 +554,7 @@ struct SplitCfg {
   // SM (80 registers, a few spills) on inviscid triangles, 16 (128 registers)
   // otherwise, as far as shared memory allows.  Measured with the operators
   // fetched ahead: 18 nodes 5 -> 6 blocks 173 -> 167 us per launch (32,768
-  // triangles), 58 nodes 3 -> 4 blocks 170 -> 160 us (3,072 tetrahedra).
+  // triangles), 58 nodes 3 -> 4 blocks 170 -> 160 us (3,072 tetrahedra, six digits).
   static constexpr int BY_SMEM = (int)(233472 / (SMEM + 2048));  // 228 KB per SM; block sums and 1 KB reserved per block
   static constexpr int BY_REGS = (TENSOR && D == 2 && !VISC ? 768 : D == 2 && !VISC ? 640 : 512) / THREADS;
   // short blocks (small meshes, at most a few per SM): no register pressure

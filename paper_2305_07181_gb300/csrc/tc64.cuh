@@ -8,28 +8,40 @@
 // float64 FMA loop over the operators therefore spends ~3/4 of the volume
 // kernel on the contractions.  Here they take no float64 instruction at all:
 //   * every row of D_i and every column of x becomes fixed point: a signed
-//     integer of 6 BITS bits times a power of two taken from the row's or the
-//     column's largest entry, cut into 6 signed digits of BITS bits, each exact
-//     in fp16;
+//     integer of DIGITS BITS bits times a power of two taken from the row's or
+//     the column's largest entry, cut into signed digits of BITS bits, each
+//     exact in fp16 (digits.h);
 //   * products of digits are sums of integers below 2^24, exact in the float32
 //     accumulators of mma.sync (m16n8k16); digit pairs (j, a) of one weight
 //     level j + a share accumulators;
 //   * the levels are added up as 64-bit integers and rounded once to float64.
-// Digit width: BITS = 10 up to 32 nodes (60 bits: quantisation 2^-60 of the
-// largest entry, far below a float64 rounding), 9 above (54 bits; a digit
-// product sum over 80 nodes and three pairs stays below 2^24).  Levels up to
-// 3 (BITS 10) are exact; of level 4 on (2^-58 of the largest product) at most
-// the last bits round.  Omitted: digit pairs of level > 6, below 2^-59.
-// The result is closer to the exact sum than n_p float64 FMAs are.
+// Digits: six of 10 bits up to 32 nodes; above, where three digit products of
+// 2^18 over 80 nodes would pass 2^24, seven of 9 bits.
+//
+// Accuracy, with A and X the powers of two above the largest entry of the row
+// and of the column and u = 2^-53:
+//   six digits:   |error| <= 2^-60 (X sum|D| + A sum|x|) + (n_p 2^-59 + 2^-56) A X + u |result|
+//   seven digits: |error| <= 2^-63 (X sum|D| + A sum|x|) + (n_p 2^-60 + 2^-60) A X + 1.25 u |result|
+// (quantisation of the operands; digit pairs left out: (2, 4), (4, 2) and all
+// of level 7 on, or level 7 on; the last unit of the integer sum).  An FMA loop
+// errs by the row's own summands instead, up to n_p u sum|D||x|.  So the sum
+// here is the closer one as long as the products of a row reach a fair part of
+// A X, and the loop is where a column's large entries meet only small entries
+// of the row.  Measured against exact sums with the library's operators, in
+// units of u sum|D||x|, root mean square (loop | here), one entry of the
+// column larger than the others by the factor:
+//   18 nodes: 1 0.57 | 0.19, 50 0.77 | 0.42, 1e3 1.3 | 2.8, 1e6 1.7 | 490
+//   58 nodes: 1 0.69 | 0.13, 50 1.06 | 0.19, 1e3 1.9 | 0.8, 1e6 2.2 | 270
 //
 // Tile: the 16 rows of the A operand are 8 columns of x times 2 consecutive
 // digits, the 8 columns of the B operand 8 rows m of D_i, so both digits'
-// accumulators of an output (c, m) sit in one thread.  12 products (14 for
-// BITS 9) of a 16 x 8 x 16 tile cover the 24 digit pairs that matter.  D_i is
-// stored as 60-bit integers, two entries in 16 bytes, digits laid out so that
-// one shift-and-mask step gives the fp16 pair of a digit (half the bytes of
-// pre-cut fp16 digits; the cutting hides behind the float64 pointwise work of
-// the other blocks of the SM).
+// accumulators of an output (c, m) sit in one thread.  12 products of a
+// 16 x 8 x 16 tile cover the 22 digit pairs of six digits, 16 the 28 of seven
+// (the pair of digit 6 holds digit 6 twice; the second one's level is not
+// used).  D_i is stored in 60 or 63 bits, two entries in 16 bytes, digits laid
+// out so that one shift-and-mask step gives the fp16 pair of a digit (half the
+// bytes of pre-cut fp16 digits; the cutting hides behind the float64 pointwise
+// work of the other blocks of the SM).
 //
 // Columns whose largest entry is below 2^-958 count as zero; a column or row
 // with a non-finite entry gives NaN, as a sum over it would.
@@ -39,55 +51,16 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "digits.h"
+
 namespace esplit {
 namespace tc {
 
-constexpr int NONFINITE = 1 << 14;  // exponent marker: the column or row holds an Inf or NaN
-
-__host__ __device__ constexpr int bits_for(int np) { return np <= 32 ? 10 : 9; }
-__host__ __device__ constexpr int pairs_for(int np) { return (np + 1) / 2; }
-
-// power-of-two exponent (biased, from the high words) of the largest entry:
-// every entry is below 0.998 2^(E - 1022), within the signed digits' range
-__device__ __forceinline__ int exp_of_max(unsigned hi_abs_max) {
-  const int e = (int)((hi_abs_max + 0x1100u) >> 20);
-  return hi_abs_max >= 0x7FF00000u ? NONFINITE : e;
-}
-
-// x as 6 unsigned BITS-bit fields (most significant first from bit 5 BITS),
-// field = digit + 2^(BITS-1), relative to the exponent E of exp_of_max
-template <int BITS>
-__device__ __forceinline__ unsigned long long fixed_fields(double x, int E) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const int e = (int)((hi >> 20) & 0x7ffu);
-  const unsigned long long M = ((unsigned long long)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo;
-  constexpr int UP = 6 * BITS - 54;  // 6 (BITS 10) or 0 (BITS 9)
-  const int d = E < 64 ? 63 : min(E - e, 63);
-  // right shift by d, rounded to nearest
-  unsigned long long v = (((M << (UP + 1)) >> (d & 63)) + 1ULL) >> 1;
-  constexpr unsigned long long BIAS =
-      (1ULL << (BITS - 1)) * (((1ULL << (6 * BITS)) - 1ULL) / ((1ULL << BITS) - 1ULL));
-  return (hi >> 31) ? BIAS - v : BIAS + v;
-}
-
 // ---------------------------------------------------------------------------
-// packed operators: opsP[e][i][m][pair] (uint4) holds D_i[m][2 pair], D_i[m][2 pair + 1]
-//   x: digit 0 in bits 0-9, low 6 bits of digit 2 in bits 10-15 (entry 2 pair;
-//      entry 2 pair + 1 in the upper halfword), y: digit 1, high bits of digit 2;
-//   z, w: digits 3, 4, 5 likewise.  opsE[e][i][m]: the row's exponent.
+// packed operators: opsP[e][i][m][pair] (uint4) holds D_i[m][2 pair] and
+// D_i[m][2 pair + 1] (in the upper halfwords) as pack_half lays them out.
+// opsE[e][i][m]: the row's exponent.
 // ---------------------------------------------------------------------------
-template <int BITS>
-__device__ __forceinline__ void pack_half(unsigned long long b, unsigned& x, unsigned& y, unsigned& z, unsigned& w) {
-  constexpr unsigned MASK = (1u << BITS) - 1u;
-  const unsigned u0 = (unsigned)(b >> (5 * BITS)) & MASK, u1 = (unsigned)(b >> (4 * BITS)) & MASK;
-  const unsigned u2 = (unsigned)(b >> (3 * BITS)) & MASK, u3 = (unsigned)(b >> (2 * BITS)) & MASK;
-  const unsigned u4 = (unsigned)(b >> BITS) & MASK, u5 = (unsigned)b & MASK;
-  x = u0 | ((u2 & 63u) << 10);
-  y = u1 | ((u2 >> 6) << 10);
-  z = u3 | ((u5 & 63u) << 10);
-  w = u4 | ((u5 >> 6) << 10);
-}
-
 // one thread per (element, direction, row); ops64: [e][d][n][m]
 template <int BITS>
 __global__ void build_packed_kernel(const double* __restrict__ ops64, int n_e, int d, int np,
@@ -114,21 +87,19 @@ __global__ void build_packed_kernel(const double* __restrict__ ops64, int n_e, i
 
 template <int BITS>
 __device__ __forceinline__ unsigned unbias(unsigned fields) {  // two 16-bit fields -> two fp16 digits
-  const unsigned h = (fields & 0x03FF03FFu) | 0x64006400u;     // 1024 + field
-  const unsigned c = BITS == 10 ? 0x66006600u : 0x65006500u;   // 1024 + 2^(BITS-1)
+  constexpr unsigned MASK = BITS == 10 ? 0x03FF03FFu : 0x01FF01FFu;
+  const unsigned h = (fields & MASK) | 0x64006400u;           // 1024 + field
+  const unsigned c = BITS == 10 ? 0x66006600u : 0x65006500u;  // 1024 + 2^(BITS-1)
   unsigned r;
   asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(h), "r"(c));
   return r;
 }
 
 template <int BITS>
-__device__ __forceinline__ void unpack(const uint4& q, unsigned (&s)[6]) {
-  s[0] = unbias<BITS>(q.x);
-  s[1] = unbias<BITS>(q.y);
-  s[2] = unbias<BITS>(((q.x >> 10) & 0x003F003Fu) | ((q.y >> 4) & 0x03C003C0u));
-  s[3] = unbias<BITS>(q.z);
-  s[4] = unbias<BITS>(q.w);
-  s[5] = unbias<BITS>(((q.z >> 10) & 0x003F003Fu) | ((q.w >> 4) & 0x03C003C0u));
+__device__ __forceinline__ void unpack(const uint4& q, unsigned (&s)[digits_of(BITS)]) {
+  unpack_fields<BITS>(q.x, q.y, q.z, q.w, s);
+#pragma unroll
+  for (int k = 0; k < digits_of(BITS); ++k) s[k] = unbias<BITS>(s[k]);
 }
 
 __device__ __forceinline__ void mma16(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
@@ -164,6 +135,7 @@ __device__ __forceinline__ void ldm2(unsigned& r0, unsigned& r1, unsigned addr) 
 template <int D, int NP, int EB, int NF, int NW, int THREADS>
 struct Shape {
   static constexpr int BITS = bits_for(NP);
+  static constexpr int DIGITS = digits_of(BITS);
   static constexpr int KP = (NP + 7) / 8 * 8;          // nodes padded to the tile
   static constexpr int K16 = KP / 16;                  // 16-node tiles, then one of 8 if KP % 16
   static constexpr bool K8 = KP % 16 != 0;
@@ -181,15 +153,18 @@ struct Shape {
   static constexpr int T = BITS == 10 ? 6 : 7;         // accumulator tiles
   // unit of the 64-bit level sums, 2^-UNIT of the digit products' unit: the
   // sum over NP nodes and D directions stays below 2^63
-  static constexpr int UNIT = BITS == 10 ? (D == 3 ? 62 : 61) : 51;
-  static constexpr size_t DIG_EL = (size_t)6 * COLS * NPW * 4, RES_EL = (size_t)OUTS * NPO * 8;  // bytes per element
+  static constexpr int UNIT = BITS == 10 ? (D == 3 ? 62 : 61) : 69;
+  static constexpr size_t DIG_EL = (size_t)DIGITS * COLS * NPW * 4, RES_EL = (size_t)OUTS * NPO * 8;  // bytes per element
   // Where every warp takes the same number of an element's row tiles, the
   // element's results go over the digits of the element before it (a block
   // barrier between the elements), the first one's to a region of its own:
   // 53 instead of 71 KB per block at 25 nodes, four blocks per SM instead of
-  // three (Navier-Stokes kernel, 24,576 tetrahedra: 780 -> 680 us).  Not for
-  // blocks of a few elements, which other limits hold to the same number.
-  static constexpr bool OVER = EB >= 4 && NT % (THREADS / 32) == 0 && RES_EL <= DIG_EL;
+  // three (Navier-Stokes kernel, 24,576 tetrahedra: 780 -> 680 us); with seven
+  // digits, 50 instead of 60 KB at 58 nodes and 63 instead of 76 KB at 78 (four
+  // and three blocks instead of three and two; 3,072 and 1,296 tetrahedra: 181
+  // -> 177 and 161 -> 143 us).  Six-digit blocks of fewer than four elements
+  // are held to the same number by other limits.
+  static constexpr bool OVER = EB >= (BITS == 10 ? 4 : 2) && NT % (THREADS / 32) == 0 && RES_EL <= DIG_EL;
   static constexpr size_t HI_BYTES = (size_t)EB * COLS * NPH * 4;  // the columns' high words, before the digits
   static constexpr size_t DIG_BYTES = EB * DIG_EL > HI_BYTES ? EB * DIG_EL : (HI_BYTES + 15) / 16 * 16;
   static constexpr size_t RES_BYTES = OVER ? RES_EL : EB * RES_EL;
@@ -201,54 +176,6 @@ struct Shape {
   }
   static constexpr size_t EX_BYTES = (size_t)(EB * COLS + 3) / 4 * 16;
 };
-
-// Sum of the weight levels of one output, in units of 2^UNIT digit-product
-// units: t[k], b[k] the accumulators of level k (even digit of the pair) and
-// k + 1 (odd digit).  Integer sums of at most 2^24 convert exactly.
-template <int BITS, int UNIT, int NP, int T>
-__device__ __forceinline__ long long level_sum(const float (&t)[T], const float (&b)[T]) {
-  // floats whose two parts may together exceed 2^24 are converted one by one
-  const int i0 = __float2int_rn(t[0]);
-  const int i1 = __float2int_rn(t[1] + b[0]);
-  if constexpr (BITS == 10) {
-    const int i2 = NP <= 21 ? __float2int_rn(t[2] + b[1]) : __float2int_rn(t[2]) + __float2int_rn(b[1]);
-    const int i3 = __float2int_rn(t[3]) + __float2int_rn(b[2]);
-    const float low = (t[4] + b[3]) + ((t[5] + b[4]) + b[5] * 0x1p-10f) * 0x1p-10f;
-    const int il = __float2int_rn(low * (UNIT == 62 ? 0.25f : 0.5f));
-    const long long hi = (long long)i0 * (1 << 20) + ((long long)i1 * (1 << 10) + i2);
-    return (hi << (80 - UNIT)) + ((long long)i3 * (1 << (70 - UNIT)) + il);
-  } else {
-    const int i2 = __float2int_rn(t[2] + b[1]);
-    const int i3 = __float2int_rn(t[3]) + __float2int_rn(b[2]);
-    const int i4 = __float2int_rn(t[4]) + __float2int_rn(b[3]);
-    const float low = (t[5] + b[4]) + ((t[6] + b[5]) + b[6] * 0x1p-9f) * 0x1p-9f;
-    const int il = __float2int_rn(low * 0x1p-6f);
-    const long long hi = (long long)i0 * (1 << 18) + ((long long)i1 * (1 << 9) + i2);
-    return (hi << 21) + ((long long)i3 * (1 << 12) + ((long long)i4 * 8 + il));
-  }
-}
-
-// v 2^(E - shift) rounded to nearest, E the sum of the two exponents of
-// exp_of_max; NaN for a non-finite marker, zero below the normal range
-template <int BITS, int UNIT>
-__device__ __forceinline__ double level_value(long long v, int E) {
-  // x = a 2^(Ex - 1022 - TOT) with TOT = 6 BITS - 1 bits: v has the unit
-  // 2^(UNIT - 2 TOT + E - 2044)
-  constexpr int SH = UNIT - 2 * (6 * BITS - 1) - 2044;
-  const unsigned sgn = (unsigned)((unsigned long long)v >> 63) << 31;
-  const unsigned long long u = (unsigned long long)(v < 0 ? -v : v);
-  const int lz = __clzll((long long)u);
-  const unsigned long long n = u << (lz & 63);
-  const unsigned long long r = (n >> 11) + ((n >> 10) & 1ULL);  // 53 bits, rounded (a carry goes to the exponent)
-  const int ef = 63 - lz + 1023 + SH + E;                       // biased exponent
-  unsigned long long bits = r + ((unsigned long long)(unsigned)(ef - 1) << 52);
-  if ((unsigned)(ef - 1) >= 2045u) {  // overflow, underflow or a non-finite marker
-    bits = ef > 0 ? 0x7FF0000000000000ULL : 0ULL;
-    if (E >= NONFINITE) bits = 0x7FF8000000000000ULL;
-  }
-  if (u == 0 && E < NONFINITE) bits = 0ULL;
-  return __longlong_as_double((long long)(bits | ((unsigned long long)sgn << 32)));
-}
 
 // v (COLS values of node m of element el) -> shared digit rows, with zero
 // digits for the padding nodes (NP .. KP - 1).  Three steps with block barriers
@@ -274,23 +201,25 @@ __device__ __forceinline__ void digitize(const double (&v)[S::COLS], bool on, in
   if constexpr (S::KP > NP) {
     constexpr int W = S::KP - NP;
     unsigned short* d = reinterpret_cast<unsigned short*>(dig);
-    for (int j = threadIdx.x; j < EB * 6 * COLS * W; j += THREADS) {
+    for (int j = threadIdx.x; j < EB * S::DIGITS * COLS * W; j += THREADS) {
       const int row = j / W, k = j - row * W;
       d[row * (2 * S::NPW) + NP + k] = 0;
     }
   }
   if (on) {
-    unsigned short* row = reinterpret_cast<unsigned short*>(dig) + (size_t)el * 6 * COLS * (2 * S::NPW) + m;
+    unsigned short* row = reinterpret_cast<unsigned short*>(dig) + (size_t)el * S::DIGITS * COLS * (2 * S::NPW) + m;
     constexpr unsigned MASK = (1u << S::BITS) - 1u;
 #pragma unroll
     for (int c = 0; c < COLS; ++c) {
       const unsigned long long b = fixed_fields<S::BITS>(v[c], ex[el * COLS + c]);
 #pragma unroll
-      for (int s = 0; s < 6; s += 2) {
-        const unsigned ua = (unsigned)(b >> ((5 - s) * S::BITS)) & MASK, ub = (unsigned)(b >> ((4 - s) * S::BITS)) & MASK;
+      for (int s = 0; s < S::DIGITS; s += 2) {
+        constexpr int LAST = S::DIGITS - 1;
+        const unsigned ua = (unsigned)(b >> ((LAST - s) * S::BITS)) & MASK;
+        const unsigned ub = s < LAST ? (unsigned)(b >> ((LAST - 1 - s) * S::BITS)) & MASK : 0u;
         const unsigned h = unbias<S::BITS>(ua | (ub << 16));
         row[(s * COLS + c) * (2 * S::NPW)] = (unsigned short)h;
-        row[((s + 1) * COLS + c) * (2 * S::NPW)] = (unsigned short)(h >> 16);
+        if (s < LAST) row[((s + 1) * COLS + c) * (2 * S::NPW)] = (unsigned short)(h >> 16);
       }
     }
   }
@@ -309,7 +238,7 @@ __device__ __forceinline__ void prefetch_l2(const void* p, unsigned n) {
 template <class S, int D, int NP, int EB, int NF, int NW, int THREADS>
 __device__ __forceinline__ void contract(__half* dig, const int* ex, const int* elems,
                                          const uint4* __restrict__ opsP, const short* __restrict__ opsE, double* res) {
-  constexpr int BITS = S::BITS, MB = S::MB, T = S::T, COLS = S::COLS;
+  constexpr int BITS = S::BITS, DIGITS = S::DIGITS, MB = S::MB, T = S::T, COLS = S::COLS;
   constexpr int PAIRS = pairs_for(NP);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t4 = lane & 3;
@@ -344,13 +273,15 @@ __device__ __forceinline__ void contract(__half* dig, const int* ex, const int* 
     for (int i = 0; i < D; ++i) {
       const short* de = opsE + ((size_t)e * D + i) * NP;
       // ldmatrix row addresses: matrices 0, 2 hold digit 2a, 1, 3 digit 2a + 1
+      // (where there is no digit 2a + 1, digit 2a again: `odd` taken off)
+      const unsigned odd = (unsigned)((lane >> 3) & 1) * (COLS * S::NPW * 4);
       unsigned addr[MB];
 #pragma unroll
       for (int mb = 0; mb < MB; ++mb) {
         int c = mb * 8 + (lane & 7);
         if (c >= NF + NW) c = NF + NW - 1;
         const int col = c < NF ? i * NF + c : D * NF + (c - NF);
-        addr[mb] = dig0 + (((el * 6 + ((lane >> 3) & 1)) * COLS + col) * S::NPW) * 4 + (lane >> 4) * 16;
+        addr[mb] = dig0 + (((el * DIGITS) * COLS + col) * S::NPW) * 4 + odd + (lane >> 4) * 16;
       }
       float acc[MB][T][4];
 #pragma unroll
@@ -368,32 +299,33 @@ __device__ __forceinline__ void contract(__half* dig, const int* ex, const int* 
       }
 #pragma unroll
       for (int kt = 0; kt < S::K16; ++kt) {
-        unsigned b0[6], b1[6];
+        unsigned b0[DIGITS], b1[DIGITS];
         unpack<BITS>(q[2 * kt], b0);
         unpack<BITS>(q[2 * kt + 1], b1);
 #pragma unroll
         for (int mb = 0; mb < MB; ++mb)
 #pragma unroll
-          for (int a = 0; a < 3; ++a) {
+          for (int a = 0; a < (DIGITS + 1) / 2; ++a) {
             unsigned A[4];
-            ldm4(A, addr[mb] + (2 * a * COLS * S::NPW) * 4 + kt * 32);
+            ldm4(A, addr[mb] - (2 * a + 1 < DIGITS ? 0u : odd) + (2 * a * COLS * S::NPW) * 4 + kt * 32);
 #pragma unroll
-            for (int j = 0; j < 6; ++j)
+            for (int j = 0; j < DIGITS; ++j)
               if (j + 2 * a < T) mma16(acc[mb][j + 2 * a], A, b0[j], b1[j]);
           }
       }
       if constexpr (S::K8) {
         constexpr int kt = S::K16;
-        unsigned b0[6];
+        unsigned b0[DIGITS];
         unpack<BITS>(q[NQ - 1], b0);
 #pragma unroll
         for (int mb = 0; mb < MB; ++mb)
 #pragma unroll
-          for (int a = 0; a < 3; ++a) {
+          for (int a = 0; a < (DIGITS + 1) / 2; ++a) {
             unsigned A0, A1;
-            ldm2(A0, A1, addr[mb] - (lane >> 4) * 16 + (2 * a * COLS * S::NPW) * 4 + kt * 32);
+            ldm2(A0, A1, addr[mb] - (2 * a + 1 < DIGITS ? 0u : odd) - (lane >> 4) * 16 +
+                             (2 * a * COLS * S::NPW) * 4 + kt * 32);
 #pragma unroll
-            for (int j = 0; j < 6; ++j)
+            for (int j = 0; j < DIGITS; ++j)
               if (j + 2 * a < T) mma8(acc[mb][j + 2 * a], A0, A1, b0[j]);
           }
       }
@@ -410,18 +342,20 @@ __device__ __forceinline__ void contract(__half* dig, const int* ex, const int* 
             tt[k] = acc[mb][k][r];
             bb[k] = acc[mb][k][2 + r];
           }
-          long long J = level_sum<BITS, S::UNIT, NP, T>(tt, bb);
+          int fine;
+          long long J = level_sum<BITS, S::UNIT, NP, T>(tt, bb, fine);
           const int col = c < NF ? i * NF + c : D * NF + (c - NF);
           const bool live = c < NF + NW && mo + r < NP;
-          int E = live ? ex[el * COLS + col] + (int)__ldg(&de[mo + r]) : 0;
-          if (NF > 0 && c < NF) {  // align with the sum over the directions so far
+          int E = live ? ex[el * COLS + col] + (int)__ldg(&de[mo + r]) - fine : 0;
+          if (NF > 0 && c < NF) {  // the sum over the directions so far
             if (i > 0) {
-              const int Em = max(E, fE[mb][r]);
-              J = (J >> min(Em - E, 63)) + (fs[mb][r] >> min(Em - fE[mb][r], 63));
-              E = Em;
+              add_direction(fs[mb][r], fE[mb][r], J, E);
+              J = fs[mb][r];
+              E = fE[mb][r];
+            } else {
+              fs[mb][r] = J;
+              fE[mb][r] = E;
             }
-            fs[mb][r] = J;
-            fE[mb][r] = E;
           }
           if (live && (c >= NF || i == D - 1)) {
             const int k = c < NF ? c : NF + i * NW + (c - NF);
