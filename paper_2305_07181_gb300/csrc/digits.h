@@ -153,7 +153,9 @@ IM_FN double level_value(long long v, int E) {
   const unsigned long long r = (n >> 11) + ((n >> 10) & 1ULL);  // 53 bits, rounded (a carry goes to the exponent)
   const int ef = 63 - lz + 1023 + SH + E;                       // biased exponent
   unsigned long long bits = r + ((unsigned long long)(unsigned)(ef - 1) << 52);
-  if ((unsigned)(ef - 1) >= 2045u) {  // overflow, underflow or a non-finite marker
+  // overflow, underflow or a non-finite marker (from the largest exponent,
+  // 2046, a carry of the rounding gives the bits of infinity by itself)
+  if ((unsigned)(ef - 1) >= 2046u) {
     bits = ef > 0 ? 0x7FF0000000000000ULL : 0ULL;
     if (bad) bits = 0x7FF8000000000000ULL;
   }

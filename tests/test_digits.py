@@ -207,3 +207,28 @@ def test_non_finite_entries_give_nan(exe, n_p, d):
             good = [(_data("ordinary", rng, n_p), _data("ordinary", rng, n_p)) for _ in range(d - 1)]
             cases += [(n_p, d, [(v, o)] + good), (n_p, d, good + [(o, v)])]
     assert all(r != r for r in _sums(exe, cases))
+
+
+@pytest.mark.parametrize("n_p,d", SIZES)
+def test_sums_at_the_end_of_the_float64_range(exe, n_p, d):
+    """Finite sums up to the largest float64 come out finite, and infinite ones
+    from there on; below the normal range they are zero."""
+    top, zero = 1.7976931348623157e308, ([0.0] * n_p, [0.0] * n_p)
+    cases = []
+    for f in (0.49, 0.51, 0.75, 0.999, 1.0, 1.01):     # of 2^1024: biased exponents 2045, 2046, beyond
+        for s in (1.0, -1.0):
+            x = [0.0] * n_p
+            x[0], x[n_p - 1] = s * f * (top / 2), s * f * (top / 2)
+            cases.append((n_p, d, [([1.0] * n_p, x)] + [zero] * (d - 1)))
+    for v in (2.0 ** -1022, 2.0 ** -1023, 2.0 ** -1060):
+        cases.append((n_p, d, [([v * 2.0 ** 500] * n_p, [2.0 ** -500] + [0.0] * (n_p - 1))] + [zero] * (d - 1)))
+    got = _sums(exe, cases)
+    for (_, _, dirs), r in zip(cases, got):
+        a, x = dirs[0]
+        want = sum(Fraction(p) * Fraction(v) for p, v in zip(a, x))
+        if abs(want) > Fraction(top):
+            assert r == (float("inf") if want > 0 else -float("inf"))
+        elif abs(want) < Fraction(1, 2 ** 1022):
+            assert r == 0.0
+        else:
+            assert abs(Fraction(r) - want) <= abs(want) / 2 ** 50
