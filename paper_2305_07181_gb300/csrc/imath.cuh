@@ -5,16 +5,18 @@
 // float64 log and exp (fmath.cuh) take 17 and 14 float64 instructions; these
 // take none, ~60 integer and float32 instructions each, which hide behind the
 // float64 work around them.  Numbers are fixed point, 64-bit integers of
-// 2^-57: absolute error of the logarithm below 2^-55.5 whatever its size, so a
-// power formed from it (q = rho^a p^b) is good to a few 2^-55 relative, while
-// a float64 logarithm of size 2 alone carries 2^-53 into the exponential.
+// 2^-57: absolute error of the logarithm below 2^-57.3 whatever its size (half
+// a unit, and 10 units of 2^-62 from the terms below), so a power formed from
+// it (q = rho^a p^b) is good to a few 2^-56 relative, while a float64 logarithm
+// of size 2 alone carries 2^-53 into the exponential.
 //
 //   log:  x = 2^k m, m in [1, 2); j the top 8 bits of m's fraction;
 //         z = m r_j / 2^14 - 1 exactly (14-bit r_j ~ 2^14/m: the 67-bit
 //         product modulo 2^64), |z| < 2^-8.9;
 //         ln x = k ln 2 + T_j + z - z^2 (1/2 - z/3) - z^4 (1/4 - z/5 + z^2/6),
 //         T_j = -ln(r_j / 2^14) tabulated; the last term, below 2^-37, in
-//         float32.  log_fixed62 the same in units of 2^-62 near 1.
+//         float32 (error below 6 units of 2^-62).  The terms are added in units
+//         of 2^-62 and rounded once; log_fixed62, near 1, keeps those units.
 //   exp:  X = N ln2/512 + r, |r| < 2^-10.5, N = 512 K + j;
 //         exp X = 2^K 2^(j/512) (1 + r + r^2/2 + r^3/6 (1 + r/4 + r^2/20)),
 //         the cubic term, below 2^-34, in float32.
@@ -82,9 +84,9 @@ IM_FN bool log_fixed(double x, long long& L) {
   const long long w = (1LL << 61) - __mul64hi(a, 0x2AAAAAAAAAAAABLL);           // 1/2 - z/3, unit 2^-62 (2^55 / 3)
   const long long s = __mul64hi(h, w);                                          // z^2 (1/2 - z/3), unit 2^-76
   const float zf = __int2float_rn((int)(a >> 32)) * 0x1p-39f, z2 = zf * zf;
-  const int t = __float2int_rn(z2 * z2 * (0.25f + zf * (zf * 0.16666667f - 0.2f)) * 0x1p+57f);
-  const long long kl = (long long)k * LN2_HI + (((long long)k * LN2_LO) >> 32);
-  L = kl + ((IM_LOAD(&LOG_T[j]) + 16) >> 5) + ((z + 256) >> 9) - ((s + (1LL << 18)) >> 19) - t;
+  const int t = __float2int_rn(z2 * z2 * (0.25f + zf * (zf * 0.16666667f - 0.2f)) * 0x1p+62f);
+  const long long low = (((long long)k * LN2_LO) >> 27) + IM_LOAD(&LOG_T[j]) + (z >> 4) - (s >> 14) - t;  // unit 2^-62
+  L = (long long)k * LN2_HI + ((low + 16) >> 5);
   return true;
 }
 
