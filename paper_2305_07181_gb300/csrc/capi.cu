@@ -354,7 +354,7 @@ int esplit_upload_mesh(esplit_ctx* c, int n_e, const double* J, const double* La
     dalloc(c, &c->b.opsD32, 0);
     c->opsD_stride = 0;
   }
-  const size_t tensor_rows = d >= 2 ? (size_t)n_e * d * NP : 0;
+  const size_t tensor_rows = esplit::tensor_path(d, NP) ? (size_t)n_e * d * NP : 0;
   if ((rc = dalloc(c, &c->b.opsP, tensor_rows * ((NP + 1) / 2)))) return rc;
   if ((rc = dalloc(c, &c->b.opsE, tensor_rows))) return rc;
   c->partial_cap = 0;

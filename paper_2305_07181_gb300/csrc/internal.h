@@ -21,6 +21,9 @@ inline int spread_block(size_t n, int most) {
   while (b > 32 && (n + b - 1) / b < (size_t)SMS) b /= 2;
   return b;
 }
+// whether the split kernels of this operator contract on the tensor cores
+// (tc64.cuh), from packed operators; else in float64 loops
+constexpr bool tensor_path(int d, int np) { return d >= 2 && np > 8; }
 constexpr int SMALL_BLOCKS = 4 * SMS;  // short blocks up to four per SM, see split_cached_launch
 
 // row length of the float32 path's staged operators: the smallest multiple of
@@ -69,7 +72,7 @@ struct Buffers {
   // per-element derivative operators D_i = H^-1 Q_x_i, transposed ([i][n][m])
   double* ops64 = nullptr;     // [n_e][d][n_p][n_p]
   // D_i as 60-bit fixed point, two entries per uint4, and the rows' exponents
-  // (tc64.cuh; triangles and tetrahedra)
+  // (tc64.cuh; null where tensor_path is false)
   uint4* opsP = nullptr;       // [n_e][d][n_p][ceil(n_p / 2)]
   short* opsE = nullptr;       // [n_e][d][n_p]
   float* ops32 = nullptr;      // [n_e][d][n_p][n_p] ops64 rounded to float32

@@ -541,7 +541,7 @@ int launch_face_bc(esplit_ctx* c, const double* u, double* out, int add, double*
 // ---------------------------------------------------------------------------
 template <int D, int NP, int EB, bool VISC, int TH = round32(EB * NP)>
 struct SplitCfg {
-  static constexpr bool TENSOR = D >= 2 && NP > 8;
+  static constexpr bool TENSOR = tensor_path(D, NP);
   static constexpr int NC = D + 2;
   static constexpr int THREADS = TH;
   using S = tc::Shape<D, NP, EB, NC, NC, TH>;  // f_i summed over i, w per direction

@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(64) face_vjp_kernel(const double* __restrict__
 // pointwise part is left.
 template <int D, int NP, int EB, int TH = round32(EB * NP)>
 struct VjpCfg {
-  static constexpr bool TENSOR = NP > 8;
+  static constexpr bool TENSOR = tensor_path(D, NP);
   static constexpr int NC = D + 2;
   static constexpr int THREADS = TH;
   using S1 = tc::Shape<D, NP, EB, 0, 2 * NC, TH>;
