@@ -75,12 +75,13 @@ def render() -> str:
         el.append(l)
     lines += arr("EXP_T_HI", eh) + arr("EXP_T_LO", el)
     # Taylor coefficients
-    lines.append("// log1p(r) = r + r^2 (C2 + r (C3 + ... + r C9)),  Ck = (-1)^(k+1)/k")
-    for k in range(2, 10):
+    lines.append("// log1p(r) = r + r^2 (C2 + r (C3 + ... + r C9)),  Ck = (-1)^(k+1)/k (through C12 for")
+    lines.append("// the direct series of log1p at |x| < 2^-5)")
+    for k in range(2, 13):
         lines.append(f"constexpr double LOG_C{k} = {float(Decimal((-1) ** (k + 1)) / k)!r};")
-    lines.append("// expm1(r) = r + r^2 (E2 + r (E3 + ... + r E6)),  Ek = 1/k!")
+    lines.append("// expm1(r) = r + r^2 (E2 + r (E3 + ... + r E7)),  Ek = 1/k!")
     f = Decimal(1)
-    for k in range(1, 7):
+    for k in range(1, 14):
         f *= k
         if k >= 2:
             lines.append(f"constexpr double EXP_E{k} = {float(1 / f)!r};")
