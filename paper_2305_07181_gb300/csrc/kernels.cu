@@ -1027,14 +1027,17 @@ __global__ void __launch_bounds__(EB * NP) hadamard_volume_kernel(
 
 namespace esplit {
 
-template <int NP>
+template <int D, int NP>
 struct VolCfg {
   // split volume kernel: blocks of about 128 threads that fill their warps
   // (126 of 128 threads at n_p = 7 and 18, 120 at 12, 189 of 192 at 27, 125 at
   // 25, 116 of 128 at 58, 156 of 160 at 78), so that several blocks share an
-  // SM and one block's tensor phase runs beside another's float64 phase
-  static constexpr int EB_SPLIT = NP == 7 ? 18 : NP == 12 ? 10 : NP == 18 ? 7 : NP == 27 ? 7 : NP == 25 ? 5
-                                  : NP > 32 ? 2 : 128 / NP;
+  // SM and one block's tensor phase runs beside another's float64 phase.
+  // 12-node tetrahedra: 60 of 64 threads.  Ten elements need 77.6 KB in 3D, two
+  // blocks (8 warps) per SM; measured per launch with ten and with five, 24,576
+  // tetrahedra 260 and 184 us (viscous 461 and 315), 4,374 65 and 43 (106 and 67)
+  static constexpr int EB_SPLIT = NP == 7 ? 18 : NP == 12 ? (D == 3 ? 5 : 10) : NP == 18 ? 7 : NP == 27 ? 7
+                                  : NP == 25 ? 5 : NP > 32 ? 2 : 128 / NP;
   // larger operators (tetrahedra of degree 3 and 4): the pair contributions
   // pass through shared memory in chunks of HAD_KC pair offsets, which leaves
   // room for more elements per block
@@ -1134,7 +1137,7 @@ static int residual_np(esplit_ctx* c, const double* u, double* r, cudaStream_t s
   const int* lsplit = scheme == ESPLIT_SCHEME_HYBRID ? c->b.list_split : nullptr;
   const int* lhad = scheme == ESPLIT_SCHEME_HYBRID ? c->b.list_had : nullptr;
   if (n_split > 0) {
-    constexpr int EB = VolCfg<NP>::EB_SPLIT;
+    constexpr int EB = VolCfg<D, NP>::EB_SPLIT;
     int nb;
     ProfScope ps(c, PG_SPLIT, s);
     double* pp = prod ? prod + np_used : nullptr;
@@ -1158,8 +1161,8 @@ static int residual_np(esplit_ctx* c, const double* u, double* r, cudaStream_t s
     np_used += nb;
   }
   if (n_had > 0) {
-    constexpr int EB = VolCfg<NP>::EB_HAD;
-    constexpr int KC = VolCfg<NP>::HAD_KC;
+    constexpr int EB = VolCfg<D, NP>::EB_HAD;
+    constexpr int KC = VolCfg<D, NP>::HAD_KC;
     size_t smem = sizeof(T) * ((size_t)EB * (D + 7) * NP + (size_t)EB * NP * KC * (D + 2) + (size_t)EB * NP);
     auto* kern = scheme == ESPLIT_SCHEME_HADAMARD_IR ? hadamard_volume_kernel<T, D, NP, EB, 1, KC>
                                                      : hadamard_volume_kernel<T, D, NP, EB, 0, KC>;
