@@ -527,16 +527,17 @@ int launch_face_bc(esplit_ctx* c, const double* u, double* out, int add, double*
 //
 // Pointwise work in float64, one node per thread.  Triangles and tetrahedra:
 // the contractions on the tensor cores (tc64.cuh: exact digit products, one
-// rounding; as accurate as a float64 sum or better), so the float64 pipe has
-// only the nodal state, fluxes and A~_i products left (the FP32-bulk setting
-// takes this kernel too: compensated float32 contractions measured slower,
-// 97 against 78 us on 18,432 triangles p 2).  Lines and 7-node
+// rounding; the header compares the error with a float64 sum's), so the float64
+// pipe has only the nodal state, fluxes and A~_i products left (the FP32-bulk
+// setting takes this kernel too: compensated float32 contractions measured
+// slower, 97 against 78 us on 18,432 triangles p 2).  Lines and 7-node
 // triangles: float64 FMA loops, too short for the tiles.
 // Measured per launch, float64 loops before and now: 32,768 triangles p 3 490
-// and 163 us, 7,442 triangles p 4 210 and 83, 3,072 tetrahedra p 3 740 and 177,
-// 24,576 tetrahedra p 2 with viscous terms 1,650 and 680.  Bound now by the
-// latency of its phases: float64 pipe and issue slots 60 % busy, tensor pipe
-// 20 % (18 nodes, 24 warps per SM).
+// and 160 us, 7,442 triangles p 4 210 and 81, 3,072 tetrahedra p 3 740 and 178,
+// 24,576 tetrahedra p 2 with viscous terms 1,650 and 600.  Bound now by the
+// latency of its phases: float64 pipe and issue slots 61 % busy, tensor pipe
+// 21 % (18 nodes, 24 warps per SM); 25, 42 and 39 % at 58 nodes, 46, 52 and
+// 25 % with viscous terms (16 warps per SM).
 // Optional: block partial of sum H w^T r (entropy production, float64).
 // ---------------------------------------------------------------------------
 template <int D, int NP, int EB, bool VISC, int TH = round32(EB * NP)>

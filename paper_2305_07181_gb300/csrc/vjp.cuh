@@ -12,11 +12,12 @@
 //              + facet part (dG/du)^T (-cot_km/H_km + cot_vn/H_vn).
 // The pointwise derivatives are exact: the facet terms by a hand-written
 // reverse sweep at the values, the volume's pointwise part with closed-form
-// products and one dual direction (dual.cuh; see split_vjp_kernel); the
-// contractions are transposed applications of the stored per-element
-// operators.  Float64 throughout.
-// Included by kernels.cu (one device translation unit: the constant-memory
-// operator tables are shared).
+// products and one dual direction (dual.cuh; see split_vjp_kernel).  The
+// contractions apply the forward operators: D_i^T y = E_i (y/H) - H D_i (y/H)
+// (Def. 1), on the tensor cores as the residual's (tc64.cuh).  Float64
+// throughout.
+// Included by vjp.cu, the reverse mode's own translation unit with its own
+// copy of the constant-memory operator tables.
 #pragma once
 
 namespace esplit {
